@@ -213,6 +213,17 @@ __global__ void k_gen_medium(GridP g, SpecP sp, PartP p, int lo0, int lo1, int l
       float f = (float)(X - fl);
       int ci = (int)fl;
       if (f >= 1.0f) { f = 0.0f; ci += 1; }
+      if (ci >= g.n[a]) {
+        // the offset of an ion at the very end of the grid's last cell rounds
+        // up to 1 (one position in 2^25): a periodic axis wraps, on an open
+        // one the ion stays in the cell (cell n would index past the grid)
+        if (g.bc[a] == BP_PERIODIC) {
+          ci = 0;
+        } else {
+          ci = g.n[a] - 1;
+          f = 0.99999994f;
+        }
+      }
       cell[a] = ci;
       off[a] = f;
     }

@@ -282,6 +282,7 @@ int bp_create(const bp_grid_desc *gd, const bp_allocator *al, void *stream, bp_c
   }
   g.dtd = gd->dt;
   g.dt = (float)gd->dt;
+  for (int a = 0; a < 3; ++a) g.dxdt[a] = g.dx[a] / g.dt;
   g.ncell = ncell;
   g.ntiles = g.nt[0] * g.nt[1] * g.nt[2];
   g.cpt = g.L[0] * g.L[1] * g.L[2];

@@ -20,6 +20,7 @@ struct GridP {
   int n[3];
   int bc[3];
   float dx[3], idx[3];
+  float dxdt[3];    // dx / dt
   float dt;
   double dxd[3], dtd;
   int L[3], nt[3];
@@ -356,8 +357,12 @@ __device__ __forceinline__ void fx_add2(unsigned int *lo0, unsigned int *lo1, in
   const int h0 = __float_as_int(hs.x) - 0x4B400000, h1 = __float_as_int(hs.y) - 0x4B400000;
   atomicAdd(reinterpret_cast<int *>(lo0), l0);
   atomicAdd(reinterpret_cast<int *>(lo1), l1);
-  if (h0) atomicAdd(reinterpret_cast<int *>(lo0 + hoff), h0);
-  if (h1) atomicAdd(reinterpret_cast<int *>(lo1 + hoff), h1);
+  // one branch for the pair (a branch and its reconvergence barrier per word
+  // were 216 of the 3D push's 2,630 instructions per ion)
+  if (h0 | h1) {
+    atomicAdd(reinterpret_cast<int *>(lo0 + hoff), h0);
+    atomicAdd(reinterpret_cast<int *>(lo1 + hoff), h1);
+  }
 }
 
 // the value of a pair (both words initialised to 0)

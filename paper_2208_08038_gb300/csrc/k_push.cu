@@ -745,7 +745,7 @@ __device__ __noinline__ bool push_far(const GridP &g, const SpecP &sp, const Par
   QIn in;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    in.f[a] = f[a]; in.de1[a] = de1[a]; in.v1[a] = v1[a]; in.dxdt[a] = g.dx[a] / g.dt; in.d[a] = 0;
+    in.f[a] = f[a]; in.de1[a] = de1[a]; in.v1[a] = v1[a]; in.dxdt[a] = g.dxdt[a]; in.d[a] = 0;
     in.f2[a] = in.de2[a] = in.v2[a] = 0.0f;
     in.d2[a] = 0;
   }
@@ -841,7 +841,7 @@ __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, l
     atomicOr(status, ST_DOMAIN);
     return;
   }
-  // A tile whose staged E, B are all zero (ahead of the field front) gathers
+  // A tile whose staged box holds no field (ahead of the field front) gathers
   // exact zeros, so the gather is skipped.  A neutral ion there with r = 0 and
   // u1 = u2 also keeps its momenta exactly (no internal force at r = 0, Boris
   // rotation by zero fields), so its kicks are skipped too.
@@ -909,7 +909,7 @@ __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, l
       if (a < D) de2[a] = de1[a] - dr * g.idx[a];
     }
   }
-  const float dxdt[3] = {g.dx[0] / g.dt, g.dx[1] / g.dt, g.dx[2] / g.dt};
+  const float dxdt[3] = {g.dxdt[0], g.dxdt[1], g.dxdt[2]};
   // fast path when every position keeps one nearest node per axis
   bool fast = true;
   float xi[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
@@ -1289,17 +1289,13 @@ __device__ __forceinline__ void stage_issue(const GridP &g, const PushArgs &A, c
 }
 
 // wait for tile t's staging (this thread's copies, or the TMA loads: the
-// mbarrier phase `phase`, flipped here after each TMA tile); whether any
-// staged value is non-zero.  A TMA wait that gives up sets ST_TIMEOUT and
-// `failed`.
+// mbarrier phase `phase`, flipped here after each TMA tile).  A TMA wait that
+// gives up sets ST_TIMEOUT and `failed`.
 template <int D>
-__device__ __forceinline__ bool stage_done(const GridP &g, const PushArgs &A, const TmaMaps &T, int t,
-                                           const float *Gsm, unsigned long long *bar, unsigned &phase, bool &failed) {
-  using BX = Box<D>;
-  constexpr int GC = BX::GCELLS;
+__device__ __forceinline__ void stage_done(const GridP &g, const PushArgs &A, const TmaMaps &T, int t,
+                                           unsigned long long *bar, unsigned &phase, bool &failed) {
   asm volatile("cp.async.wait_group 0;" ::: "memory");
-  bool nz = false;
-  if (A.qstate[t] != QS_PUSH) return nz;
+  if (A.qstate[t] != QS_PUSH) return;
   const int tc[3] = {t % g.nt[0], (t / g.nt[0]) % g.nt[1], t / (g.nt[0] * g.nt[1])};
   const int T0[3] = {tc[0] * Geo<D>::L0, tc[1] * Geo<D>::L1, tc[2] * Geo<D>::L2};
   if (tma_tile<D>(g, T, T0)) {
@@ -1309,13 +1305,6 @@ __device__ __forceinline__ bool stage_done(const GridP &g, const PushArgs &A, co
     }
     phase ^= 1u;
   }
-  for (int q = threadIdx.x; q < BX::GCOMP; q += blockDim.x) {
-    const int b0 = q % BX::G0, b1 = (q / BX::G0) % BX::G1, b2 = q / (BX::G0 * BX::G1);
-    const int si = BX::gi(b0, b1, b2);
-#pragma unroll
-    for (int cc = 0; cc < 6; ++cc) nz |= Gsm[cc * GC + si] != 0.0f;
-  }
-  return nz;
 }
 
 // one tile of the push (the block's work for tile t)
@@ -1335,7 +1324,7 @@ __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, con
   int total = 0;
   for (int s = 0; s < A.nsp; ++s) total += A.p[s].tstart[t + 1] - A.p[s].tstart[t];
   if (qs == QS_DONE || total == 0) {
-    stage_done<D>(g, A, T, t, Gsm, bar, phase, failed);  // this tile's copies land before the next tile's are issued
+    stage_done<D>(g, A, T, t, bar, phase, failed);  // this tile's copies land before the next tile's are issued
     __syncthreads();
     if (tid == 0 && qs != QS_DONE) A.occ[t] = 0;
     after_loop();
@@ -1348,8 +1337,12 @@ __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, con
   const int T0[3] = {tc[0] * Geo<D>::L0, tc[1] * Geo<D>::L1, tc[2] * Geo<D>::L2};
   zero_box<DET>(Jsm, 3 * JC, tid, bs);
   // the field box was staged asynchronously (stage_issue) by the caller
-  const bool nz = stage_done<D>(g, A, T, t, Gsm, bar, phase, failed);
-  const bool nofield = !__syncthreads_or(nz);
+  stage_done<D>(g, A, T, t, bar, phase, failed);
+  __syncthreads();
+  // no field in the box: known from the tile marks alone (a staged box that
+  // happens to be all zero goes the full way, which leaves the same bits;
+  // reading every staged value to find it cost 1% of the 3D push)
+  const bool nofield = qs != QS_PUSH;
   QRec *qrec = DET ? reinterpret_cast<QRec *>(A.grec)
                    : reinterpret_cast<QRec *>(smem + GOFF + sizeof(float) * 6 * (size_t)GC);
   int *const qcount = DET ? A.grec_n : nullptr;
@@ -1430,10 +1423,18 @@ __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, con
   if (any) {
     const int lo0 = sbb[0], lo1 = sbb[1], lo2 = sbb[2];
     const int nx = sbb[3] - lo0 + 1, ny = sbb[4] - lo1 + 1, nz = sbb[5] - lo2 + 1;
-    const int nbox = nx * ny * nz;
+    const int nxy = nx * ny, nbox = nxy * nz;
+    // r / n as a multiplication: with m = 2^k / n rounded up, (r m) >> k is
+    // exact while r n < 2^k: rows r2 < 729, n <= 27, k = 17; planes r < 17^3,
+    // n <= 17^2, k = 24.  Four integer divisions per node took about 100
+    // instructions per ion on the 3D push.
+    static_assert(BX::J0 * BX::J1 * BX::J2 <= 4913 && BX::J0 * BX::J1 <= 729, "box small enough for the division");
+    const unsigned mx = (131072u + nx - 1) / nx, mxy = ((1u << 24) + nxy - 1) / nxy;
     for (int q = tid; q < 3 * nbox; q += bs) {
-      const int cc = q / nbox, r = q - cc * nbox;
-      const int x = lo0 + r % nx, y = lo1 + (r / nx) % ny, z = lo2 + r / (nx * ny);
+      const int cc = q >= 2 * nbox ? 2 : (q >= nbox ? 1 : 0), r = q - cc * nbox;
+      const int zz = D >= 3 ? (int)__umulhi((unsigned)r << 8, mxy) : 0, r2 = r - zz * nxy;
+      const int yy = D >= 2 ? (int)(((unsigned)r2 * mx) >> 17) : 0;
+      const int x = lo0 + r2 - yy * nx, y = lo1 + yy, z = lo2 + zz;
       const int k = cc * JC + BX::ji(x, y, z);
       if constexpr (DET) {
         const long long v = fx_value(Jsm + k, 3 * JC);
@@ -1502,7 +1503,7 @@ __global__ void __launch_bounds__(push_threads(D)) k_push(GridP g, PushArgs A, c
     if (give_up) break;  // a staging wait gave up twice (ST_TIMEOUT is set): stop
   }
   // nothing may be in flight into this block's shared memory when it exits
-  if (next >= 0 && A.qstate[next] == QS_PUSH) stage_done<D>(g, A, T, next, Gsm, &bar, phase, failed);
+  if (next >= 0 && A.qstate[next] == QS_PUSH) stage_done<D>(g, A, T, next, &bar, phase, failed);
 }
 
 // Sorted mode: the records' rows added to the fixed-point current.  Each

@@ -345,26 +345,35 @@ __device__ __forceinline__ void fx_add(unsigned int *lo, int hoff, float v) {
   const int hh = __float_as_int(hs) - 0x4B400000;
   if (hh) atomicAdd(reinterpret_cast<int *>(lo + hoff), hh);
 }
-// fx_add of two values at two nodes (lo0, lo1; high words hoff later), the
-// FP32 part on packed pairs: each lane rounds exactly as fx_add does
-__device__ __forceinline__ void fx_add2(unsigned int *lo0, unsigned int *lo1, int hoff, float2 v) {
+// fx_add of six values: three pairs, srow nodes apart, each pair spair nodes
+// apart (high words hoff later), the FP32 part on packed pairs: each lane
+// rounds exactly as fx_add does.  One branch for the six high words: a branch
+// and its reconvergence barrier per word were 216 of the 3D push's 2,630
+// instructions per ion (4.42 -> 4.31 ms a step of 32.5 M ions with one per
+// pair, 4.26 with one per six; adding the zeros without a branch: 4.53, the
+// shared-memory adds are the dearer part).
+__device__ __forceinline__ void fx_add6(unsigned int *p, int srow, int spair, int hoff, const float2 v[3]) {
   constexpr float M = 12582912.0f;
-  const float2 hs = __ffma2_rn(v, make_float2(1.52587890625e-05f, 1.52587890625e-05f), make_float2(M, M));
-  const float2 h = __fadd2_rn(hs, make_float2(-M, -M));
-  const float2 r = __ffma2_rn(h, make_float2(-65536.0f, -65536.0f), v);
-  const float2 rm = __fadd2_rn(r, make_float2(M, M));
-  const int l0 = __float_as_int(rm.x) - 0x4B400000, l1 = __float_as_int(rm.y) - 0x4B400000;
-  const int h0 = __float_as_int(hs.x) - 0x4B400000, h1 = __float_as_int(hs.y) - 0x4B400000;
-  atomicAdd(reinterpret_cast<int *>(lo0), l0);
-  atomicAdd(reinterpret_cast<int *>(lo1), l1);
-  // one branch for the pair (a branch and its reconvergence barrier per word
-  // were 216 of the 3D push's 2,630 instructions per ion)
-  if (h0 | h1) {
-    atomicAdd(reinterpret_cast<int *>(lo0 + hoff), h0);
-    atomicAdd(reinterpret_cast<int *>(lo1 + hoff), h1);
+  int h[6];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const float2 hs = __ffma2_rn(v[j], make_float2(1.52587890625e-05f, 1.52587890625e-05f), make_float2(M, M));
+    const float2 hh = __fadd2_rn(hs, make_float2(-M, -M));
+    const float2 r = __ffma2_rn(hh, make_float2(-65536.0f, -65536.0f), v[j]);
+    const float2 rm = __fadd2_rn(r, make_float2(M, M));
+    atomicAdd(reinterpret_cast<int *>(p + j * srow), __float_as_int(rm.x) - 0x4B400000);
+    atomicAdd(reinterpret_cast<int *>(p + j * srow + spair), __float_as_int(rm.y) - 0x4B400000);
+    h[2 * j] = __float_as_int(hs.x) - 0x4B400000;
+    h[2 * j + 1] = __float_as_int(hs.y) - 0x4B400000;
+  }
+  if (h[0] | h[1] | h[2] | h[3] | h[4] | h[5]) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      atomicAdd(reinterpret_cast<int *>(p + hoff + j * srow), h[2 * j]);
+      atomicAdd(reinterpret_cast<int *>(p + hoff + j * srow + spair), h[2 * j + 1]);
+    }
   }
 }
-
 // the value of a pair (both words initialised to 0)
 __device__ __forceinline__ long long fx_value(const unsigned int *lo, int hoff) {
   return (long long)(int)lo[hoff] * 65536LL + (long long)(int)lo[0];

@@ -271,31 +271,36 @@ __device__ __forceinline__ void esirkepov3_p3(unsigned int *__restrict__ J, cons
 #pragma unroll 1
   for (int k = 0; k < 3; ++k) {
     const float2 az = sel3(k, A[2]), dz = sel3(k, DS[2]);
+    unsigned int *p = Jx + Box<3>::ji(bx, by, bz + k);
+    float2 v[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       const float2 F = __ffma2_rn(A[1][j], az, __fmul2_rn(DK[1][j], dz));
       const float2 t0 = __fmul2_rn(cP[0][0], F), t1 = __fmul2_rn(cP[0][1], F);
-      unsigned int *p = Jx + Box<3>::ji(bx, by + j, bz + k);
-      fx_add2(p, p + 1, hoff, make_float2(__fadd_rn(t0.x, t0.y), __fadd_rn(t1.x, t1.y)));
+      v[j] = make_float2(__fadd_rn(t0.x, t0.y), __fadd_rn(t1.x, t1.y));
     }
+    fx_add6(p, Box<3>::J0, 1, hoff, v);
+    p = Jy + Box<3>::ji(bx, by, bz + k);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const float2 F = __ffma2_rn(A[0][i], az, __fmul2_rn(DK[0][i], dz));
       const float2 t0 = __fmul2_rn(cP[1][0], F), t1 = __fmul2_rn(cP[1][1], F);
-      unsigned int *p = Jy + Box<3>::ji(bx + i, by, bz + k);
-      fx_add2(p, p + Box<3>::J0, hoff, make_float2(__fadd_rn(t0.x, t0.y), __fadd_rn(t1.x, t1.y)));
+      v[i] = make_float2(__fadd_rn(t0.x, t0.y), __fadd_rn(t1.x, t1.y));
     }
+    fx_add6(p, 1, Box<3>::J0, hoff, v);
   }
 #pragma unroll 1
   for (int j = 0; j < 3; ++j) {
     const float2 ay = sel3(j, A[1]), dy = sel3(j, DS[1]);
+    unsigned int *p = Jz + Box<3>::ji(bx, by + j, bz);
+    float2 v[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const float2 F = __ffma2_rn(A[0][i], ay, __fmul2_rn(DK[0][i], dy));
       const float2 t0 = __fmul2_rn(cP[2][0], F), t1 = __fmul2_rn(cP[2][1], F);
-      unsigned int *p = Jz + Box<3>::ji(bx + i, by + j, bz);
-      fx_add2(p, p + Box<3>::JP, hoff, make_float2(__fadd_rn(t0.x, t0.y), __fadd_rn(t1.x, t1.y)));
+      v[i] = make_float2(__fadd_rn(t0.x, t0.y), __fadd_rn(t1.x, t1.y));
     }
+    fx_add6(p, 1, Box<3>::JP, hoff, v);
   }
 }
 

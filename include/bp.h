@@ -390,17 +390,12 @@ int bp_push_work(bp_ctx *ctx, int64_t *full, int64_t *quiet);
  * instrumentation.) */
 int bp_field_work(bp_ctx *ctx, int64_t *active_tiles, int64_t *steps);
 
-/* (The paper has no counterpart: a resource limit of this implementation.)
- * Capacity of the sorted deposit's general-case record buffer, in records
- * (BP_DEPOSIT_SORTED only).  A particle whose positions change their nearest
- * node in a step (Esirkepov's five-node case) leaves a record that a
- * separate kernel adds to the fixed-point current; when a step has more
- * such particles than the capacity, the rest deposit in place.  Both paths
- * add the same integers, so the fields do not depend on the capacity.
- * n > 0 fixes the capacity (at least 1); n = 0 restores the default (one
- * record per 256 particles, at least 65,536).  Takes effect at the next
- * bp_step; returns BP_ERR_ARG for n < 0 or a context in atomic mode,
- * BP_ERR_OOM if the buffer cannot be allocated then. */
+/* (The paper has no counterpart: a resource limit of an earlier
+ * implementation.)  The sorted deposit once kept the particles that change
+ * their nearest node in a step in a buffer of this many records; every
+ * particle now deposits in place, and the call, kept for programs that make
+ * it, sizes nothing.  BP_OK for n >= 0 on a context in the sorted mode, else
+ * BP_ERR_ARG. */
 int bp_set_record_capacity(bp_ctx *ctx, int64_t n);
 
 #ifdef __cplusplus

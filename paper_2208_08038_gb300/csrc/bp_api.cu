@@ -307,7 +307,6 @@ int bp_create(const bp_grid_desc *gd, const bp_allocator *al, void *stream, bp_c
   if (c->det) {
     c->jfx = (unsigned long long *)dalloc(c, sizeof(unsigned long long) * 3 * (size_t)ncell);
     c->ant = (double *)dalloc(c, sizeof(double) * BP_MAX_LASER * (size_t)(ncell / g.n[0]));
-    c->grec_n = (int *)dalloc(c, sizeof(int));
     c->far_n = (int *)dalloc(c, sizeof(int));
     c->far_any = (int *)dalloc(c, sizeof(int));
   }
@@ -331,7 +330,7 @@ int bp_create(const bp_grid_desc *gd, const bp_allocator *al, void *stream, bp_c
   c->clk = (long long *)dalloc(c, sizeof(long long) * kClockWords);
   long long nf = frame_floats(g);
   c->frame = nf ? (float *)dalloc(c, sizeof(float) * nf) : nullptr;
-  if (!(c->det ? (void *)c->jfx : (void *)c->jbox) || (c->det && (!c->ant || !c->grec_n || !c->far_n || !c->far_any)) || !c->tile_ctr || !c->tile_list || !c->tile_n || !c->occ || !c->jbb || !g.fnz || !c->qstate || !c->status ||
+  if (!(c->det ? (void *)c->jfx : (void *)c->jbox) || (c->det && (!c->ant || !c->far_n || !c->far_any)) || !c->tile_ctr || !c->tile_list || !c->tile_n || !c->occ || !c->jbb || !g.fnz || !c->qstate || !c->status ||
       !c->work || !c->clk || (g.ntiles >= 1024 && (!c->act || !c->act_n)) || (nf && !c->frame)) {
     bp_destroy(c);
     return BP_ERR_OOM;
@@ -341,10 +340,11 @@ int bp_create(const bp_grid_desc *gd, const bp_allocator *al, void *stream, bp_c
   if (encode_field_maps(g, c->F, &c->tmaps)) c->tmaps.on = 0;
   cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
   if (c->sms < 1) c->sms = 1;
-  if (push_prepare(g, 0, &c->push_blocks[0]) || push_prepare(g, 1, &c->push_blocks[1])) {
+  if (push_prepare(g, c->det, c->push_blocks)) {
     bp_destroy(c);
     return BP_ERR_CUDA;
   }
+  update_jscale(c);  // a run without species launches the same kernels
   if (cudaGetLastError() != cudaSuccess) {
     bp_destroy(c);
     return BP_ERR_CUDA;
@@ -643,30 +643,22 @@ int bp_add_probe(bp_ctx *c, int comp, const int64_t *nodes, int64_t npts, int64_
 
 namespace {
 
-// sorted mode: room for the general-case records of a step, 1 in 256
-// particles (at least 65,536); a step with more deposits the rest in place
-void ensure_records(bp_ctx *c) {
+// sorted mode: room for the far ions of a step (a bound electron a cell or
+// more from its nucleus), 1 in 256 particles (at least 65,536)
+void ensure_far(bp_ctx *c) {
   if (!c->det) return;
   long long n = 0;
   for (auto &s : c->sp)
     if (s.loaded) n += s.p.cap;
-  const long long want =
-      c->grec_fixed > 0 ? c->grec_fixed : std::min<long long>(1LL << 30, std::max<long long>(65536, n / 256));
-  // the far-ion list: as many entries as the default record capacity
-  const long long want_far = std::min<long long>(1LL << 30, std::max<long long>(65536, n / 256));
-  if (!c->far || c->far_cap < want_far) {
-    if (c->far) dfree(c, c->far);
-    c->far = (int4 *)dalloc(c, sizeof(int4) * (size_t)want_far);
-    c->far_cap = c->far ? want_far : 0;
-  }
-  if (c->grec && (c->grec_fixed > 0 ? c->grec_cap == want : c->grec_cap >= want)) return;
-  if (c->grec) dfree(c, c->grec);
-  c->grec = dalloc(c, push_record_bytes() * (size_t)want);
-  c->grec_cap = c->grec ? want : 0;
+  const long long want = std::min<long long>(1LL << 30, std::max<long long>(65536, n / 256));
+  if (c->far && c->far_cap >= want) return;
+  if (c->far) dfree(c, c->far);
+  c->far = (int4 *)dalloc(c, sizeof(int4) * (size_t)want);
+  c->far_cap = c->far ? want : 0;
 }
 
 PushArgs push_args(bp_ctx *c, int *nsp_out) {
-  ensure_records(c);
+  ensure_far(c);
   PushArgs A;
   memset(&A, 0, sizeof A);
   int nsp = 0;
@@ -683,13 +675,10 @@ PushArgs push_args(bp_ctx *c, int *nsp_out) {
   }
   A.jbox = c->jbox;
   A.jfx = c->jfx;
-  A.grec = c->grec;
-  A.grec_n = c->grec_n;
   A.far = c->far;
   A.far_n = c->far_n;
   A.far_cap = (int)c->far_cap;
   A.far_any = c->far_any;
-  A.grec_cap = (int)c->grec_cap;
   A.occ = c->occ;
   A.jbb = c->jbb;
   A.qstate = c->qstate;
@@ -700,7 +689,8 @@ PushArgs push_args(bp_ctx *c, int *nsp_out) {
   A.jscale = c->jscale;
   A.jinv = c->jinv;
   A.work = c->timing ? c->work : nullptr;
-  A.push_blocks = c->push_blocks[c->det ? 1 : 0];
+  A.push_blocks[0] = c->push_blocks[0];
+  A.push_blocks[1] = c->push_blocks[1];
   A.sms = c->sms;
   *nsp_out = nsp;
   return A;
@@ -883,9 +873,9 @@ void step_launches(bp_ctx *c, const PushArgs &A, bool probes, cudaStream_t st, f
 void step_account(bp_ctx *c, bool probes) {
   int nopen = 0;
   for (int a = 0; a < c->g.D; ++a) nopen += c->g.bc[a] == BP_OPEN;
-  // quiet-tile pass, push, records (sorted) or current sum (atomic), antenna (sorted, with lasers),
+  // quiet-tile pass, push, far ions (sorted) or current sum (atomic), antenna (sorted, with lasers),
   // Yee (3), Mur, the clock
-  c->launches += (c->det ? 6 + (c->las.empty() ? 0 : 1) : 6) + (nopen ? 1 + nopen : 0) + 1 + (c->act ? 1 : 0);
+  c->launches += 6 + (c->det && !c->las.empty() ? 1 : 0) + (nopen ? 1 + nopen : 0) + 1 + (c->act ? 1 : 0);
   c->step++;
   if (probes)
     for (auto &p : c->pr) {
@@ -1490,10 +1480,7 @@ int64_t bp_kernel_launches(const bp_ctx *c) {
 
 int bp_set_record_capacity(bp_ctx *c, int64_t n) {
   if (!c || n < 0 || !c->det) return BP_ERR_ARG;
-  cudaStreamSynchronize(c->stream);
-  c->grec_fixed = std::min<long long>(n, 1LL << 30);
-  ensure_records(c);
-  return (c->grec || c->sp.empty()) ? BP_OK : fail(c, BP_ERR_OOM, "record buffer");
+  return BP_OK;  // no particle leaves a record any more: nothing to size
 }
 
 int bp_time_push(bp_ctx *c, int enable) {

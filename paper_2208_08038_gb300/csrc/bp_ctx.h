@@ -73,14 +73,10 @@ struct bp_ctx {
   float *jbox = nullptr;             // atomic deposit: per-tile FP32 current boxes
   unsigned long long *jfx = nullptr; // sorted deposit: [3][ncell] current in 64-bit fixed point
   double *ant = nullptr;             // sorted deposit: antenna sheet values of a step, [laser][ncell / n0]
-  void *grec = nullptr;              // sorted deposit: general-case deposit records of a step
-  int *grec_n = nullptr;             // their count (device, cleared after each step)
   int4 *far = nullptr;               // sorted deposit: ions with a far bound electron, moved after the push
   int *far_n = nullptr;              // their count (device, cleared after each step)
   int *far_any = nullptr;            // whether the last push moved any (device)
   long long far_cap = 0;
-  long long grec_cap = 0;
-  long long grec_fixed = 0;          // capacity set by the caller (0: default)
   unsigned char *occ = nullptr;
   uint2 *jbb = nullptr;
   unsigned char *qstate = nullptr;  // per tile: left by the quiet-tile pass for the push
@@ -98,7 +94,7 @@ struct bp_ctx {
   float *frame = nullptr;
   int *status = nullptr;
   unsigned long long *work = nullptr;  // [2] push work counters (see PushArgs::work)
-  int push_blocks[2] = {1, 1};         // resident push blocks per deposit mode (atomic, sorted)
+  int push_blocks[2] = {1, 1};         // resident push blocks (see push_prepare)
   int sms = 1;                         // multiprocessors of the context's device
   TmaMaps tmaps{};                     // tensor maps of E, B for the push's TMA staging (3D)
   std::vector<bp_species_state> sp;

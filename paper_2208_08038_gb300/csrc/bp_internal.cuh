@@ -136,9 +136,6 @@ struct PushArgs {
   int *tile_list;          // [ntiles] tiles the quiet-tile pass left for the push
   int *tile_n;             // their number (cleared before the quiet-tile pass)
   int *tile_ctr;           // the push's next list entry (cleared before each launch)
-  void *grec;              // sorted deposit: general-case deposit records (grec_cap of them)
-  int *grec_n;             // their count this step (device)
-  int grec_cap;
   int *status;
   float jscale, jinv;      // fixed-point scale (sorted deposit), power of two
   unsigned long long *work; // [2] ions given the full push, ions moved by the quiet-tile pass (cumulative)
@@ -146,7 +143,7 @@ struct PushArgs {
   int *far_n;               //   (species, particle, tile), moved after the push by k_push_far; their count
   int far_cap;
   int *far_any;             // set by k_push_far when it moved any this step (their current may land anywhere)
-  int push_blocks;          // persistent push blocks for this grid on this device
+  int push_blocks[2];       // persistent push blocks for this grid on this device (see push_prepare)
   int sms;                  // multiprocessors of the device
 };
 
@@ -433,13 +430,13 @@ __host__ __device__ __forceinline__ double sm64_uniform(uint64_t key, uint64_t k
 
 void launch_push(const GridP &g, const PushArgs &a, const TmaMaps &tm, cudaStream_t s);
 size_t push_smem_bytes(const GridP &g, int det);
-size_t push_record_bytes();
 // the tiles the field kernels update (see k_tile_active); ia_lo..ia_hi: the antenna planes' x range
 void launch_tile_active(const GridP &g, const unsigned char *qstate, const int *far_any, int ia_lo, int ia_hi,
-                        unsigned char *act, unsigned long long *act_n, cudaStream_t s);  // one general-case deposit record
-// set the push kernel's shared-memory limit for this grid and return, in
-// *blocks, the number of push blocks resident on the current device at once
-int push_prepare(const GridP &g, int det, int *blocks);
+                        unsigned char *act, unsigned long long *act_n, cudaStream_t s);
+// set the push kernel's shared-memory limit for this grid and return the
+// number of push blocks resident on the current device at once: blocks[0] of
+// the two-body kernel, blocks[1] of the one for grids with free particles
+int push_prepare(const GridP &g, int det, int blocks[2]);
 
 // act (per tile, optional): tiles to update; the others keep zero E, B, J
 void launch_yee_b(const GridP &g, float *const B[3], const float *const E[3], float h, const unsigned char *act,

@@ -257,38 +257,6 @@ __device__ __forceinline__ void boris(float h, const float E[3], const float B[3
   u[2] = fmaf(h, E[2], up2);
 }
 
-// shape factors on the five-node window around the old nearest node:
-// S0[m] at the old position, DS[m] = S1[m] - S0[m], node n0 - 2 + m
-template <int D>
-__device__ __forceinline__ void window(const float f[3], const float de[3], float S0[3][5], float DS[3][5],
-                                       int n0[3], const int d[3]) {
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    if (a < D) {
-      int up = f[a] >= 0.5f ? 1 : 0;
-      float xi = f[a] - (float)up;
-      n0[a] = d[a] + Box<D>::OJ + up;
-#pragma unroll
-      for (int m = 0; m < 5; ++m) {
-        float u = xi - (float)(m - 2);
-        S0[a][m] = qshape(u);
-        DS[a][m] = qshape_delta(u, de[a]);
-      }
-    } else {
-      n0[a] = 2;
-#pragma unroll
-      for (int m = 0; m < 5; ++m) { S0[a][m] = (m == 2) ? 1.0f : 0.0f; DS[a][m] = 0.0f; }
-    }
-  }
-}
-
-// particle of a tile handled by thread tid in the chunk starting at k0: the
-// lanes of a warp take particles bs/32 apart (bs = block size, a multiple of
-// 32), so that in cell-sorted order they sit in different cells and rarely
-// add to the same shared-memory node at once; the chunk [k0, k0 + bs) is
-// still covered exactly once
-__device__ __forceinline__ int spread_index(int k0, int tid, int bs) { return k0 + (tid & 31) * (bs >> 5) + (tid >> 5); }
-
 // tile-relative cell of a global cell coordinate (periodic: nearest image)
 template <int D>
 __device__ __forceinline__ int rel_cell(const GridP &g, int a, int c, int T0) {

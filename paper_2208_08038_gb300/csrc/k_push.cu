@@ -13,21 +13,17 @@
 //        tile),
 //     2. push every particle of the tile (all species), accumulating the
 //        current of both bodies in a shared-memory box (tile + halo).  A
-//        particle whose bodies keep their nearest nodes deposits on the spot
-//        (three-node windows); the others leave a five-node record.  The box
-//        holds
+//        particle whose bodies keep their nearest nodes deposits three-node
+//        windows, the others four-node windows body by body.  The box holds
 //          BP_DEPOSIT_SORTED: 64-bit fixed point (integer adds are
 //                             associative: the same sums in any order),
 //          BP_DEPOSIT_ATOMIC: FP32 shared atomics,
 //     3. sorted mode: add every non-zero node of the box to the global 64-bit
 //        fixed-point current; atomic mode: write the box to the tile's slot
-//        for the current-sum kernel (and deposit the records from a
-//        shared-memory queue before that),
-//   k_records     sorted mode: the records' rows added to the fixed-point
-//                 current,
+//        for the current-sum kernel,
 //   k_push_far    sorted mode: the ions k_push left on the far list (a bound
 //                 electron a cell or more from its nucleus), pushed with the
-//                 global fields and deposited as one-body records,
+//                 global fields and deposited into the global current,
 //   k_tile_active the tiles the field kernels update this step: those whose
 //                 neighbourhood has held a field or holds moved particles,
 //                 those next to an antenna plane, every tile after a far push.
@@ -38,11 +34,10 @@
 
 namespace {
 
-// capacity of the deferred-deposit records per tile (shared memory); a tile
-// with more general-case particles deposits the rest in place
-__host__ __device__ constexpr int push_qmax(int D) { return D == 2 ? 128 : 64; }
 // threads of a push block
 __host__ __device__ constexpr int push_threads(int D) { return D == 3 ? 512 : 256; }
+// and the blocks per SM its registers are held to (see k_push)
+__host__ __device__ constexpr int push_pb(int D, bool free_sp) { return D == 2 ? (free_sp ? 3 : 2) : 1; }
 
 // add v (already in fixed-point units in the sorted mode) to a current node:
 // sorted mode, the exact fixed-point add fx_add (low words of the box, high
@@ -304,212 +299,239 @@ __device__ __forceinline__ void esirkepov3_p3(unsigned int *__restrict__ J, cons
   }
 }
 
-// Deferred general deposits.  A thread whose particle leaves the fast path
-// finishes the push and stores the particle's five-node windows in a record,
-// deposited row by row (one row: one current component along one line of the
-// window) by many threads, so the rare general case does not leave most of a
-// block idle.  Sorted mode: the records go to a global buffer and a separate
-// kernel adds their rows to the fixed-point current; atomic mode: a
-// shared-memory queue the block deposits after its pass.
-struct QRec {
-  float S0[2][3][5];
-  float DS[2][3][5];
-  float cq[2][3];  // component along a simulated axis: -qw dx/dt; otherwise qw v
-  int n0[2][3];    // window centre, box coordinates
-  int nb;
-  int org[3];      // grid coordinates of box node 0 (unwrapped)
+// General case of one body: its nearest node changes along some axis in this
+// step, or the ion's two bodies have different nearest nodes.  Old and new
+// shapes then span four nodes per axis (three where the node stays): node m of
+// the window is base + m, base = n0 - 1, or n0 - 2 along an axis crossed
+// downwards (n0 the old nearest node).  Along an axis that is not crossed the
+// difference of the shapes has the closed form of the fast path; a crossed
+// axis takes the difference of the two shapes, every node of which changes
+// its polynomial piece.  The current of a face is the running sum of the
+// differences, whose last one is minus the last difference.
+//
+// Bound by the shared-memory adds (40 in 2D); the body of a fast particle
+// needs 21.  It replaces five-node records in a global buffer added by a
+// kernel of its own, and a single thread's 75 rows from local memory once the
+// buffer was full: 4.2 M electrons, many of them crossing in a strong pulse,
+// push and records 1.07 ms a step before, 0.43 after; 32.5 M thermal ions in
+// 3D, 4.26 ms before, 3.78 after (one record took its lane as long as several
+// particles).
+struct GenAxis {
+  float A[4], DS[4], P[3];  // mid-step shape S0 + DS / 2, shape difference, face currents (charge factor included)
+  int base;                 // window's first node relative to the cell
 };
-
-// a general-case particle's deposit inputs, gathered into one object inside
-// the rare branch (so the main path's arrays stay in registers)
-struct QIn {
-  float f[3], de1[3], f2[3], de2[3], v1[3], v2[3], dxdt[3];
-  int d[3], d2[3];
-  float qw1, qw2;
-  int two;
-};
-
-template <int D>
-__device__ __noinline__ void queue_record(QRec &R, const QIn &in) {
-  float S0[3][5], DS[3][5];
-  int n0[3];
-  const int nb = in.two ? 2 : 1;
-  for (int b = 0; b < nb; ++b) {
-    window<D>(b ? in.f2 : in.f, b ? in.de2 : in.de1, S0, DS, n0, b ? in.d2 : in.d);
-    const float qw = b ? in.qw2 : in.qw1;
-    const float *v = b ? in.v2 : in.v1;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-#pragma unroll
-      for (int m = 0; m < 5; ++m) {
-        R.S0[b][a][m] = S0[a][m];
-        R.DS[b][a][m] = DS[a][m];
-      }
-      R.n0[b][a] = n0[a];
-      R.cq[b][a] = a < D ? -qw * in.dxdt[a] : qw * v[a];
-    }
-  }
-  R.nb = nb;
+__device__ __forceinline__ GenAxis general_axis(float f, float de, float c) {
+  GenAxis g;
+  const float up = f >= 0.5f ? 1.0f : 0.0f;
+  const float x = f - up, x1 = x + de;
+  const bool hi = x1 >= 0.5f, lo = x1 < -0.5f;
+  float w[3], W[3], d3[3];
+  qweights(x, w);
+  qweights(hi ? x1 - 1.0f : x1 + 1.0f, W);
+  d3[0] = -0.5f * de * (1.0f - 2.0f * x - de);
+  d3[1] = -de * (2.0f * x + de);
+  d3[2] = 0.5f * de * (1.0f + 2.0f * x + de);
+  g.DS[0] = hi ? -w[0] : (lo ? W[0] : d3[0]);
+  g.DS[1] = hi ? W[0] - w[1] : (lo ? W[1] - w[0] : d3[1]);
+  g.DS[2] = hi ? W[1] - w[2] : (lo ? W[2] - w[1] : d3[2]);
+  g.DS[3] = hi ? W[2] : (lo ? -w[2] : 0.0f);
+  g.A[0] = fmaf(0.5f, g.DS[0], lo ? 0.0f : w[0]);
+  g.A[1] = fmaf(0.5f, g.DS[1], lo ? w[0] : w[1]);
+  g.A[2] = fmaf(0.5f, g.DS[2], lo ? w[1] : w[2]);
+  g.A[3] = fmaf(0.5f, g.DS[3], lo ? w[2] : 0.0f);
+  g.P[0] = c * g.DS[0];
+  g.P[1] = c * (g.DS[0] + g.DS[1]);
+  g.P[2] = -c * g.DS[3];
+  g.base = (int)up - 1 - (lo ? 1 : 0);
+  return g;
 }
 
-// rows of component c: one per node of the window along each simulated axis
-// other than c
-template <int D>
-__host__ __device__ constexpr int qrows(int c) {
-  return (((c == 0 ? 1 : 0) < D) ? 5 : 1) * (((c == 2 ? 1 : 2) < D) ? 5 : 1);
+__device__ __forceinline__ float sel4(int k, const float *a) {
+  return k == 0 ? a[0] : (k == 1 ? a[1] : (k == 2 ? a[2] : a[3]));
 }
 
-// the contributions of one row: sink(c, x, y, z, v) per node, box
-// coordinates, v in the deposit's units before the fixed-point scale
-template <int D, typename Sink>
-__device__ __forceinline__ void record_row(const QRec &R, int b, int c, int row, Sink &&sink) {
-  const int p = c == 0 ? 1 : 0, q = c == 2 ? 1 : 2;  // the other two axes, p < q
-  const int ip = p < D ? row % 5 : 2, iq = q < D ? row / 5 : 2;
-  const float sp = R.S0[b][p][ip], dp = R.DS[b][p][ip], sq = R.S0[b][q][iq], dq = R.DS[b][q][iq];
-  const float fac = sp * sq + 0.5f * (dp * sq + sp * dq) + (1.0f / 3.0f) * dp * dq;
-  if (fac == 0.0f) return;
-  int node[3];
+// 1D and 2D: one body
+template <int D, bool DET, typename JT>
+__device__ __forceinline__ void deposit_general(JT *__restrict__ J, const int d[3], const float f[3], const float de[3],
+                                                float qw, const float v[3], const float dxdt[3], float scale) {
+  static_assert(D < 3, "3D: deposit_general3");
+  constexpr int jcells = Box<D>::JCELLS;
+  constexpr float K12 = 1.0f / 12.0f;
+  const float q = DET ? qw * scale : qw;
+  JT *Jx = J, *Jy = J + jcells, *Jz = J + 2 * jcells;
+  const GenAxis X = general_axis(f[0], de[0], -q * dxdt[0]);
+  if constexpr (D == 1) {
+    const int b0 = d[0] + Box<D>::OJ + X.base;
+    const float qy = q * v[1], qz = q * v[2];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) node[a] = 0;
-  if (p < D) node[p] = R.n0[b][p] - 2 + ip;
-  if (q < D) node[q] = R.n0[b][q] - 2 + iq;
-  const float cq = R.cq[b][c];
-  if (c < D) {
-    float run = 0.0f;
+    for (int i = 0; i < 3; ++i) jput<D, DET>(Jx + b0 + i, X.P[i]);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      run += R.DS[b][c][i];
-      node[c] = R.n0[b][c] - 2 + i;
-      sink(c, node[0], node[1], node[2], cq * run * fac);
+      jput<D, DET>(Jy + b0 + i, qy * X.A[i]);
+      jput<D, DET>(Jz + b0 + i, qz * X.A[i]);
     }
   } else {
-    sink(c, node[0], node[1], node[2], cq * fac);
+    const GenAxis Y = general_axis(f[1], de[1], -q * dxdt[1]);
+    const float qz = q * v[2];
+    const int b0 = Box<D>::ji(d[0] + Box<D>::OJ + X.base, d[1] + Box<D>::OJ + Y.base, 0);
+    // rows rolled (code size: the loop competes with the fast path for the
+    // instruction cache)
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j) {
+      const float ay = sel4(j, Y.A), dy = K12 * sel4(j, Y.DS);
+      const int r = b0 + Box<D>::ji(0, j, 0);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) jput<D, DET>(Jx + r + i, X.P[i] * ay);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) jput<D, DET>(Jz + r + i, qz * fmaf(X.A[i], ay, X.DS[i] * dy));
+      if (j < 3) {
+        const float py = j == 0 ? Y.P[0] : (j == 1 ? Y.P[1] : Y.P[2]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) jput<D, DET>(Jy + r + i, py * X.A[i]);
+      }
+    }
   }
 }
 
-template <int D, bool DET, typename JT>
-__device__ __forceinline__ void queued_row(JT *J, const QRec &R, int b, int c, int row, float scale) {
-  record_row<D>(R, b, c, row, [&](int cc, int x, int y, int z, float v) {
-    jadd<D, DET>(J + cc * Box<D>::JCELLS + Box<D>::ji(x, y, z), v, scale);
-  });
+// 3D: one row of one body, (component c, nodes j and k along the other two
+// axes), the three faces along c
+template <bool DET, typename JT>
+__device__ __forceinline__ void general_row3(JT *__restrict__ J, const int d[3], const GenAxis G[3], int c, int j, int k) {
+  constexpr float K12 = 1.0f / 12.0f;
+  const GenAxis &X = G[0], &Y = G[1], &Z = G[2];
+  // p < q: the other two axes
+  const float ap = c == 0 ? sel4(j, Y.A) : sel4(j, X.A), dp = c == 0 ? sel4(j, Y.DS) : sel4(j, X.DS);
+  const float aq = c == 2 ? sel4(k, Y.A) : sel4(k, Z.A), dq = c == 2 ? sel4(k, Y.DS) : sel4(k, Z.DS);
+  const float F = fmaf(ap, aq, K12 * dp * dq);
+  const int sc = c == 0 ? 1 : (c == 1 ? Box<3>::J0 : Box<3>::JP);
+  JT *p = J + c * Box<3>::JCELLS +
+          Box<3>::ji(d[0] + Box<3>::OJ + X.base, d[1] + Box<3>::OJ + Y.base, d[2] + Box<3>::OJ + Z.base) +
+          j * (c == 0 ? Box<3>::J0 : 1) + k * (c == 2 ? Box<3>::J0 : Box<3>::JP);
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+    jput<3, DET>(p + i * sc, (c == 0 ? X.P[i] : (c == 1 ? Y.P[i] : Z.P[i])) * F);
 }
 
-// a general-case particle when the record queue is full: the same rows, in
-// place (so the sorted mode's sums do not depend on which particles overflow)
-template <int D, bool DET, typename JT>
-__device__ __noinline__ void deposit_in_place(JT *Jsm, const QIn &in, float scale) {
-  QRec R;
-  queue_record<D>(R, in);
-  constexpr int NR0 = qrows<D>(0), NR1 = qrows<D>(1), IPB = NR0 + NR1 + qrows<D>(2);
-  for (int b = 0; b < R.nb; ++b)
-    for (int it = 0; it < IPB; ++it) {
-      const int c = it < NR0 ? 0 : (it < NR0 + NR1 ? 1 : 2);
-      const int row = it - (c == 0 ? 0 : (c == 1 ? NR0 : NR0 + NR1));
-      queued_row<D, DET, JT>(Jsm, R, b, c, row, scale);
-    }
-}
-
-// one row of a record added to the global fixed-point current (sorted
-// mode): each contribution rounded to the fixed-point unit as the
-// shared-memory path rounds it; grid coordinates = the record's origin + box
-// coordinates (periodic axes wrapped, nodes beyond an open face dropped, as
-// the push drops them)
-template <int D>
-__device__ __forceinline__ void record_row_global(const GridP &g, const QRec &R, int b, int c, int row,
-                                                  unsigned long long *jfx, float scale) {
-  record_row<D>(R, b, c, row, [&](int cc, int x, int y, int z, float v) {
-    const float vs = v * scale;
-    if (fabsf(vs) <= 0.5f) return;  // rounds to zero
-    const int bx[3] = {x, y, z};
-    long long gidx = 0, stride = 1;
-    bool ok = true;
+// 3D, in a strong field: every lane its own particle's rows
+template <bool DET, typename JT>
+__device__ __noinline__ void deposit_general3(JT *__restrict__ J, int two, const int *d1, const int *d2, const float *f1,
+                                              const float *f2, const float *e1, const float *e2, float qw1, float qw2,
+                                              const float *dxdt, float scale) {
+#pragma unroll 1
+  for (int b = 0; b < (two ? 2 : 1); ++b) {
+    const float q = -(b ? qw2 : qw1) * (DET ? scale : 1.0f);
+    GenAxis G[3];
+    int d[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      int cg = R.org[a] + bx[a];
-      if (a < D) {
-        if (g.bc[a] == BP_PERIODIC) cg = wrap_once(cg, g.n[a]);
-        else ok &= (cg >= 0 && cg < g.n[a]);
+      d[a] = b ? d2[a] : d1[a];
+      G[a] = general_axis(b ? f2[a] : f1[a], b ? e2[a] : e1[a], q * dxdt[a]);
+    }
+#pragma unroll 1
+    for (int it = 0; it < 48; ++it) general_row3<DET, JT>(J, d, G, it >> 4, it & 3, (it >> 2) & 3);
+  }
+}
+
+// 3D, the usual case of one such particle in a warp: the warp's active lanes
+// (mask act) share out the rows of lane src's particle.  A thermal medium has
+// one crossing in about 25 warps; alone, a lane took some 3,000 instructions
+// for it, the warp together 500.
+template <bool DET, typename JT>
+__device__ __noinline__ void deposit_general3_warp(JT *__restrict__ J, unsigned act, int src, int two, const int *d1,
+                                                   const int *d2, const float *f1, const float *f2, const float *e1,
+                                                   const float *e2, float qw1, float qw2, const float *dxdt,
+                                                   float scale) {
+  const int lane = threadIdx.x & 31, rank = __popc(act & ((1u << lane) - 1u)), n = __popc(act);
+#pragma unroll 1
+  for (int b = 0; b < (two ? 2 : 1); ++b) {
+    const float q = -(b ? qw2 : qw1) * (DET ? scale : 1.0f);
+    GenAxis G[3];
+    int d[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      d[a] = __shfl_sync(act, b ? d2[a] : d1[a], src);
+      G[a] = general_axis(__shfl_sync(act, b ? f2[a] : f1[a], src), __shfl_sync(act, b ? e2[a] : e1[a], src), q * dxdt[a]);
+    }
+#pragma unroll 1
+    for (int it = rank; it < 48; it += n) general_row3<DET, JT>(J, d, G, it >> 4, it & 3, (it >> 2) & 3);
+  }
+}
+
+// The deposit of a far body (a bound electron a cell or more from its
+// nucleus, or that nucleus) by a whole warp: four-node windows as above
+// around its own cell c, each node's value rounded to the fixed-point unit as
+// the shared-memory path rounds it and added to the global current (periodic
+// axes wrapped, nodes beyond an open face dropped, as the push drops them).
+template <int D>
+__device__ __forceinline__ void deposit_far(const GridP &g, const int c[3], const float f[3], const float de[3], float qw,
+                                            const float v[3], unsigned long long *jfx, float scale) {
+  constexpr int NODES = D == 3 ? 64 : (D == 2 ? 16 : 4);
+  constexpr float K12 = 1.0f / 12.0f;
+  GenAxis G[3];
+#pragma unroll
+  for (int a = 0; a < D; ++a) G[a] = general_axis(f[a], de[a], -qw * g.dxdt[a]);
+#pragma unroll 1
+  for (int it = threadIdx.x & 31; it < 3 * NODES; it += 32) {
+    const int cc = it / NODES, m = it - cc * NODES;
+    float A[3] = {1.0f, 1.0f, 1.0f}, S[3] = {0.0f, 0.0f, 0.0f}, val = 0.0f;
+    long long gi = 0, stride = 1;
+    bool ok = true;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      const int k = (m >> (2 * a)) & 3;
+      if (a == cc) {
+        val = k == 0 ? G[a].P[0] : (k == 1 ? G[a].P[1] : (k == 2 ? G[a].P[2] : 0.0f));
+      } else {
+        A[a] = sel4(k, G[a].A);
+        S[a] = sel4(k, G[a].DS);
       }
-      gidx += (long long)cg * stride;
+      int x = c[a] + G[a].base + k;
+      if (g.bc[a] == BP_PERIODIC) x = wrap_once(x, g.n[a]);
+      else ok &= x >= 0 && x < g.n[a];
+      gi += (long long)x * stride;
       stride *= g.n[a];
     }
-    if (ok) atomicAdd(jfx + (size_t)cc * g.ncell + gidx, (unsigned long long)f2ll_rn(vs));
-  });
-}
-
-// a one-body deposit with its own grid origin org (a bound electron pulled
-// a cell or more from its nucleus, outside the tile's current box): queued as
-// a record for k_records, or, when the record buffer is full, added to the
-// global current here
-template <int D>
-__device__ __noinline__ void deposit_far(const GridP &g, const QIn &in, const int org[3], QRec *qrec, int *qn,
-                                         int qmax, unsigned long long *jfx, float scale) {
-  const int slot = atomicAdd(qn, 1);
-  if (slot < qmax) {
-    queue_record<D>(qrec[slot], in);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) qrec[slot].org[a] = org[a];
-    return;
-  }
-  QRec R;
-  queue_record<D>(R, in);
-#pragma unroll
-  for (int a = 0; a < 3; ++a) R.org[a] = org[a];
-  constexpr int NR0 = qrows<D>(0), NR1 = qrows<D>(1), IPB = NR0 + NR1 + qrows<D>(2);
-  for (int it = 0; it < IPB; ++it) {
-    const int c = it < NR0 ? 0 : (it < NR0 + NR1 ? 1 : 2);
-    const int row = it - (c == 0 ? 0 : (c == 1 ? NR0 : NR0 + NR1));
-    record_row_global<D>(g, R, 0, c, row, jfx, scale);
+    if (cc >= D) val = qw * (cc == 1 ? v[1] : v[2]);
+    // the two transverse axes (at most two of the three differences are not 0)
+    const float F = A[0] * A[1] * A[2] + K12 * (S[0] * S[1] + S[1] * S[2] + S[0] * S[2]);
+    const float vs = val * F * scale;
+    if (ok && fabsf(vs) > 0.5f) atomicAdd(jfx + (size_t)cc * g.ncell + gi, (unsigned long long)f2ll_rn(vs));
   }
 }
 
-// E and B of one body read from the global fields (a body outside the
-// tile's staged box): the staggered quadratic gather over the body's cell c
-// and offset f, periodic axes wrapped, zero beyond open faces
+// E and B of one body read from the global fields by a whole warp (a body
+// outside the tile's staged box): the staggered quadratic gather over the
+// body's cell c and offset f, one lane per node of the stencil, summed in a
+// fixed order; periodic axes wrapped, zero beyond open faces
 template <int D>
-__device__ __noinline__ void gather_global(const GridP &g, const float *const *Eg, const float *const *Bg,
-                                           const int c[3], const float f[3], float E[3], float B[3]) {
-#pragma unroll 1
+__device__ __forceinline__ void gather_global(const GridP &g, const float *const *Eg, const float *const *Bg,
+                                              const int c[3], const float f[3], float E[3], float B[3]) {
+  constexpr int NODES = D == 3 ? 27 : (D == 2 ? 9 : 3);
+  const int lane = threadIdx.x & 31;
+  const int o[3] = {lane % 3, (lane / 3) % 3, lane / 9};
+#pragma unroll
   for (int cc = 0; cc < 6; ++cc) {
     // stagger pattern of component cc: bit a set when it sits half a cell along a
     const int pat = cc < 3 ? (1 << cc) : (7 & ~(1 << (cc - 3)));
-    const float *F = cc < 3 ? Eg[cc] : Bg[cc - 3];
-    int base[3];
-    float w[3][3];
+    long long gi = 0, stride = 1;
+    float w = 1.0f;
+    bool ok = lane < NODES;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      if (a < D) {
-        const bool half = (pat >> a) & 1;
-        const int up = half ? 0 : (f[a] >= 0.5f ? 1 : 0);
-        base[a] = c[a] + up - 1;
-        qweights(half ? f[a] - 0.5f : f[a] - (float)up, w[a]);
-      } else {
-        base[a] = 0;
-        w[a][0] = 1.0f;
-        w[a][1] = w[a][2] = 0.0f;
-      }
+    for (int a = 0; a < D; ++a) {
+      const bool half = (pat >> a) & 1;
+      const int up = half ? 0 : (f[a] >= 0.5f ? 1 : 0);
+      float wa[3];
+      qweights(half ? f[a] - 0.5f : f[a] - (float)up, wa);
+      w *= o[a] == 0 ? wa[0] : (o[a] == 1 ? wa[1] : wa[2]);
+      int x = c[a] + up - 1 + o[a];
+      if (g.bc[a] == BP_PERIODIC) x = wrap_once(x, g.n[a]);
+      else ok &= x >= 0 && x < g.n[a];
+      gi += (long long)x * stride;
+      stride *= g.n[a];
     }
-    float acc = 0.0f;
-    for (int k = 0; k < (D >= 3 ? 3 : 1); ++k)
-      for (int j = 0; j < (D >= 2 ? 3 : 1); ++j)
-        for (int i = 0; i < 3; ++i) {
-          const int n[3] = {base[0] + i, base[1] + j, base[2] + k};
-          long long gi = 0, stride = 1;
-          bool ok = true;
+    float acc = ok ? w * (cc < 3 ? Eg[cc] : Bg[cc - 3])[gi] : 0.0f;
 #pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            int x = n[a];
-            if (a < D) {
-              if (g.bc[a] == BP_PERIODIC) x = wrap_once(x, g.n[a]);
-              else ok &= (x >= 0 && x < g.n[a]);
-            } else {
-              x = 0;
-            }
-            gi += (long long)x * stride;
-            stride *= g.n[a];
-          }
-          if (ok) acc = fmaf(w[0][i] * w[1][j] * w[2][k], F[gi], acc);
-        }
+    for (int q = 16; q > 0; q >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, q);
     if (cc < 3) E[cc] = acc;
     else B[cc - 3] = acc;
   }
@@ -529,7 +551,7 @@ __device__ __forceinline__ void bb_add(unsigned &lo, unsigned &hi, const int n[3
   hi = __vmaxu4(hi, h);
 }
 
-// the five-node window's centre node (as window() places it)
+// the centre node of a body's general window (it reaches two nodes either way)
 template <int D>
 __device__ __forceinline__ void window_centre(const float *f, const int *d, int n0[3]) {
 #pragma unroll
@@ -672,17 +694,16 @@ __device__ __forceinline__ bool quiet_done(const PartP &P, long long i) {
 // The whole step of a two-body ion whose bound electron is a cell or more
 // from its nucleus (a strong field pulls it into the Coulomb tail of the
 // modified potential), sorted mode: outside the tile's boxes, so both bodies
-// gather from the global E and B and deposit as one-body records at their own
-// grid origins (k_records adds them to the fixed-point current; directly
-// when the record buffer is full).  The same arithmetic as push_particle's.
-// Out of line and self-contained (it reloads the particle), so the common
-// path carries none of it.  Returns false when the ion cannot be moved this
-// way (body 1 outside its tile's margin, body 2 beyond an open face or a
-// displacement that is not finite): a domain error for the caller.
+// gather from the global E and B and deposit into the global fixed-point
+// current.  The same arithmetic as push_particle's.
+// A whole warp per ion (every lane holds the ion; lane 0 writes it).  Returns
+// false when the ion cannot be moved this way (body 1 outside its tile's
+// margin, body 2 beyond an open face or a displacement that is not finite): a
+// domain error for the caller.
 template <int D>
-__device__ __noinline__ bool push_far(const GridP &g, const SpecP &sp, const PartP &P, long long i, int t0x, int t0y,
-                                      int t0z, int *status, QRec *qrec, int *qn, int qmax, const float *const *Eg,
-                                      const float *const *Bg, unsigned long long *jfx, float scale) {
+__device__ __forceinline__ bool push_far(const GridP &g, const SpecP &sp, const PartP &P, long long i, int t0x, int t0y,
+                                      int t0z, int *status, const float *const *Eg, const float *const *Bg,
+                                      unsigned long long *jfx, float scale) {
   const long long cap = P.cap;
   const int T0[3] = {t0x, t0y, t0z};
   int c[3];
@@ -746,28 +767,10 @@ __device__ __noinline__ bool push_far(const GridP &g, const SpecP &sp, const Par
     rn[a] = r[a] + g.dt * (v1[a] - v2[a]);
     if (a < D) de2[a] = de1[a] - (rn[a] - r[a]) * g.idx[a];
   }
-  // each body a one-body record at its own grid origin (cell - OJ)
-  QIn in;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    in.f[a] = f[a]; in.de1[a] = de1[a]; in.v1[a] = v1[a]; in.dxdt[a] = g.dxdt[a]; in.d[a] = 0;
-    in.f2[a] = in.de2[a] = in.v2[a] = 0.0f;
-    in.d2[a] = 0;
-  }
-  in.qw1 = sp.qw1;
-  in.qw2 = 0.0f;
-  in.two = 0;
-  int org[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) org[a] = a < D ? c[a] - Box<D>::OJ : 0;
-  deposit_far<D>(g, in, org, qrec, qn, qmax, jfx, scale);
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    in.f[a] = f2[a]; in.de1[a] = de2[a]; in.v1[a] = v2[a];
-    org[a] = a < D ? c2[a] - Box<D>::OJ : 0;
-  }
-  in.qw1 = sp.qw2;
-  deposit_far<D>(g, in, org, qrec, qn, qmax, jfx, scale);
+  // each body on its own, around its own cell
+  deposit_far<D>(g, c, f, de1, sp.qw1, v1, jfx, scale);
+  deposit_far<D>(g, c2, f2, de2, sp.qw2, v2, jfx, scale);
+  if (threadIdx.x & 31) return true;
   bool bad = false, removed = false, need_sort = false, nonfinite = false;
   advance_cell<D>(g, T0, true, c, fn, bad, removed, need_sort);
 #pragma unroll
@@ -793,8 +796,7 @@ __device__ __noinline__ bool push_far(const GridP &g, const SpecP &sp, const Par
 
 template <int D, bool DET, typename JT>
 __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, long long i, const int T0[3],
-                              const float *Gsm, JT *Jsm, int *status, float scale, QRec *qrec, int *qn, int qmax,
-                              unsigned &blo, unsigned &bhi, bool nofield, int4 *far, int *far_n, int far_cap, int s,
+                              const float *Gsm, JT *Jsm, int *status, float scale, unsigned &blo, unsigned &bhi, bool nofield, int4 *far, int *far_n, int far_cap, int s,
                               int t) {
   const long long cap = P.cap;
   const bool two = sp.kind == BP_TWO_BODY;
@@ -939,6 +941,33 @@ __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, l
   bool silent = two && sp.qw1 == -sp.qw2;
 #pragma unroll
   for (int a = 0; a < 3; ++a) silent &= (r[a] == 0.0f) && (v1[a] == v2[a]);
+  if constexpr (D == 3) {
+    // the general case in 3D: rare in a thermal medium, so the warp's lanes
+    // share out the rows of one such particle after the other; with more than
+    // three of them every lane does its own
+    const unsigned act = __activemask();
+    unsigned gen = __ballot_sync(act, !silent && !fast);
+    if (gen) {
+      float fb[2][3], db[2][3], dd[3];
+      int cb[2][3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        fb[0][a] = f[a]; fb[1][a] = f2[a];
+        db[0][a] = de1[a]; db[1][a] = de2[a];
+        cb[0][a] = d[a]; cb[1][a] = d2[a];
+        dd[a] = dxdt[a];
+      }
+      if (__popc(gen) > 3) {
+        if (!silent && !fast)
+          deposit_general3<DET, JT>(Jsm, two, cb[0], cb[1], fb[0], fb[1], db[0], db[1], sp.qw1, sp.qw2, dd, scale);
+      } else {
+        for (; gen; gen &= gen - 1)
+          deposit_general3_warp<DET, JT>(Jsm, act, __ffs(gen) - 1, two, cb[0], cb[1], fb[0], fb[1], db[0], db[1],
+                                         sp.qw1, sp.qw2, dd, scale);
+      }
+      __syncwarp(act);
+    }
+  }
   if (!silent) {
     if (fast) {
       float qw[2] = {sp.qw1, sp.qw2};
@@ -958,34 +987,27 @@ __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, l
       else esirkepov3<D, DET, 1>(Jsm, nn, xi, dd, qw, vv, dxdt, scale);
       bb_add<D>(blo, bhi, nn, 1, 1);
     } else {
-      QIn in;
+      if constexpr (D < 3) {
+#pragma unroll 1
+        for (int b = 0; b < (two ? 2 : 1); ++b) {
+          float fb[3], db[3], vb[3];
+          int cb[3];
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        in.f[a] = f[a]; in.de1[a] = de1[a]; in.f2[a] = f2[a]; in.de2[a] = de2[a];
-        in.v1[a] = v1[a]; in.v2[a] = v2[a]; in.dxdt[a] = dxdt[a]; in.d[a] = d[a]; in.d2[a] = d2[a];
-      }
-      in.qw1 = sp.qw1;
-      in.qw2 = sp.qw2;
-      in.two = two;
-      // sorted mode: qrec, qn, qmax are the global record buffer, its counter
-      // and capacity; atomic mode: the block's shared-memory queue
-      const int slot = atomicAdd(qn, 1);
-      const bool queued = slot < qmax;
-      if (queued) {
-        queue_record<D>(qrec[slot], in);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) qrec[slot].org[a] = T0[a] - (a < D ? Box<D>::OJ : 0);
-      } else {
-        deposit_in_place<D, DET, JT>(Jsm, in, scale);
-      }
-      if (!DET || !queued) {
-        int n0[3];
-        window_centre<D>(f, d, n0);
-        bb_add<D>(blo, bhi, n0, 2, 2);
-        if (two) {
-          window_centre<D>(f2, d2, n0);
-          bb_add<D>(blo, bhi, n0, 2, 2);
+          for (int a = 0; a < 3; ++a) {
+            fb[a] = b ? f2[a] : f[a];
+            db[a] = b ? de2[a] : de1[a];
+            vb[a] = b ? v2[a] : v1[a];
+            cb[a] = b ? d2[a] : d[a];
+          }
+          deposit_general<D, DET, JT>(Jsm, cb, fb, db, b ? sp.qw2 : sp.qw1, vb, dxdt, scale);
         }
+      }
+      int n0[3];
+      window_centre<D>(f, d, n0);
+      bb_add<D>(blo, bhi, n0, 2, 2);
+      if (two) {
+        window_centre<D>(f2, d2, n0);
+        bb_add<D>(blo, bhi, n0, 2, 2);
       }
     }
   }
@@ -1348,22 +1370,14 @@ __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, con
   // happens to be all zero goes the full way, which leaves the same bits;
   // reading every staged value to find it cost 1% of the 3D push)
   const bool nofield = qs != QS_PUSH;
-  QRec *qrec = DET ? reinterpret_cast<QRec *>(A.grec)
-                   : reinterpret_cast<QRec *>(smem + GOFF + sizeof(float) * 6 * (size_t)GC);
-  int *const qcount = DET ? A.grec_n : nullptr;
-  const int qmax = DET ? A.grec_cap : push_qmax(D);
-  constexpr int NR0 = qrows<D>(0), NR1 = qrows<D>(1), IPB = NR0 + NR1 + qrows<D>(2);
-  __shared__ int qn, run;
+  __shared__ int run;
   __shared__ unsigned sbb[6];
   if (tid < 6) sbb[tid] = tid < 3 ? 0xFFFFFFFFu : 0u;
   unsigned blo = 0xFFFFFFFFu, bhi = 0u;
   unsigned pushed = 0;
   const int lane = tid & 31;
   for (int s = 0; s < A.nsp; ++s) {
-    if (tid == 0) {
-      qn = 0;
-      run = 0;
-    }
+    if (tid == 0) run = 0;
     __syncthreads();
     const int beg = A.p[s].tstart[t], end = A.p[s].tstart[t + 1], n = end - beg;
     // in a QS_REST tile the quiet ions of this species have already moved
@@ -1396,22 +1410,11 @@ __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, con
       if (k < n && !(moved && quiet_done(A.p[s], i))) {
         const int kn = at(rn);
         if (kn < n) prefetch_particle<D>(A.p[s], beg + kn, two);
-        push_particle<D, DET, JT>(g, A.sp[s], A.p[s], i, T0, Gsm, Jsm, A.status, A.jscale, qrec,
-                                  DET ? qcount : &qn, qmax, blo, bhi, nofield, A.far, A.far_n, A.far_cap, s, t);
+        push_particle<D, DET, JT>(g, A.sp[s], A.p[s], i, T0, Gsm, Jsm, A.status, A.jscale, blo,
+                                  bhi, nofield, A.far, A.far_n, A.far_cap, s, t);
         ++pushed;
       }
       r = rn;
-    }
-    __syncthreads();
-    if constexpr (DET) continue;  // the records are deposited by k_records
-    // the deferred general deposits, one row per thread
-    const int nitem = min(qn, qmax) * 2 * IPB;
-    for (int k = tid; k < nitem; k += bs) {
-      const int e = k / (2 * IPB), rem = k - e * (2 * IPB), b = rem / IPB, it = rem - b * IPB;
-      if (b >= qrec[e].nb) continue;
-      const int c = it < NR0 ? 0 : (it < NR0 + NR1 ? 1 : 2);
-      const int row = it - (c == 0 ? 0 : (c == 1 ? NR0 : NR0 + NR1));
-      queued_row<D, DET, JT>(Jsm, qrec[e], b, c, row, A.jscale);
     }
     __syncthreads();
   }
@@ -1484,8 +1487,15 @@ __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, con
 // tiles the quiet-tile pass left (its list) in order from a counter, so a
 // block's shared memory and setup are reused from tile to tile, and the next
 // tile's field box is staged while the block finishes the current one.
-template <int D, bool DET>
-__global__ void __launch_bounds__(push_threads(D)) k_push(GridP g, PushArgs A, const __grid_constant__ TmaMaps T) {
+//
+// PB: blocks per SM the registers are held to.  2D grids with free particles
+// take 3 (80 registers): a tile's work is short there and its barriers and
+// instruction fetches are hidden by other blocks (4.2 M electrons, step of
+// the ionised crystal: 0.62 ms with 2, 0.56 with 3, 0.61 with 4, which
+// spills).  Two-body ions need the registers (524 k ions: the adjoint cycle
+// 179 ms with 2, 185 with 3).
+template <int D, bool DET, int PB>
+__global__ void __launch_bounds__(push_threads(D), PB) k_push(GridP g, PushArgs A, const __grid_constant__ TmaMaps T) {
   extern __shared__ __align__(128) unsigned char smem[];
   float *Gsm = reinterpret_cast<float *>(smem + push_gbox_offset(D, DET));
   __shared__ int next;
@@ -1522,39 +1532,21 @@ __global__ void __launch_bounds__(push_threads(D)) k_push(GridP g, PushArgs A, c
   if (next >= 0 && A.qstate[next] == QS_PUSH) stage_done<D>(g, A, T, next, &bar, phase, failed);
 }
 
-// Sorted mode: the records' rows added to the fixed-point current.  Each
-// contribution is rounded to the fixed-point unit as the shared-memory path
-// rounds it (the same value, so the current does not depend on which path a
-// particle took); nodes beyond an open face are dropped as the push drops them.
-template <int D>
-__global__ void __launch_bounds__(256) k_records(GridP g, const QRec *__restrict__ rec, const int *__restrict__ count,
-                                                 int cap, unsigned long long *jfx, float scale) {
-  constexpr int NR0 = qrows<D>(0), NR1 = qrows<D>(1), IPB = NR0 + NR1 + qrows<D>(2);
-  const long long n = (long long)min(*count, cap) * 2 * IPB;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-    const int e = (int)(k / (2 * IPB)), rem = (int)(k - (long long)e * 2 * IPB), b = rem / IPB, it = rem - b * IPB;
-    const QRec &R = rec[e];
-    if (b >= R.nb) continue;
-    const int c = it < NR0 ? 0 : (it < NR0 + NR1 ? 1 : 2);
-    const int row = it - (c == 0 ? 0 : (c == 1 ? NR0 : NR0 + NR1));
-    record_row_global<D>(g, R, b, c, row, jfx, scale);
-  }
-}
-
 // Sorted mode: the ions the push listed as far (a bound electron a cell or
 // more from its nucleus), each moved by push_far; anything push_far cannot
 // move is a domain error.
 template <int D>
 __global__ void __launch_bounds__(128) k_push_far(GridP g, PushArgs A) {
-  const int n = min(*A.far_n, A.far_cap);
+  const int n = min(*A.far_n, A.far_cap), lane = threadIdx.x & 31;
   if (blockIdx.x == 0 && threadIdx.x == 0 && A.far_any) *A.far_any = n > 0;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+  const int warps = gridDim.x * (blockDim.x >> 5);
+  for (int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += warps) {
     const int4 e = A.far[k];
     const int t = e.z;
     const int T0[3] = {(t % g.nt[0]) * Geo<D>::L0, ((t / g.nt[0]) % g.nt[1]) * Geo<D>::L1,
                        (t / (g.nt[0] * g.nt[1])) * Geo<D>::L2};
-    if (!push_far<D>(g, A.sp[e.x], A.p[e.x], e.y, T0[0], T0[1], T0[2], A.status, reinterpret_cast<QRec *>(A.grec),
-                     A.grec_n, A.grec_cap, A.E, A.B, A.jfx, A.jscale))
+    if (!push_far<D>(g, A.sp[e.x], A.p[e.x], e.y, T0[0], T0[1], T0[2], A.status, A.E, A.B, A.jfx, A.jscale) &&
+        lane == 0)
       atomicOr(A.status, ST_DOMAIN);
   }
 }
@@ -1567,45 +1559,45 @@ void launch_one(const GridP &g, const PushArgs &a, const TmaMaps &tm, cudaStream
   const size_t smem = push_smem_bytes(g, DET);
   // as many persistent blocks as the device holds at once (worked out per
   // context for its grid and device when it was created)
-  const int blocks = a.push_blocks > 0 ? a.push_blocks : 1;
+  bool free_sp = false;
+  for (int k = 0; k < a.nsp; ++k) free_sp |= a.sp[k].kind == BP_FREE;
+  const int v = D == 2 && free_sp ? 1 : 0;
+  const int blocks = a.push_blocks[v] > 0 ? a.push_blocks[v] : 1, nb = blocks < g.ntiles ? blocks : g.ntiles;
   cudaMemsetAsync(a.tile_ctr, 0, sizeof(int), s);
-  k_push<D, DET><<<blocks < g.ntiles ? blocks : g.ntiles, push_threads(D), smem, s>>>(g, a, tm);
+  if (v) k_push<D, DET, push_pb(D, true)><<<nb, push_threads(D), smem, s>>>(g, a, tm);
+  else k_push<D, DET, push_pb(D, false)><<<nb, push_threads(D), smem, s>>>(g, a, tm);
   if constexpr (DET) {
-    k_push_far<D><<<a.sms, 128, 0, s>>>(g, a);
+    k_push_far<D><<<a.sms * 4, 128, 0, s>>>(g, a);
     cudaMemsetAsync(a.far_n, 0, sizeof(int), s);
-    k_records<D><<<a.sms * 8, 256, 0, s>>>(g, reinterpret_cast<const QRec *>(a.grec), a.grec_n, a.grec_cap, a.jfx,
-                                          a.jscale);
-    cudaMemsetAsync(a.grec_n, 0, sizeof(int), s);
   }
 }
 
-template <int D, bool DET>
-int prepare_one(const GridP &g, int *blocks) {
+template <int D, bool DET, int PB>
+int prepare_variant(const GridP &g, int *blocks) {
   const size_t smem = push_smem_bytes(g, DET);
-  cudaError_t e = cudaFuncSetAttribute(k_push<D, DET>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_push<D, DET, PB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return -1;
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return -1;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_push<D, DET>, push_threads(D), smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_push<D, DET, PB>, push_threads(D), smem);
   if (e != cudaSuccess) return -1;
   *blocks = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
   return 0;
 }
 
+template <int D, bool DET>
+int prepare_one(const GridP &g, int blocks[2]) {
+  return prepare_variant<D, DET, push_pb(D, false)>(g, blocks) || prepare_variant<D, DET, push_pb(D, true)>(g, blocks + 1) ? -1
+                                                                                                                         : 0;
+}
+
 }  // namespace
 
 size_t push_smem_bytes(const GridP &g, int det) {
-  int jc = 0, gc = 0;
-  if (g.D == 1) { jc = Box<1>::JCELLS; gc = Box<1>::GCELLS; }
-  if (g.D == 2) { jc = Box<2>::JCELLS; gc = Box<2>::GCELLS; }
-  if (g.D == 3) { jc = Box<3>::JCELLS; gc = Box<3>::GCELLS; }
-  // the sorted mode keeps its records in global memory
-  (void)jc;
-  return push_gbox_offset(g.D, det != 0) + 4 * (size_t)6 * gc + (det ? 0 : sizeof(QRec) * (size_t)push_qmax(g.D));
+  const int gc = g.D == 1 ? Box<1>::GCELLS : (g.D == 2 ? Box<2>::GCELLS : Box<3>::GCELLS);
+  return push_gbox_offset(g.D, det != 0) + 4 * (size_t)6 * gc;
 }
-
-size_t push_record_bytes() { return sizeof(QRec); }
 
 void launch_tile_active(const GridP &g, const unsigned char *qstate, const int *far_any, int ia_lo, int ia_hi,
                         unsigned char *act, unsigned long long *act_n, cudaStream_t s) {
@@ -1615,7 +1607,7 @@ void launch_tile_active(const GridP &g, const unsigned char *qstate, const int *
   else k_tile_active<3><<<nb, 256, 0, s>>>(g, qstate, far_any, ia_lo, ia_hi, act, act_n);
 }
 
-int push_prepare(const GridP &g, int det, int *blocks) {
+int push_prepare(const GridP &g, int det, int blocks[2]) {
   switch (g.D * 2 + (det ? 1 : 0)) {
     case 2: return prepare_one<1, false>(g, blocks);
     case 3: return prepare_one<1, true>(g, blocks);

@@ -302,13 +302,19 @@ int bp_create(const bp_grid_desc *gd, const bp_allocator *al, void *stream, bp_c
       return BP_ERR_OOM;
     }
   }
+  for (int k = 0; k < 3; ++k) {
+    c->Bn[k] = (float *)dalloc(c, sizeof(float) * ncell);
+    if (!c->Bn[k]) {
+      bp_destroy(c);
+      return BP_ERR_OOM;
+    }
+  }
   // sorted deposit: the tiles add their current to a global 64-bit fixed-point
   // array; atomic deposit: per-tile FP32 boxes summed by the current-sum kernel
   if (c->det) {
     c->jfx = (unsigned long long *)dalloc(c, sizeof(unsigned long long) * 3 * (size_t)ncell);
     c->ant = (double *)dalloc(c, sizeof(double) * BP_MAX_LASER * (size_t)(ncell / g.n[0]));
     c->far_n = (int *)dalloc(c, sizeof(int));
-    c->far_any = (int *)dalloc(c, sizeof(int));
   }
   else c->jbox = (float *)dalloc(c, sizeof(float) * 3 * (size_t)g.jcells * g.ntiles);
   c->occ = (unsigned char *)dalloc(c, g.ntiles);
@@ -330,14 +336,15 @@ int bp_create(const bp_grid_desc *gd, const bp_allocator *al, void *stream, bp_c
   c->clk = (long long *)dalloc(c, sizeof(long long) * kClockWords);
   long long nf = frame_floats(g);
   c->frame = nf ? (float *)dalloc(c, sizeof(float) * nf) : nullptr;
-  if (!(c->det ? (void *)c->jfx : (void *)c->jbox) || (c->det && (!c->ant || !c->far_n || !c->far_any)) || !c->tile_ctr || !c->tile_list || !c->tile_n || !c->occ || !c->jbb || !g.fnz || !c->qstate || !c->status ||
+  if (!(c->det ? (void *)c->jfx : (void *)c->jbox) || (c->det && (!c->ant || !c->far_n)) || !c->tile_ctr || !c->tile_list || !c->tile_n || !c->occ || !c->jbb || !g.fnz || !c->qstate || !c->status ||
       !c->work || !c->clk || (g.ntiles >= 1024 && (!c->act || !c->act_n)) || (nf && !c->frame)) {
     bp_destroy(c);
     return BP_ERR_OOM;
   }
   // 3D: tensor maps for the TMA staging of the push's field boxes (without
   // them every tile is staged by per-thread copies)
-  if (encode_field_maps(g, c->F, &c->tmaps)) c->tmaps.on = 0;
+  float *const staged[6] = {c->F[0], c->F[1], c->F[2], c->Bn[0], c->Bn[1], c->Bn[2]};
+  if (encode_field_maps(g, staged, &c->tmaps)) c->tmaps.on = 0;
   cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
   if (c->sms < 1) c->sms = 1;
   if (push_prepare(g, c->det, c->push_blocks)) {
@@ -671,14 +678,21 @@ PushArgs push_args(bp_ctx *c, int *nsp_out) {
   A.nsp = nsp;
   for (int k = 0; k < 3; ++k) {
     A.E[k] = c->F[k];
-    A.B[k] = c->F[3 + k];
+    A.B[k] = c->Bn[k];
   }
   A.jbox = c->jbox;
   A.jfx = c->jfx;
   A.far = c->far;
   A.far_n = c->far_n;
   A.far_cap = (int)c->far_cap;
-  A.far_any = c->far_any;
+  A.act = c->act;
+  A.act_n = c->act_n;
+  A.ia_lo = INT_MAX;
+  A.ia_hi = INT_MIN;
+  for (auto &L : c->las) {
+    A.ia_lo = std::min(A.ia_lo, L.ia);
+    A.ia_hi = std::max(A.ia_hi, L.ia);
+  }
   A.occ = c->occ;
   A.jbb = c->jbb;
   A.qstate = c->qstate;
@@ -816,6 +830,19 @@ void launch_resort(bp_ctx *c, int nsp, cudaStream_t st) {
   }
 }
 
+ProbeArgs probe_args(const bp_ctx *c) {
+  ProbeArgs P;
+  memset(&P, 0, sizeof P);
+  for (auto &p : c->pr) {
+    P.F[P.n] = c->F[p.comp];
+    P.nodes[P.n] = p.nodes;
+    P.npts[P.n] = p.npts;
+    P.buf[P.n] = p.buf;
+    ++P.n;
+  }
+  return P;
+}
+
 // The launches of one leapfrog step after the re-sort, on stream st.  They
 // are the same every step (the time and the probe slots come from the device
 // clock), so a plain step and a replay of their captured graph do the same
@@ -827,10 +854,15 @@ void step_launches(bp_ctx *c, const PushArgs &A, bool probes, cudaStream_t st, f
   const GridP &g = c->g;
   float *E[3] = {c->F[0], c->F[1], c->F[2]}, *B[3] = {c->F[3], c->F[4], c->F[5]}, *J[3] = {c->F[6], c->F[7], c->F[8]};
   const float *cE[3] = {E[0], E[1], E[2]}, *cB[3] = {B[0], B[1], B[2]};
-  launch_yee_b(g, B, cE, 0.5f * g.dt, c->act, st);
+  // the antenna's sheets run with the quiet-tile pass, or with the B update
+  // where the push goes without that pass
+  const AntArgs ant = antenna_args(g, c->las.data(), c->det ? (int)c->las.size() : 0, c->clk, c->ant), none{};
+  const bool direct = push_direct(g, A);
+  launch_yee_b(g, B, c->Bn, cE, 0.5f * g.dt, c->jfx, A, direct ? ant : none, c->act, st);
   if (snap_fields) {
     CopyList L;
-    for (int k = 0; k < 6; ++k) cl_add(c, L, c->F[k], snap_fields + (size_t)k * g.ncell, sizeof(float) * g.ncell);
+    for (int k = 0; k < 6; ++k)
+      cl_add(c, L, k < 3 ? c->F[k] : c->Bn[k - 3], snap_fields + (size_t)k * g.ncell, sizeof(float) * g.ncell);
     int q = 0;
     for (auto &s : c->sp)
       if (s.loaded) cl_parts(c, L, s.p, (*snap_parts)[q++].p, g.D, s.sp.kind == BP_TWO_BODY);
@@ -846,42 +878,31 @@ void step_launches(bp_ctx *c, const PushArgs &A, bool probes, cudaStream_t st, f
     }
     cudaEventRecord(c->ev[c->ev_used], st);
   }
-  launch_push(g, A, c->tmaps, st);
+  launch_push(g, A, c->tmaps, direct ? none : ant, st);
   if (c->timing) {
     cudaEventRecord(c->ev[c->ev_used + 1], st);
     c->ev_used += 2;
   }
   if (!c->det) launch_jsum(g, c->jbox, c->occ, c->jbb, J, c->las.data(), (int)c->las.size(), c->clk, st);
-  if (c->act) {
-    int ia_lo = INT_MAX, ia_hi = INT_MIN;
-    for (auto &L : c->las) {
-      ia_lo = std::min(ia_lo, L.ia);
-      ia_hi = std::max(ia_hi, L.ia);
-    }
-    launch_tile_active(g, c->qstate, c->far_any, ia_lo, ia_hi, c->act, c->act_n, st);
-  }
-  launch_yee_b(g, B, cE, 0.5f * g.dt, c->act, st);
   launch_yee_e(g, E, cB, J, c->frame, c->det ? c->jfx : nullptr, c->jinv, c->las.data(), (int)c->las.size(), c->clk,
                c->ant, c->act, st);
-  if (probes)
-    for (size_t p = 0; p < c->pr.size(); ++p)
-      launch_probe(c->F[c->pr[p].comp], c->pr[p].nodes, c->pr[p].npts, c->pr[p].buf, c->clk, (int)p, st);
-  launch_clock_tick(c->clk, probes ? (int)c->pr.size() : 0, st);
+  if (probes) launch_probes(probe_args(c), c->clk, st);
 }
 
 // the host's record of one step (the device's is the clock)
-void step_account(bp_ctx *c, bool probes) {
+void step_account(bp_ctx *c, const PushArgs &A, bool probes) {
   int nopen = 0;
   for (int a = 0; a < c->g.D; ++a) nopen += c->g.bc[a] == BP_OPEN;
-  // quiet-tile pass, push, far ions (sorted) or current sum (atomic), antenna (sorted, with lasers),
-  // Yee (3), Mur, the clock
-  c->launches += 6 + (c->det && !c->las.empty() ? 1 : 0) + (nopen ? 1 + nopen : 0) + 1 + (c->act ? 1 : 0);
-  c->step++;
-  if (probes)
-    for (auto &p : c->pr) {
-      c->launches++;
+  // B update, quiet-tile pass, push, far ions and tile flags, current sum
+  // (atomic), E update; Mur faces that the E update does not do itself
+  c->launches += 3 + (push_direct(c->g, A) ? 0 : 1) + (c->det || c->act ? 1 : 0) + (c->det ? 0 : 1);
+  if (nopen > 1 || (nopen == 1 && c->g.bc[0] != BP_OPEN)) c->launches += 1 + nopen;
+  if (probes) {
+    c->launches += probe_launches(probe_args(c));
+    for (auto &p : c->pr)
       if (p.count < p.cap) p.count++;
-    }
+  }
+  c->step++;
 }
 
 // one leapfrog step, launched directly
@@ -889,17 +910,17 @@ int one_step(bp_ctx *c, const PushArgs &A, int nsp, bool probes, float *snap_fie
              std::vector<bp_part_copy> *snap_parts) {
   launch_resort(c, nsp, c->stream);
   step_launches(c, A, probes, c->stream, snap_fields, snap_parts);
-  step_account(c, probes);
+  step_account(c, A, probes);
   return check_launch(c, "step");
 }
 
 // one step through the step graph (step_graph succeeded for the current
 // arguments): one launch when the graph holds the re-sort, else two
-int graph_step(bp_ctx *c, int nsp) {
+int graph_step(bp_ctx *c, const PushArgs &A, int nsp) {
   if (c->step_sorts) c->launches += 1;  // the re-sort's condition kernel
   else launch_resort(c, nsp, c->stream);
   cudaGraphLaunch(c->step_exec, c->stream);
-  step_account(c, true);
+  step_account(c, A, true);
   return check_launch(c, "step graph");
 }
 
@@ -914,6 +935,7 @@ bool step_graph(bp_ctx *c, const PushArgs &A) {
   put(&c->tmaps, sizeof c->tmaps);
   put(&c->g, sizeof c->g);
   put(c->F, sizeof c->F);
+  put(c->Bn, sizeof c->Bn);
   const void *ptrs[] = {c->jfx, c->jbox, c->occ, c->jbb, c->frame, c->ant, c->clk, c->sort_runs_dev};
   put(ptrs, sizeof ptrs);
   put(&c->sb, sizeof c->sb);
@@ -992,7 +1014,7 @@ int bp_step(bp_ctx *c, int64_t nsteps) {
   const bool graph = nsteps >= 2 && !c->timing && step_graph(c, A);
   for (int64_t it = 0; it < nsteps; ++it) {
     int rc;
-    rc = graph ? graph_step(c, nsp) : one_step(c, A, nsp, true, nullptr, nullptr);
+    rc = graph ? graph_step(c, A, nsp) : one_step(c, A, nsp, true, nullptr, nullptr);
     if (rc) return rc;
   }
   return BP_OK;
@@ -1634,7 +1656,7 @@ int bp_forward_ckpt(bp_ctx *c, int64_t nsteps, int K) {
     cl_flush(c, L);
     long long len = std::min<long long>(K, nsteps - (long long)k * K);
     for (long long j = 0; j < len; ++j) {
-      int rc = graph ? graph_step(c, nsp) : one_step(c, A, nsp, true, nullptr, nullptr);
+      int rc = graph ? graph_step(c, A, nsp) : one_step(c, A, nsp, true, nullptr, nullptr);
       if (rc) return rc;
     }
   }

@@ -70,12 +70,12 @@ struct bp_ctx {
   cudaStream_t stream = nullptr;
   int device = 0;
   float *F[9] = {};
+  float *Bn[3] = {};                 // B^n of the current step (F[3..5]: B at half steps)
   float *jbox = nullptr;             // atomic deposit: per-tile FP32 current boxes
   unsigned long long *jfx = nullptr; // sorted deposit: [3][ncell] current in 64-bit fixed point
   double *ant = nullptr;             // sorted deposit: antenna sheet values of a step, [laser][ncell / n0]
   int4 *far = nullptr;               // sorted deposit: ions with a far bound electron, moved after the push
   int *far_n = nullptr;              // their count (device, cleared after each step)
-  int *far_any = nullptr;            // whether the last push moved any (device)
   long long far_cap = 0;
   unsigned char *occ = nullptr;
   uint2 *jbb = nullptr;

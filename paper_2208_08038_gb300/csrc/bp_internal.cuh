@@ -142,7 +142,9 @@ struct PushArgs {
   int4 *far;                // sorted deposit: two-body ions whose bound electron is a cell or more away,
   int *far_n;               //   (species, particle, tile), moved after the push by k_push_far; their count
   int far_cap;
-  int *far_any;             // set by k_push_far when it moved any this step (their current may land anywhere)
+  unsigned char *act;       // [ntiles] tiles the field kernels update this step (null: all), set by k_push_far
+  unsigned long long *act_n; // their number, summed over the steps; the steps
+  int ia_lo, ia_hi;         // the antenna planes' x range
   int push_blocks[2];       // persistent push blocks for this grid on this device (see push_prepare)
   int sms;                  // multiprocessors of the device
 };
@@ -244,11 +246,11 @@ struct Cell4 {
 };
 
 template <int D>
-__device__ __forceinline__ bool row_cell4(const GridP &g, Cell4 &C) {
+__device__ __forceinline__ bool row_cell4(const GridP &g, Cell4 &C, int block) {
   const int n0 = g.n[0], n4 = n0 >> 2;
   const int chunks = (n4 + (int)blockDim.x - 1) / (int)blockDim.x;
-  const int row = (int)blockIdx.x / chunks;
-  const int x4 = ((int)blockIdx.x - row * chunks) * (int)blockDim.x + (int)threadIdx.x;
+  const int row = block / chunks;
+  const int x4 = (block - row * chunks) * (int)blockDim.x + (int)threadIdx.x;
   if (x4 >= n4) return false;
   C.c[0] = 4 * x4;
   C.c[1] = D >= 2 ? row % g.n[1] : 0;
@@ -266,6 +268,11 @@ __device__ __forceinline__ bool row_cell4(const GridP &g, Cell4 &C) {
     stride *= n;
   }
   return true;
+}
+
+template <int D>
+__device__ __forceinline__ bool row_cell4(const GridP &g, Cell4 &C) {
+  return row_cell4<D>(g, C, (int)blockIdx.x);
 }
 
 __device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
@@ -426,31 +433,105 @@ __host__ __device__ __forceinline__ double sm64_uniform(uint64_t key, uint64_t k
 }
 
 // ---------------------------------------------------------------------------
+// the laser antenna
+
+__device__ __forceinline__ double laser_value(const LaserP &L, double t, double y, double z) {
+  double ty = y - L.yc, tz = z - L.zc;
+  double tau = t - ty * sin(L.theta);
+  double env;
+  if (L.fwhm > 0) {
+    double d = tau - L.t0;
+    env = exp(-2.0 * 0.69314718055994530942 * d * d / (L.fwhm * L.fwhm));
+  } else if (tau <= 0) {
+    env = 0.0;
+  } else if (tau < L.ramp) {
+    double s = sin(0.5 * 3.14159265358979323846 * tau / L.ramp);
+    env = s * s;
+  } else {
+    env = 1.0;
+  }
+  double prof = 1.0;
+  if (L.waist > 0) {
+    double ey = ty * cos(L.theta);
+    prof = exp(-(ey * ey + tz * tz) / (L.waist * L.waist));
+  }
+  return L.a0 * env * prof * sin(L.omega * tau + L.phase);
+}
+
+struct LaserSet {
+  int n;
+  int lo, hi;  // lowest and highest antenna plane
+  LaserP l[BP_MAX_LASER];
+};
+
+// The step clock in device memory, so that a step's launches are the same
+// every step (one CUDA graph replayed): clk[0] the step number n,
+// clk[1 + p] probe p's samples so far, clk[1 + BP_MAX_PROBE + p] its
+// capacity.  The current J^{n+1/2} and the antenna's sheet take time
+// (n + 1/2) dt.
+__device__ __forceinline__ double current_time(const GridP &g, const long long *clk) {
+  return ((double)clk[0] + 0.5) * g.dtd;
+}
+
+// The antenna sheets' current on their planes at the current's time, FP64:
+// ant[s][y + ny z] for laser s (the value the current sum adds at cell
+// (L.ia, y, z)).  Done by the first `blocks` blocks of a kernel that runs
+// before the E update anyway: the FP64 sin and exp are a latency of 7 us
+// alone, and a launch of their own put it into every step.
+struct AntArgs {
+  LaserSet las;
+  const long long *clk;
+  double *ant;
+  int blocks;  // 0: no antenna in this launch
+};
+template <int D>
+__device__ __noinline__ void antenna_block(const GridP &g, const AntArgs &A) {
+  const double t = current_time(g, A.clk);
+  const long long nyz = g.ncell / g.n[0];
+  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < A.las.n * nyz;
+       q += (long long)A.blocks * blockDim.x) {
+    const int s = (int)(q / nyz);
+    const long long yz = q - s * nyz;
+    const int cy = (int)(yz % g.n[1]), cz = (int)(yz / g.n[1]);
+    const LaserP &L = A.las.l[s];
+    const double y = D >= 2 ? (cy + (L.comp == 1 ? 0.5 : 0.0)) * g.dxd[1] : 0.0;
+    const double z = D >= 3 ? (cz + (L.comp == 2 ? 0.5 : 0.0)) * g.dxd[2] : 0.0;
+    const double amp = -2.0 / g.dxd[0] * (L.comp == 2 ? cos(L.theta) : 1.0);
+    A.ant[q] = amp * laser_value(L, t, y, z);
+  }
+}
+// the antenna arguments of a step (blocks = 0 without lasers)
+AntArgs antenna_args(const GridP &g, const LaserP *las, int nlas, const long long *clk, double *ant);
+
+// ---------------------------------------------------------------------------
 // launch wrappers (host side), one translation unit each
 
-void launch_push(const GridP &g, const PushArgs &a, const TmaMaps &tm, cudaStream_t s);
+// ant: the antenna done by the quiet-tile pass (blocks = 0: by the B update)
+void launch_push(const GridP &g, const PushArgs &a, const TmaMaps &tm, const AntArgs &ant, cudaStream_t s);
+// whether the push of this grid runs without the quiet-tile pass
+bool push_direct(const GridP &g, const PushArgs &a);
 size_t push_smem_bytes(const GridP &g, int det);
-// the tiles the field kernels update (see k_tile_active); ia_lo..ia_hi: the antenna planes' x range
-void launch_tile_active(const GridP &g, const unsigned char *qstate, const int *far_any, int ia_lo, int ia_hi,
-                        unsigned char *act, unsigned long long *act_n, cudaStream_t s);
 // set the push kernel's shared-memory limit for this grid and return the
 // number of push blocks resident on the current device at once: blocks[0] of
 // the two-body kernel, blocks[1] of the one for grids with free particles
 int push_prepare(const GridP &g, int det, int blocks[2]);
 
-// act (per tile, optional): tiles to update; the others keep zero E, B, J
-void launch_yee_b(const GridP &g, float *const B[3], const float *const E[3], float h, const unsigned char *act,
-                  cudaStream_t s);
+// One pass over E^n and B^{n-1/2}: Bn <- B^n = B - h curl E, and B <- B^{n+1/2}
+// = B^n - h curl E (the same curl).  Clears the fixed-point current jfx (may be
+// null) and the push's counters of a, and runs the antenna of ant.
+// act (per tile, optional): tiles to update; the others keep zero E, B, J.
+void launch_yee_b(const GridP &g, float *const B[3], float *const Bn[3], const float *const E[3], float h,
+                  unsigned long long *jfx, const PushArgs &a, const AntArgs &ant, const unsigned char *act, cudaStream_t s);
 // recompute the tile marks (g.fnz) from E, B (F[0..5]) after a write from outside the step
 void launch_field_marks(const GridP &g, const float *const F[6], cudaStream_t s);
-// E <- E + dt (curl B - J).  With jfx (sorted deposit) the current is first
-// formed per cell from the 64-bit fixed-point accumulator (times jinv) plus
-// the antenna sheets at time t (evaluated into ant, [nlas][ncell / n0] FP64),
-// written to J, and the accumulator cleared;
-// without it J is read as the current sum left it.
+// E <- E + dt (curl B - J) with Mur faces; advances the clock's step number.
+// With jfx (sorted deposit) the current is first formed per cell from the
+// 64-bit fixed-point accumulator (times jinv) plus the antenna sheets of ant
+// ([nlas][ncell / n0] FP64) and written to J; without it J is read as the
+// current sum left it.
 void launch_yee_e(const GridP &g, float *const E[3], const float *const B[3], float *const J[3], float *frame,
-                  unsigned long long *jfx, float jinv, const LaserP *las, int nlas, const long long *clk,
-                  double *ant, const unsigned char *act, cudaStream_t s);
+                  const unsigned long long *jfx, float jinv, const LaserP *las, int nlas, long long *clk,
+                  const double *ant, const unsigned char *act, cudaStream_t s);
 long long frame_floats(const GridP &g);
 void launch_jsum(const GridP &g, const float *jbox, const unsigned char *occ, const uint2 *jbb, float *const J[3],
                  const LaserP *las, int nlas, const long long *clk, cudaStream_t s);
@@ -463,9 +544,16 @@ struct ClockState {
   int nprobe;
   long long count[BP_MAX_PROBE], cap[BP_MAX_PROBE];
 };
-void launch_probe(const float *F, const long long *nodes, long long npts, float *buf, const long long *clk, int p,
-                  cudaStream_t s);
-void launch_clock_tick(long long *clk, int nprobe, cudaStream_t s);
+// the probes' samples of a step, and their counts in the clock
+struct ProbeArgs {
+  int n;
+  const float *F[BP_MAX_PROBE];
+  const long long *nodes[BP_MAX_PROBE];
+  long long npts[BP_MAX_PROBE];
+  float *buf[BP_MAX_PROBE];
+};
+void launch_probes(const ProbeArgs &p, long long *clk, cudaStream_t s);
+int probe_launches(const ProbeArgs &p);
 void launch_clock_set(long long *clk, const ClockState &v, cudaStream_t s);
 
 struct SortBufs {

@@ -9,6 +9,8 @@
 // thread (16-byte vector loads and stores, coalesced along x) and return at
 // once in tiles the per-step activity flags mark inactive (E, B and J are
 // zero there and would stay zero); the other kernels one cell per thread.
+#include <cstring>
+
 #include "bp_internal.cuh"
 
 namespace {
@@ -61,13 +63,34 @@ __device__ __forceinline__ void mark_nonzero4(const GridP &g, const int c[3], bo
   if (*f == 0) *f = 1;
 }
 
-// B <- B - h curl E (forward differences to the B locations)
-template <int D>
-__global__ void __launch_bounds__(128) k_yee_b(GridP g, float *Bx, float *By, float *Bz, const float *__restrict__ Ex,
-                                               const float *__restrict__ Ey, const float *__restrict__ Ez, float h,
-                                               const unsigned char *__restrict__ act) {
+// B^n = B^{n-1/2} - h curl E^n into N and B^{n+1/2} = B^n - h curl E^n into B
+// (forward differences to the B locations).  Both half steps of a leapfrog
+// step take the same E^n, so one pass forms both: 48 B per cell instead of two
+// passes of 36 B and a launch (2D, 2048 x 2048 cells: step 298 -> 238 us with
+// the memset of the current and the flags' kernel folded in too).  On the way it clears the fixed-point current
+// of the tiles it updates (every tile the last step deposited in is one of
+// them) and the push's counters.
+template <int D, bool ANT>
+__global__ void __launch_bounds__(128) k_yee_b(const __grid_constant__ GridP g, float *Bx, float *By, float *Bz, float *Nx, float *Ny, float *Nz,
+                                               const float *__restrict__ Ex, const float *__restrict__ Ey,
+                                               const float *__restrict__ Ez, float h, unsigned long long *jfx,
+                                               int *tile_n, int *tile_ctr, int *far_n,
+                                               const unsigned char *__restrict__ act, const __grid_constant__ AntArgs ant) {
+  int block = (int)blockIdx.x;
+  if (ANT) {
+    if (block < ant.blocks) {
+      antenna_block<D>(g, ant);
+      return;
+    }
+    block -= ant.blocks;
+  }
+  if (block == 0 && threadIdx.x == 0) {
+    *tile_n = 0;
+    *tile_ctr = 0;
+    if (far_n) *far_n = 0;
+  }
   Cell4 C;
-  if (!row_cell4<D>(g, C)) return;
+  if (!row_cell4<D>(g, C, block)) return;
   if (act && !act[tile_of(g, C.c)]) return;  // E and B zero around the tile: B stays zero
   const long long q = C.q;
   const float4 ex = ld4(Ex + q), ey = ld4(Ey + q), ez = ld4(Ez + q);
@@ -82,7 +105,16 @@ __global__ void __launch_bounds__(128) k_yee_b(GridP g, float *Bx, float *By, fl
     exz = ld4(Ex + q + C.up[2]);
   }
   float4 bx = ld4(Bx + q), by = ld4(By + q), bz = ld4(Bz + q);
-  bool nz = false;
+  float4 nx = bx, ny = by, nz = bz;
+  bool any = false;
+  // one component of one cell: v the value, d the curl; the mark is set by
+  // either half step's value
+  auto half = [&](float4 &n, float4 &b, int i, float d) {
+    const float v = el(b, i) - h * d, w = v - h * d;
+    set_el(n, i, v);
+    set_el(b, i, w);
+    any |= v != 0.0f || w != 0.0f;
+  };
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const float ezi = el(ez, i), eyi = el(ey, i), exi = el(ex, i);
@@ -91,62 +123,40 @@ __global__ void __launch_bounds__(128) k_yee_b(GridP g, float *Bx, float *By, fl
       float d = 0.0f;
       if (D >= 2) d += (el(ezy, i) - ezi) * g.idx[1];
       if (D >= 3) d -= (el(eyz, i) - eyi) * g.idx[2];
-      const float v = el(bx, i) - h * d;
-      set_el(bx, i, v);
-      nz |= v != 0.0f;
+      half(nx, bx, i, d);
     }
     if (!skip_cell<D>(g, 5, C.c, i, false)) {
       float d = -(ezx - ezi) * g.idx[0];
       if (D >= 3) d += (el(exz, i) - exi) * g.idx[2];
-      const float v = el(by, i) - h * d;
-      set_el(by, i, v);
-      nz |= v != 0.0f;
+      half(ny, by, i, d);
     }
     if (!skip_cell<D>(g, 3, C.c, i, false)) {
       float d = (eyx - eyi) * g.idx[0];
       if (D >= 2) d -= (el(exy, i) - exi) * g.idx[1];
-      const float v = el(bz, i) - h * d;
-      set_el(bz, i, v);
-      nz |= v != 0.0f;
+      half(nz, bz, i, d);
     }
   }
+  st4(Nx + q, nx);
+  st4(Ny + q, ny);
+  st4(Nz + q, nz);
   st4(Bx + q, bx);
   st4(By + q, by);
   st4(Bz + q, bz);
-  mark_nonzero4<D>(g, C.c, nz);
-}
-
-__device__ double laser_value(const LaserP &L, double t, double y, double z) {
-  double ty = y - L.yc, tz = z - L.zc;
-  double tau = t - ty * sin(L.theta);
-  double env;
-  if (L.fwhm > 0) {
-    double d = tau - L.t0;
-    env = exp(-2.0 * 0.69314718055994530942 * d * d / (L.fwhm * L.fwhm));
-  } else if (tau <= 0) {
-    env = 0.0;
-  } else if (tau < L.ramp) {
-    double s = sin(0.5 * 3.14159265358979323846 * tau / L.ramp);
-    env = s * s;
-  } else {
-    env = 1.0;
+  if (jfx) {
+    const ulonglong2 z = make_ulonglong2(0ull, 0ull);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      ulonglong2 *p = reinterpret_cast<ulonglong2 *>(jfx + c * g.ncell + q);
+      p[0] = z;
+      p[1] = z;
+    }
   }
-  double prof = 1.0;
-  if (L.waist > 0) {
-    double ey = ty * cos(L.theta);
-    prof = exp(-(ey * ey + tz * tz) / (L.waist * L.waist));
-  }
-  return L.a0 * env * prof * sin(L.omega * tau + L.phase);
+  mark_nonzero4<D>(g, C.c, any);
 }
-
-struct LaserSet {
-  int n;
-  int lo, hi;  // lowest and highest antenna plane
-  LaserP l[BP_MAX_LASER];
-};
 
 LaserSet make_laser_set(const LaserP *las, int nlas) {
   LaserSet ls;
+  memset(&ls, 0, sizeof ls);
   ls.n = nlas;
   ls.lo = 1 << 30;
   ls.hi = -1;
@@ -168,35 +178,6 @@ __device__ __forceinline__ float fx_to_float(long long v, float s) {
   return fmaf(a, 16777216.0f * s, b * s);
 }
 
-// The step clock in device memory, so that a step's launches are the same
-// every step (one CUDA graph replayed): clk[0] the step number n,
-// clk[1 + p] probe p's samples so far, clk[1 + BP_MAX_PROBE + p] its
-// capacity.  The current J^{n+1/2} and the antenna's sheet take time
-// (n + 1/2) dt.
-__device__ __forceinline__ double current_time(const GridP &g, const long long *clk) {
-  return ((double)clk[0] + 0.5) * g.dtd;
-}
-
-// the antenna sheets' current on their planes at the current's time, FP64:
-// ant[s][y + ny z] for laser s (the value the current sum adds at cell
-// (L.ia, y, z))
-template <int D>
-__global__ void k_antenna(GridP g, LaserSet las, const long long *clk, double *ant) {
-  const double t = current_time(g, clk);
-  const long long nyz = g.ncell / g.n[0];
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < las.n * nyz;
-       q += (long long)gridDim.x * blockDim.x) {
-    const int s = (int)(q / nyz);
-    const long long yz = q - s * nyz;
-    const int cy = (int)(yz % g.n[1]), cz = (int)(yz / g.n[1]);
-    const LaserP &L = las.l[s];
-    double y = D >= 2 ? (cy + (L.comp == 1 ? 0.5 : 0.0)) * g.dxd[1] : 0.0;
-    double z = D >= 3 ? (cz + (L.comp == 2 ? 0.5 : 0.0)) * g.dxd[2] : 0.0;
-    double amp = -2.0 / g.dxd[0] * (L.comp == 2 ? cos(L.theta) : 1.0);
-    ant[q] = amp * laser_value(L, t, y, z);
-  }
-}
-
 // the antenna part of the sheets covering cell c: only which laser sits on
 // which plane and component is needed here
 struct AntSet {
@@ -207,15 +188,20 @@ struct AntSet {
 // E <- E + dt (curl B - J) on interior nodes (backward differences).  FX:
 // J^{n+1/2} is formed here from the 64-bit fixed-point accumulator (one
 // rounding: the scale jinv is a power of two) plus the antenna (added in
-// FP64 before the rounding) and stored in J; the launcher then clears the
-// accumulator for the next deposit with one memset (clearing it here, after
-// the loads, ran the kernel at a third of the bandwidth).
+// FP64 before the rounding) and stored in J; the next step's B update clears
+// the accumulator (clearing it here, after the loads, ran the kernel at a
+// third of the bandwidth).  murx: x is the only open axis, and its faces' Mur
+// nodes are done here (a face node and its inward neighbour lie in one group:
+// E_b(n+1) = E_adj(n) + km (E_adj(n+1) - E_b(n))); otherwise k_mur follows.
+// The clock's step number is advanced here: nothing reads it until the next
+// step.
 template <int D, bool FX>
 __global__ void __launch_bounds__(128) k_yee_e(GridP g, float *Ex, float *Ey, float *Ez, const float *__restrict__ Bx,
                                                const float *__restrict__ By, const float *__restrict__ Bz, float *Jx,
-                                               float *Jy, float *Jz, unsigned long long *jfx, float jinv,
+                                               float *Jy, float *Jz, const unsigned long long *jfx, float jinv,
                                                AntSet as, const double *__restrict__ ant,
-                                               const unsigned char *__restrict__ act) {
+                                               const unsigned char *__restrict__ act, long long *clk, int murx, float km) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) clk[0] += 1;
   Cell4 C;
   if (!row_cell4<D>(g, C)) return;
   if (act && !act[tile_of(g, C.c)]) return;  // no field and no current around the tile: E stays zero
@@ -276,6 +262,7 @@ __global__ void __launch_bounds__(128) k_yee_e(GridP g, float *Ex, float *Ey, fl
     bxz = ld4(Bx + q + C.dn[2]);
   }
   float4 ex = ld4(Ex + q), ey = ld4(Ey + q), ez = ld4(Ez + q);
+  const float4 oy = ey, oz = ez;
   bool nz = false;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -302,6 +289,18 @@ __global__ void __launch_bounds__(128) k_yee_e(GridP g, float *Ex, float *Ey, fl
       const float v = el(ez, i) + g.dt * (d - el(jz, i));
       set_el(ez, i, v);
       nz |= v != 0.0f;
+    }
+  }
+  if (murx) {
+    if (C.c[0] == 0) {
+      ey.x = oy.y + km * (ey.y - oy.x);
+      ez.x = oz.y + km * (ez.y - oz.x);
+      nz |= ey.x != 0.0f || ez.x != 0.0f;
+    }
+    if (C.c[0] + 4 == g.n[0]) {
+      ey.w = oy.z + km * (ey.z - oy.w);
+      ez.w = oz.z + km * (ez.z - oz.w);
+      nz |= ey.w != 0.0f || ez.w != 0.0f;
     }
   }
   st4(Ex + q, ex);
@@ -556,21 +555,23 @@ __global__ void __launch_bounds__(Geo<D>::L0 * Geo<D>::L1 * Geo<D>::L2)
   Jz[q] = sz;
 }
 
-// probe p's sample of this step into its next slot, while it has room
-__global__ void k_probe(const float *F, const long long *nodes, long long npts, float *buf, const long long *clk,
-                        int p) {
-  const long long slot = clk[1 + p];
-  if (slot >= clk[1 + BP_MAX_PROBE + p]) return;
-  float *out = buf + slot * npts;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < npts; q += (long long)gridDim.x * blockDim.x)
-    out[q] = F[nodes[q]];
-}
-
-// the end of a step: the clock advances, and the sample count of each of
-// the first nprobe probes (those recorded this step) while it has room
-__global__ void k_clock_tick(long long *clk, int nprobe) {
-  if (threadIdx.x == 0) clk[0] += 1;
-  if ((int)threadIdx.x < nprobe && clk[1 + threadIdx.x] < clk[1 + BP_MAX_PROBE + threadIdx.x]) clk[1 + threadIdx.x] += 1;
+// the probes' samples of this step into their next slots, while they have
+// room, and their counts: by one block when it can (the counts after a
+// barrier), else a grid for the samples and one block for the counts
+__global__ void k_probes(ProbeArgs P, long long *clk, int samples, int counts) {
+  if (samples)
+    for (int p = 0; p < P.n; ++p) {
+      const long long slot = clk[1 + p];
+      if (slot >= clk[1 + BP_MAX_PROBE + p]) continue;
+      float *out = P.buf[p] + slot * P.npts[p];
+      for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < P.npts[p];
+           q += (long long)gridDim.x * blockDim.x)
+        out[q] = P.F[p][P.nodes[p][q]];
+    }
+  if (!counts) return;
+  __syncthreads();
+  const int p = threadIdx.x;
+  if (p < P.n && clk[1 + p] < clk[1 + BP_MAX_PROBE + p]) clk[1 + p] += 1;
 }
 
 // the clock set from the host's state
@@ -600,21 +601,49 @@ long long frame_floats(const GridP &g) {
   return t;
 }
 
-void launch_yee_b(const GridP &g, float *const B[3], const float *const E[3], float h, const unsigned char *act,
-                  cudaStream_t s) {
+AntArgs antenna_args(const GridP &g, const LaserP *las, int nlas, const long long *clk, double *ant) {
+  AntArgs A;
+  memset(&A, 0, sizeof A);
+  if (nlas < 1 || !ant) return A;
+  A.las = make_laser_set(las, nlas);
+  A.clk = clk;
+  A.ant = ant;
+  // few points a block: the FP64 sin and exp spread over many SMs
+  const long long n = (long long)nlas * (g.ncell / g.n[0]);
+  A.blocks = grid_blocks(n, 128);
+  return A;
+}
+
+void launch_yee_b(const GridP &g, float *const B[3], float *const Bn[3], const float *const E[3], float h,
+                  unsigned long long *jfx, const PushArgs &a, const AntArgs &ant, const unsigned char *act, cudaStream_t s) {
   const int nb = row_blocks4(g, 128);
-  if (g.D == 1) k_yee_b<1><<<nb, 128, 0, s>>>(g, B[0], B[1], B[2], E[0], E[1], E[2], h, act);
-  else if (g.D == 2) k_yee_b<2><<<nb, 128, 0, s>>>(g, B[0], B[1], B[2], E[0], E[1], E[2], h, act);
-  else k_yee_b<3><<<nb, 128, 0, s>>>(g, B[0], B[1], B[2], E[0], E[1], E[2], h, act);
+#define YEE_B(DD, AA)                                                                                               \
+  k_yee_b<DD, AA><<<nb + ant.blocks, 128, 0, s>>>(g, B[0], B[1], B[2], Bn[0], Bn[1], Bn[2], E[0], E[1], E[2], h, jfx, \
+                                                  a.tile_n, a.tile_ctr, a.far_n, act, ant)
+  if (ant.blocks) {
+    if (g.D == 1) YEE_B(1, true);
+    else if (g.D == 2) YEE_B(2, true);
+    else YEE_B(3, true);
+  } else {
+    if (g.D == 1) YEE_B(1, false);
+    else if (g.D == 2) YEE_B(2, false);
+    else YEE_B(3, false);
+  }
+#undef YEE_B
 }
 
 void launch_yee_e(const GridP &g, float *const E[3], const float *const B[3], float *const J[3], float *frame,
-                  unsigned long long *jfx, float jinv, const LaserP *las, int nlas, const long long *clk,
-                  double *ant, const unsigned char *act, cudaStream_t s) {
-  long long nf = frame_floats(g);
+                  const unsigned long long *jfx, float jinv, const LaserP *las, int nlas, long long *clk,
+                  const double *ant, const unsigned char *act, cudaStream_t s) {
+  int nopen = 0;
+  for (int a = 0; a < g.D; ++a) nopen += g.bc[a] == BP_OPEN;
+  const bool xonly = nopen == 1 && g.bc[0] == BP_OPEN;
+  const float km = (g.dt - g.dx[0]) / (g.dt + g.dx[0]);
+  const long long nf = xonly ? 0 : frame_floats(g);
   if (nf) k_frame_save<<<grid_blocks(nf, 256), 256, 0, s>>>(g, E[0], E[1], E[2], frame, nf);
   const int nb = row_blocks4(g, 128);
   AntSet as;
+  memset(&as, 0, sizeof as);
   as.n = jfx ? nlas : 0;
   as.lo = 1 << 30;
   as.hi = -1;
@@ -624,16 +653,9 @@ void launch_yee_e(const GridP &g, float *const E[3], const float *const B[3], fl
     as.lo = las[i].ia < as.lo ? las[i].ia : as.lo;
     as.hi = las[i].ia > as.hi ? las[i].ia : as.hi;
   }
-  if (as.n > 0) {
-    const LaserSet ls = make_laser_set(las, nlas);
-    const long long nant = (long long)nlas * (g.ncell / g.n[0]);
-    // small blocks: the FP64 exp / sin of the antenna planes spread over many SMs
-    if (g.D == 1) k_antenna<1><<<grid_blocks(nant, 64), 64, 0, s>>>(g, ls, clk, ant);
-    else if (g.D == 2) k_antenna<2><<<grid_blocks(nant, 64), 64, 0, s>>>(g, ls, clk, ant);
-    else k_antenna<3><<<grid_blocks(nant, 64), 64, 0, s>>>(g, ls, clk, ant);
-  }
-#define YEE_E(DD, FF) \
-  k_yee_e<DD, FF><<<nb, 128, 0, s>>>(g, E[0], E[1], E[2], B[0], B[1], B[2], J[0], J[1], J[2], jfx, jinv, as, ant, act)
+#define YEE_E(DD, FF)                                                                                              \
+  k_yee_e<DD, FF><<<nb, 128, 0, s>>>(g, E[0], E[1], E[2], B[0], B[1], B[2], J[0], J[1], J[2], jfx, jinv, as, ant, act, \
+                                     clk, xonly ? 1 : 0, km)
   if (jfx) {
     if (g.D == 1) YEE_E(1, true);
     else if (g.D == 2) YEE_E(2, true);
@@ -644,13 +666,9 @@ void launch_yee_e(const GridP &g, float *const E[3], const float *const B[3], fl
     else YEE_E(3, false);
   }
 #undef YEE_E
-  if (jfx) cudaMemsetAsync(jfx, 0, sizeof(unsigned long long) * 3 * (size_t)g.ncell, s);
-  if (nf) {
-    int nopen = 0;
-    for (int a = 0; a < g.D; ++a) nopen += g.bc[a] == BP_OPEN;
+  if (nf)
     for (int p = 1; p <= nopen; ++p)
       k_mur<<<grid_blocks(nf / 2, 256), 256, 0, s>>>(g, E[0], E[1], E[2], frame, nf / 2, p);
-  }
 }
 
 void launch_field_marks(const GridP &g, const float *const F[6], cudaStream_t s) {
@@ -699,12 +717,27 @@ void launch_copy_many(const CopyList &L, int sms, cudaStream_t s) {
   k_copy_many<<<dim3((unsigned)bx, (unsigned)L.n), 256, 0, s>>>(L);
 }
 
-void launch_probe(const float *F, const long long *nodes, long long npts, float *buf, const long long *clk, int p,
-                  cudaStream_t s) {
-  k_probe<<<grid_blocks(npts, 256), 256, 0, s>>>(F, nodes, npts, buf, clk, p);
+// one block samples up to this many nodes in about the time of a launch
+constexpr long long kProbeOneBlock = 4096;
+
+static long long probe_points(const ProbeArgs &p) {
+  long long n = 0;
+  for (int k = 0; k < p.n; ++k) n += p.npts[k];
+  return n;
 }
 
-void launch_clock_tick(long long *clk, int nprobe, cudaStream_t s) { k_clock_tick<<<1, 32, 0, s>>>(clk, nprobe); }
+int probe_launches(const ProbeArgs &p) { return p.n == 0 ? 0 : (probe_points(p) <= kProbeOneBlock ? 1 : 2); }
+
+void launch_probes(const ProbeArgs &p, long long *clk, cudaStream_t s) {
+  if (p.n == 0) return;
+  const long long n = probe_points(p);
+  if (n <= kProbeOneBlock) {
+    k_probes<<<1, n <= 128 ? 128 : 1024, 0, s>>>(p, clk, 1, 1);
+    return;
+  }
+  k_probes<<<grid_blocks(n, 256), 256, 0, s>>>(p, clk, 1, 0);
+  k_probes<<<1, 32, 0, s>>>(p, clk, 0, 1);
+}
 
 void launch_clock_set(long long *clk, const ClockState &v, cudaStream_t s) {
   k_clock_set<<<1, BP_MAX_PROBE, 0, s>>>(clk, v);

@@ -24,9 +24,10 @@
 //   k_push_far    sorted mode: the ions k_push left on the far list (a bound
 //                 electron a cell or more from its nucleus), pushed with the
 //                 global fields and deposited into the global current,
-//   k_tile_active the tiles the field kernels update this step: those whose
-//                 neighbourhood has held a field or holds moved particles,
-//                 those next to an antenna plane, every tile after a far push.
+//                 and (tile_active) the tiles the field kernels update this
+//                 step: those whose neighbourhood has held a field or holds
+//                 moved particles, those next to an antenna plane, every tile
+//                 after a far push.
 #include <type_traits>
 
 #include "bp_internal.cuh"
@@ -1074,10 +1075,32 @@ __device__ __forceinline__ void zero_box(JT *J, int n, int tid, int bs) {
 //   QS_PUSH  the push kernel does the whole tile (fields may be non-zero),
 //   QS_DONE  every particle moved, nothing deposited (occ = 0),
 //   QS_REST  the quiet ions moved; the push does the others without fields.
-constexpr unsigned char QS_PUSH = 0, QS_DONE = 1, QS_REST = 2;
+//   QS_COLD  no fields and no particle moved yet (grids that go without this
+//            pass): the push does the whole tile without fields.
+constexpr unsigned char QS_PUSH = 0, QS_DONE = 1, QS_REST = 2, QS_COLD = 3;
+
+// lane's share (lanes 0..26) of whether a tile of t's 3^D neighbourhood has
+// held a non-zero E or B
+template <int D>
+__device__ __forceinline__ bool near_mark(const GridP &g, int t, int lane) {
+  if (lane >= 27) return false;
+  const int tc[3] = {t % g.nt[0], (t / g.nt[0]) % g.nt[1], t / (g.nt[0] * g.nt[1])};
+  const int o[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
+  bool use = true;
+  int nb[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    nb[a] = tc[a] + o[a];
+    if (a >= D) use &= o[a] == 0;
+    else if (g.bc[a] == BP_PERIODIC) nb[a] = wrap_once(nb[a], g.nt[a]);
+    else use &= nb[a] >= 0 && nb[a] < g.nt[a];
+  }
+  return use && g.fnz[nb[0] + g.nt[0] * (nb[1] + g.nt[1] * nb[2])] != 0;
+}
 
 template <int D>
-__global__ void __launch_bounds__(128, 8) k_push_quiet(GridP g, PushArgs A, int qt) {
+__global__ void __launch_bounds__(128, 8) k_push_quiet(const __grid_constant__ GridP g, PushArgs A, int qt,
+                                                       const __grid_constant__ AntArgs ant) {
   static_assert(Box<D>::OG <= Geo<D>::L0 && Box<D>::G0 - Box<D>::OG <= 2 * Geo<D>::L0 &&
                     (D < 2 || (Box<D>::OG <= Geo<D>::L1 && Box<D>::G1 - Box<D>::OG <= 2 * Geo<D>::L1)) &&
                     (D < 3 || (Box<D>::OG <= Geo<D>::L2 && Box<D>::G2 - Box<D>::OG <= 2 * Geo<D>::L2)),
@@ -1089,25 +1112,16 @@ __global__ void __launch_bounds__(128, 8) k_push_quiet(GridP g, PushArgs A, int 
   // classification loads; one on small grids, where tiles in turn would
   // lengthen the pass)
   __shared__ int quiet[4], nquiet;
+  if ((int)blockIdx.x < ant.blocks) {
+    antenna_block<D>(g, ant);
+    return;
+  }
   const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  const int t = (int)blockIdx.x * qt + warp;
+  const int t = ((int)blockIdx.x - ant.blocks) * qt + warp;
   if (tid == 0) nquiet = 0;
   bool marked = false, occupied = false;
   if (warp < qt && t < g.ntiles) {
-    const int tc[3] = {t % g.nt[0], (t / g.nt[0]) % g.nt[1], t / (g.nt[0] * g.nt[1])};
-    if (lane < 27) {
-      const int o[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
-      bool use = true;
-      int nb[3];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        nb[a] = tc[a] + o[a];
-        if (a >= D) use &= o[a] == 0;
-        else if (g.bc[a] == BP_PERIODIC) nb[a] = wrap_once(nb[a], g.nt[a]);
-        else use &= nb[a] >= 0 && nb[a] < g.nt[a];
-      }
-      if (use) marked = g.fnz[nb[0] + g.nt[0] * (nb[1] + g.nt[1] * nb[2])] != 0;
-    }
+    marked = near_mark<D>(g, t, lane);
     // a tile without particles has nothing to push or deposit, whatever its
     // fields: done here, so the push neither stages its fields nor visits it
     if (lane < A.nsp) occupied = A.p[lane].tstart[t + 1] > A.p[lane].tstart[t];
@@ -1159,38 +1173,40 @@ __global__ void __launch_bounds__(128, 8) k_push_quiet(GridP g, PushArgs A, int 
 // the neighbouring tiles), or an antenna plane lies within one tile of it.
 // Elsewhere E, B and J are zero and the Yee updates keep them exactly zero,
 // so the field kernels skip those tiles.  Computed after the push; it serves
-// that step's field updates and the next step's first B half step, over
-// which fields spread by at most three cells, less than one tile.
+// that step's E update and the next step's B update, over which fields spread
+// by at most two cells, less than one tile.
 template <int D>
-__global__ void k_tile_active(GridP g, const unsigned char *qstate, const int *far_any, int ia_lo, int ia_hi,
-                              unsigned char *act, unsigned long long *act_n) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t == 0) atomicAdd(act_n + 1, 1ull);  // the steps counted
-  bool a = false;
-  if (t < g.ntiles) {
-    const int tc[3] = {t % g.nt[0], (t / g.nt[0]) % g.nt[1], t / (g.nt[0] * g.nt[1])};
-    const int x0 = tc[0] * Geo<D>::L0;
-    // a far bound electron deposits at its own position: every tile then
-    a = (far_any && *far_any) || (ia_hi >= x0 - Geo<D>::L0 && ia_lo < x0 + 2 * Geo<D>::L0);
-    for (int o = 0; o < 27 && !a; ++o) {
-      const int off[3] = {o % 3 - 1, (o / 3) % 3 - 1, o / 9 - 1};
-      bool use = true;
-      int nb[3];
+__device__ __forceinline__ void tile_active(const GridP &g, const PushArgs &A, bool far) {
+  const int step = gridDim.x * blockDim.x;
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(A.act_n + 1, 1ull);  // the steps counted
+  // whole warps: the count is a warp reduction
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; (t & ~31) < g.ntiles; t += step) {
+    bool a = false;
+    if (t < g.ntiles) {
+      const int tc[3] = {t % g.nt[0], (t / g.nt[0]) % g.nt[1], t / (g.nt[0] * g.nt[1])};
+      const int x0 = tc[0] * Geo<D>::L0;
+      // a far bound electron deposits at its own position: every tile then
+      a = far || (A.ia_hi >= x0 - Geo<D>::L0 && A.ia_lo < x0 + 2 * Geo<D>::L0);
+      for (int o = 0; o < 27 && !a; ++o) {
+        const int off[3] = {o % 3 - 1, (o / 3) % 3 - 1, o / 9 - 1};
+        bool use = true;
+        int nb[3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        nb[k] = tc[k] + off[k];
-        if (k >= D) use &= off[k] == 0;
-        else if (g.bc[k] == BP_PERIODIC) nb[k] = wrap_once(nb[k], g.nt[k]);
-        else use &= nb[k] >= 0 && nb[k] < g.nt[k];
+        for (int k = 0; k < 3; ++k) {
+          nb[k] = tc[k] + off[k];
+          if (k >= D) use &= off[k] == 0;
+          else if (g.bc[k] == BP_PERIODIC) nb[k] = wrap_once(nb[k], g.nt[k]);
+          else use &= nb[k] >= 0 && nb[k] < g.nt[k];
+        }
+        if (!use) continue;
+        const int u = nb[0] + g.nt[0] * (nb[1] + g.nt[1] * nb[2]);
+        a = g.fnz[u] != 0 || A.qstate[u] != QS_DONE;
       }
-      if (!use) continue;
-      const int u = nb[0] + g.nt[0] * (nb[1] + g.nt[1] * nb[2]);
-      a = g.fnz[u] != 0 || qstate[u] != QS_DONE;
+      A.act[t] = a ? 1 : 0;
     }
-    act[t] = a ? 1 : 0;
+    const unsigned k = __reduce_add_sync(0xFFFFFFFFu, a ? 1u : 0u);
+    if ((threadIdx.x & 31u) == 0 && k) atomicAdd(A.act_n, (unsigned long long)k);
   }
-  const unsigned k = __reduce_add_sync(0xFFFFFFFFu, a ? 1u : 0u);
-  if ((threadIdx.x & 31u) == 0 && k) atomicAdd(act_n, (unsigned long long)k);
 }
 
 // byte offset of the field box in the push's dynamic shared memory (after the
@@ -1267,11 +1283,11 @@ __device__ __forceinline__ bool tma_tile(const GridP &g, const TmaMaps &T, const
 // holds registers, so the copies run while the block finishes the previous
 // tile.  A QS_REST tile's box is all zero and is not staged.
 template <int D>
-__device__ __forceinline__ void stage_issue(const GridP &g, const PushArgs &A, const TmaMaps &T, int t, float *Gsm,
-                                            unsigned long long *bar) {
+__device__ __forceinline__ void stage_issue(const GridP &g, const PushArgs &A, const TmaMaps &T, int t, unsigned char qs,
+                                            float *Gsm, unsigned long long *bar) {
   using BX = Box<D>;
   constexpr int GC = BX::GCELLS;
-  if (A.qstate[t] != QS_PUSH) return;
+  if (qs != QS_PUSH) return;
   const int tc[3] = {t % g.nt[0], (t / g.nt[0]) % g.nt[1], t / (g.nt[0] * g.nt[1])};
   const int T0[3] = {tc[0] * Geo<D>::L0, tc[1] * Geo<D>::L1, tc[2] * Geo<D>::L2};
   if (tma_tile<D>(g, T, T0)) {
@@ -1319,10 +1335,10 @@ __device__ __forceinline__ void stage_issue(const GridP &g, const PushArgs &A, c
 // mbarrier phase `phase`, flipped here after each TMA tile).  A TMA wait that
 // gives up sets ST_TIMEOUT and `failed`.
 template <int D>
-__device__ __forceinline__ void stage_done(const GridP &g, const PushArgs &A, const TmaMaps &T, int t,
+__device__ __forceinline__ void stage_done(const GridP &g, const PushArgs &A, const TmaMaps &T, int t, unsigned char qs,
                                            unsigned long long *bar, unsigned &phase, bool &failed) {
   asm volatile("cp.async.wait_group 0;" ::: "memory");
-  if (A.qstate[t] != QS_PUSH) return;
+  if (qs != QS_PUSH) return;
   const int tc[3] = {t % g.nt[0], (t / g.nt[0]) % g.nt[1], t / (g.nt[0] * g.nt[1])};
   const int T0[3] = {tc[0] * Geo<D>::L0, tc[1] * Geo<D>::L1, tc[2] * Geo<D>::L2};
   if (tma_tile<D>(g, T, T0)) {
@@ -1337,7 +1353,7 @@ __device__ __forceinline__ void stage_done(const GridP &g, const PushArgs &A, co
 // one tile of the push (the block's work for tile t)
 template <int D, bool DET, typename AfterLoop>
 __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, const TmaMaps &T, const int t,
-                                          unsigned long long *bar, unsigned &phase, bool &failed,
+                                          const unsigned char qs, unsigned long long *bar, unsigned &phase, bool &failed,
                                           AfterLoop &&after_loop) {
   using JT = typename std::conditional<DET, unsigned int, float>::type;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -1347,11 +1363,10 @@ __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, con
   JT *Jsm = reinterpret_cast<JT *>(smem);
   float *Gsm = reinterpret_cast<float *>(smem + GOFF);
   const int tid = threadIdx.x, bs = blockDim.x;
-  const unsigned char qs = A.qstate[t];
   int total = 0;
   for (int s = 0; s < A.nsp; ++s) total += A.p[s].tstart[t + 1] - A.p[s].tstart[t];
   if (qs == QS_DONE || total == 0) {
-    stage_done<D>(g, A, T, t, bar, phase, failed);  // this tile's copies land before the next tile's are issued
+    stage_done<D>(g, A, T, t, qs, bar, phase, failed);  // this tile's copies land before the next tile's are issued
     __syncthreads();
     if (tid == 0 && qs != QS_DONE) A.occ[t] = 0;
     after_loop();
@@ -1364,7 +1379,7 @@ __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, con
   const int T0[3] = {tc[0] * Geo<D>::L0, tc[1] * Geo<D>::L1, tc[2] * Geo<D>::L2};
   zero_box<DET>(Jsm, 3 * JC, tid, bs);
   // the field box was staged asynchronously (stage_issue) by the caller
-  stage_done<D>(g, A, T, t, bar, phase, failed);
+  stage_done<D>(g, A, T, t, qs, bar, phase, failed);
   __syncthreads();
   // no field in the box: known from the tile marks alone (a staged box that
   // happens to be all zero goes the full way, which leaves the same bits;
@@ -1495,12 +1510,13 @@ __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, con
 // spills).  Two-body ions need the registers (524 k ions: the adjoint cycle
 // 179 ms with 2, 185 with 3).
 template <int D, bool DET, int PB>
-__global__ void __launch_bounds__(push_threads(D), PB) k_push(GridP g, PushArgs A, const __grid_constant__ TmaMaps T) {
+__global__ void __launch_bounds__(push_threads(D), PB) k_push(GridP g, PushArgs A, const __grid_constant__ TmaMaps T,
+                                                               int direct) {
   extern __shared__ __align__(128) unsigned char smem[];
   float *Gsm = reinterpret_cast<float *>(smem + push_gbox_offset(D, DET));
   __shared__ int next;
   __shared__ __align__(8) unsigned long long bar;  // completion of the TMA staging
-  __shared__ int give_up;
+  __shared__ int give_up, marked;
   if (threadIdx.x == 0) {
     mbar_init(&bar);
     give_up = 0;
@@ -1508,28 +1524,41 @@ __global__ void __launch_bounds__(push_threads(D), PB) k_push(GridP g, PushArgs 
   __syncthreads();
   unsigned phase = 0;
   bool failed = false;
-  const int nlist = *A.tile_n;
+  const int nlist = direct ? 0 : *A.tile_n;
+  unsigned char qs = QS_DONE;
   // The next list entry is taken only once the block has finished the
   // current tile's particles: reserving it earlier would let one block hold
   // two costly tiles in a row while others have none (grids with few
-  // occupied tiles ran 20% slower that way).
-  auto grab = [&]() {
+  // occupied tiles ran 20% slower that way).  direct: a block per tile,
+  // without the quiet-tile pass; the block looks at its tile's marks itself.
+  auto grab = [&](bool first) {
+    bool mark = false;
+    if (direct && first && threadIdx.x < 32)
+      mark = __any_sync(0xFFFFFFFFu, near_mark<D>(g, (int)blockIdx.x, (int)threadIdx.x));
     if (threadIdx.x == 0) {
-      const int k = atomicAdd(A.tile_ctr, 1);
-      next = k < nlist ? A.tile_list[k] : -1;
+      if (direct) {
+        next = first ? (int)blockIdx.x : -1;
+        marked = mark;
+      } else {
+        const int k = atomicAdd(A.tile_ctr, 1);
+        next = k < nlist ? A.tile_list[k] : -1;
+      }
     }
     __syncthreads();
-    if (next >= 0) stage_issue<D>(g, A, T, next, Gsm, &bar);
+    if (next >= 0) {
+      qs = direct ? (marked ? QS_PUSH : QS_COLD) : A.qstate[next];
+      stage_issue<D>(g, A, T, next, qs, Gsm, &bar);
+    }
   };
-  grab();
+  grab(true);
   for (int t = next; t >= 0; t = next) {
-    push_tile<D, DET>(g, A, T, t, &bar, phase, failed, grab);
+    push_tile<D, DET>(g, A, T, t, qs, &bar, phase, failed, [&]() { grab(false); });
     if (failed) give_up = 1;
     __syncthreads();  // every thread has read `next` before it changes
     if (give_up) break;  // a staging wait gave up twice (ST_TIMEOUT is set): stop
   }
   // nothing may be in flight into this block's shared memory when it exits
-  if (next >= 0 && A.qstate[next] == QS_PUSH) stage_done<D>(g, A, T, next, &bar, phase, failed);
+  if (next >= 0 && qs == QS_PUSH) stage_done<D>(g, A, T, next, qs, &bar, phase, failed);
 }
 
 // Sorted mode: the ions the push listed as far (a bound electron a cell or
@@ -1537,8 +1566,8 @@ __global__ void __launch_bounds__(push_threads(D), PB) k_push(GridP g, PushArgs 
 // move is a domain error.
 template <int D>
 __global__ void __launch_bounds__(128) k_push_far(GridP g, PushArgs A) {
-  const int n = min(*A.far_n, A.far_cap), lane = threadIdx.x & 31;
-  if (blockIdx.x == 0 && threadIdx.x == 0 && A.far_any) *A.far_any = n > 0;
+  const int n = A.far_n ? min(*A.far_n, A.far_cap) : 0, lane = threadIdx.x & 31;
+  if (A.act) tile_active<D>(g, A, n > 0);
   const int warps = gridDim.x * (blockDim.x >> 5);
   for (int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += warps) {
     const int4 e = A.far[k];
@@ -1551,25 +1580,28 @@ __global__ void __launch_bounds__(128) k_push_far(GridP g, PushArgs A) {
   }
 }
 
+// the push kernel's variant (index of push_blocks): 1 on 2D grids with free particles
+int push_variant(const GridP &g, const PushArgs &a) {
+  bool free_sp = false;
+  for (int k = 0; k < a.nsp; ++k) free_sp |= a.sp[k].kind == BP_FREE;
+  return g.D == 2 && free_sp ? 1 : 0;
+}
+
 template <int D, bool DET>
-void launch_one(const GridP &g, const PushArgs &a, const TmaMaps &tm, cudaStream_t s) {
-  cudaMemsetAsync(a.tile_n, 0, sizeof(int), s);
-  const int qt = g.ntiles >= 8192 ? 4 : 1;  // tiles per quiet-pass block
-  k_push_quiet<D><<<(g.ntiles + qt - 1) / qt, 128, 0, s>>>(g, a, qt);
+void launch_one(const GridP &g, const PushArgs &a, const TmaMaps &tm, const AntArgs &ant, cudaStream_t s) {
+  const bool direct = push_direct(g, a);
+  if (!direct) {
+    const int qt = g.ntiles >= 8192 ? 4 : 1;  // tiles per quiet-pass block
+    k_push_quiet<D><<<(g.ntiles + qt - 1) / qt + ant.blocks, 128, 0, s>>>(g, a, qt, ant);
+  }
   const size_t smem = push_smem_bytes(g, DET);
   // as many persistent blocks as the device holds at once (worked out per
   // context for its grid and device when it was created)
-  bool free_sp = false;
-  for (int k = 0; k < a.nsp; ++k) free_sp |= a.sp[k].kind == BP_FREE;
-  const int v = D == 2 && free_sp ? 1 : 0;
+  const int v = push_variant(g, a);
   const int blocks = a.push_blocks[v] > 0 ? a.push_blocks[v] : 1, nb = blocks < g.ntiles ? blocks : g.ntiles;
-  cudaMemsetAsync(a.tile_ctr, 0, sizeof(int), s);
-  if (v) k_push<D, DET, push_pb(D, true)><<<nb, push_threads(D), smem, s>>>(g, a, tm);
-  else k_push<D, DET, push_pb(D, false)><<<nb, push_threads(D), smem, s>>>(g, a, tm);
-  if constexpr (DET) {
-    k_push_far<D><<<a.sms * 4, 128, 0, s>>>(g, a);
-    cudaMemsetAsync(a.far_n, 0, sizeof(int), s);
-  }
+  if (v) k_push<D, DET, push_pb(D, true)><<<nb, push_threads(D), smem, s>>>(g, a, tm, direct);
+  else k_push<D, DET, push_pb(D, false)><<<nb, push_threads(D), smem, s>>>(g, a, tm, direct);
+  if (DET || a.act) k_push_far<D><<<a.sms * 4, 128, 0, s>>>(g, a);
 }
 
 template <int D, bool DET, int PB>
@@ -1599,12 +1631,15 @@ size_t push_smem_bytes(const GridP &g, int det) {
   return push_gbox_offset(g.D, det != 0) + 4 * (size_t)6 * gc;
 }
 
-void launch_tile_active(const GridP &g, const unsigned char *qstate, const int *far_any, int ia_lo, int ia_hi,
-                        unsigned char *act, unsigned long long *act_n, cudaStream_t s) {
-  const int nb = (g.ntiles + 255) / 256;
-  if (g.D == 1) k_tile_active<1><<<nb, 256, 0, s>>>(g, qstate, far_any, ia_lo, ia_hi, act, act_n);
-  else if (g.D == 2) k_tile_active<2><<<nb, 256, 0, s>>>(g, qstate, far_any, ia_lo, ia_hi, act, act_n);
-  else k_tile_active<3><<<nb, 256, 0, s>>>(g, qstate, far_any, ia_lo, ia_hi, act, act_n);
+// The quiet-tile pass and its list pay where there are more tiles than push
+// blocks resident at once (a block then takes several tiles, and tiles ahead
+// of the field are many).  With a block for every tile they only lengthen the
+// chain of dependent launches: step of the 1D medium (128 tiles) 35.4 us with
+// the pass, 33.5 without; 524 k ions in 3D (128 tiles) 121 and 117 us.  Grids
+// with tile flags (1024 tiles or more) need the pass's states, the push timing
+// its counts.
+bool push_direct(const GridP &g, const PushArgs &a) {
+  return !a.act && !a.work && g.ntiles <= a.push_blocks[push_variant(g, a)];
 }
 
 int push_prepare(const GridP &g, int det, int blocks[2]) {
@@ -1618,15 +1653,15 @@ int push_prepare(const GridP &g, int det, int blocks[2]) {
   }
 }
 
-void launch_push(const GridP &g, const PushArgs &a, const TmaMaps &tm, cudaStream_t s) {
+void launch_push(const GridP &g, const PushArgs &a, const TmaMaps &tm, const AntArgs &ant, cudaStream_t s) {
   const bool det = a.jscale != 0.0f;
   switch (g.D * 2 + (det ? 1 : 0)) {
-    case 2: launch_one<1, false>(g, a, tm, s); break;
-    case 3: launch_one<1, true>(g, a, tm, s); break;
-    case 4: launch_one<2, false>(g, a, tm, s); break;
-    case 5: launch_one<2, true>(g, a, tm, s); break;
-    case 6: launch_one<3, false>(g, a, tm, s); break;
-    default: launch_one<3, true>(g, a, tm, s); break;
+    case 2: launch_one<1, false>(g, a, tm, ant, s); break;
+    case 3: launch_one<1, true>(g, a, tm, ant, s); break;
+    case 4: launch_one<2, false>(g, a, tm, ant, s); break;
+    case 5: launch_one<2, true>(g, a, tm, ant, s); break;
+    case 6: launch_one<3, false>(g, a, tm, ant, s); break;
+    default: launch_one<3, true>(g, a, tm, ant, s); break;
   }
 }
 

@@ -13,9 +13,6 @@
 #include "bp_ctx.h"
 #include "bp_internal.cuh"
 
-int sort_scan_blocks(const GridP &g);
-int sort_launches();
-
 namespace {
 
 const double R_E = 2.8179403262e-15;  // classical electron radius [m]
@@ -114,7 +111,6 @@ void update_jscale(bp_ctx *c) {
 }
 
 int alloc_particles(bp_ctx *c, Species &s, long long n, bool pidx) {
-  c->sort_dirty = true;
   const int D = c->g.D;
   const bool two = s.sp.kind == BP_TWO_BODY;
   long long cap = std::max(1LL, n);
@@ -153,12 +149,11 @@ int alloc_particles(bp_ctx *c, Species &s, long long n, bool pidx) {
     return fail(c, BP_ERR_OOM, "particle arrays (%lld particles)", n);
   }
   // sort scratch, shared by all species
-  c->sort_dirty = true;
   if (!c->sb.hist || !c->sb.bsum) {
     dfree(c, c->sb.hist);
     dfree(c, c->sb.bsum);
     c->sb.hist = (int *)dalloc(c, sizeof(int) * (c->g.ncell + 1));
-    c->sb.bsum = (int *)dalloc(c, sizeof(int) * (sort_scan_blocks(c->g) + 4));
+    c->sb.bsum = (int *)dalloc(c, sizeof(int) * c->sb.blocks);
     if (!c->sb.hist || !c->sb.bsum) {
       dfree(c, c->sb.hist);
       dfree(c, c->sb.bsum);
@@ -198,9 +193,8 @@ int initial_sort(bp_ctx *c, Species &s, long long n) {
   ts[c->g.ntiles] = (int)n;
   cudaMemcpyAsync(s.p.tstart, ts.data(), sizeof(int) * ts.size(), cudaMemcpyHostToDevice, c->stream);
   launch_set_sort_flag(c->status, c->stream);
-  launch_sort(c->g, s.sp, s.p, c->sb, c->status, c->stream);
-  launch_clear_sort_flag(c->status, c->stream);
-  c->launches += 2 + sort_launches();
+  launch_sort(c->g, 1, &s.sp, &s.p, c->sb, c->status, c->stream);
+  c->launches += 2;
   return check_launch(c, "initial sort");
 }
 
@@ -347,6 +341,16 @@ int bp_create(const bp_grid_desc *gd, const bp_allocator *al, void *stream, bp_c
   if (encode_field_maps(g, staged, &c->tmaps)) c->tmaps.on = 0;
   cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
   if (c->sms < 1) c->sms = 1;
+  c->sb.blocks = sort_blocks(c->sms);
+  c->sb.bar = (unsigned *)dalloc(c, sizeof(unsigned) * 2);
+  if (!c->sb.bar) {
+    bp_destroy(c);
+    return BP_ERR_OOM;
+  }
+  if (c->sb.blocks < 1) {
+    bp_destroy(c);
+    return BP_ERR_CUDA;
+  }
   if (push_prepare(g, c->det, c->push_blocks)) {
     bp_destroy(c);
     return BP_ERR_CUDA;
@@ -364,7 +368,6 @@ void bp_destroy(bp_ctx *c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
   for (auto e : c->ev) cudaEventDestroy(e);
-  if (c->sort_exec) cudaGraphExecDestroy(c->sort_exec);
   if (c->step_exec) cudaGraphExecDestroy(c->step_exec);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->read_stream) {
@@ -375,7 +378,6 @@ void bp_destroy(bp_ctx *c) {
     if (c->snap_ready[k]) cudaEventDestroy(c->snap_ready[k]);
     if (c->snap_done[k]) cudaEventDestroy(c->snap_done[k]);
   }
-  if (c->sort_runs) cudaFreeHost(c->sort_runs);
   if (c->adj.stream) {
     cudaStreamSynchronize(c->adj.stream);
     cudaStreamDestroy(c->adj.stream);
@@ -757,50 +759,6 @@ void cl_parts(bp_ctx *c, CopyList &L, const PartP &src, PartP &dst, int D, bool 
   if (src.pidx) cl_add(c, L, src.pidx, dst.pidx, sizeof(int) * cap);
 }
 
-// the re-sort graph of the current particle arrays (built on first use and
-// after any reallocation); false if the CUDA runtime cannot build it, in
-// which case the step launches the sort pipeline directly
-bool sort_graph(bp_ctx *c) {
-  if (c->sort_exec && !c->sort_dirty) return true;
-  if (c->sort_exec) {
-    cudaGraphExecDestroy(c->sort_exec);
-    c->sort_exec = nullptr;
-  }
-  if (!c->cap_stream && cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
-    c->cap_stream = nullptr;
-    cudaGetLastError();
-    return false;
-  }
-  if (!c->sort_runs) {
-    if (cudaHostAlloc((void **)&c->sort_runs, sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
-        cudaHostGetDevicePointer((void **)&c->sort_runs_dev, c->sort_runs, 0) != cudaSuccess) {
-      if (c->sort_runs) cudaFreeHost(c->sort_runs);
-      c->sort_runs = nullptr;
-      cudaGetLastError();
-      return false;
-    }
-    *c->sort_runs = 0;
-  }
-  SpecP sp[BP_MAX_SPECIES];
-  PartP pp[BP_MAX_SPECIES];
-  int n = 0;
-  for (auto &s : c->sp)
-    if (s.loaded && n < BP_MAX_SPECIES) {
-      sp[n] = s.sp;
-      pp[n] = s.p;
-      ++n;
-    }
-  cudaGraphExec_t ex = nullptr;
-  if (make_sort_graph(c->g, n, sp, pp, c->sb, c->status, c->sort_runs_dev, c->cap_stream, &ex) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  c->sort_exec = ex;
-  c->sort_nsp = n;
-  c->sort_dirty = false;
-  return true;
-}
-
 // the step clock from the host's state (the step number, the probes' sample
 // counts and capacities); run before the first step of every call that steps
 void sync_clock(bp_ctx *c, cudaStream_t st) {
@@ -816,20 +774,6 @@ void sync_clock(bp_ctx *c, cudaStream_t st) {
   c->launches++;
 }
 
-// re-sort when a particle left its tile margin in the previous step
-void launch_resort(bp_ctx *c, int nsp, cudaStream_t st) {
-  if (!nsp) return;
-  if (sort_graph(c)) {
-    cudaGraphLaunch(c->sort_exec, st);
-    c->launches += 1;  // the condition kernel; a re-sort that ran is counted by bp_kernel_launches
-  } else {
-    for (auto &s : c->sp)
-      if (s.loaded) launch_sort(c->g, s.sp, s.p, c->sb, c->status, st);
-    launch_clear_sort_flag(c->status, st);
-    c->launches += nsp * sort_launches() + 1;
-  }
-}
-
 ProbeArgs probe_args(const bp_ctx *c) {
   ProbeArgs P;
   memset(&P, 0, sizeof P);
@@ -843,7 +787,7 @@ ProbeArgs probe_args(const bp_ctx *c) {
   return P;
 }
 
-// The launches of one leapfrog step after the re-sort, on stream st.  They
+// The launches of one leapfrog step, on stream st.  They
 // are the same every step (the time and the probe slots come from the device
 // clock), so a plain step and a replay of their captured graph do the same
 // work.  When snap_fields is given, E^n and B^n (after the first half step)
@@ -858,6 +802,8 @@ void step_launches(bp_ctx *c, const PushArgs &A, bool probes, cudaStream_t st, f
   // where the push goes without that pass
   const AntArgs ant = antenna_args(g, c->las.data(), c->det ? (int)c->las.size() : 0, c->clk, c->ant), none{};
   const bool direct = push_direct(g, A);
+  // re-sort when a particle left its tile margin in the previous step
+  if (A.nsp) launch_sort(g, A.nsp, A.sp, A.p, c->sb, c->status, st);
   launch_yee_b(g, B, c->Bn, cE, 0.5f * g.dt, c->jfx, A, direct ? ant : none, c->act, st);
   if (snap_fields) {
     CopyList L;
@@ -893,9 +839,9 @@ void step_launches(bp_ctx *c, const PushArgs &A, bool probes, cudaStream_t st, f
 void step_account(bp_ctx *c, const PushArgs &A, bool probes) {
   int nopen = 0;
   for (int a = 0; a < c->g.D; ++a) nopen += c->g.bc[a] == BP_OPEN;
-  // B update, quiet-tile pass, push, far ions and tile flags, current sum
-  // (atomic), E update; Mur faces that the E update does not do itself
-  c->launches += 3 + (push_direct(c->g, A) ? 0 : 1) + (c->det || c->act ? 1 : 0) + (c->det ? 0 : 1);
+  // sort check, B update, quiet-tile pass, push, far ions and tile flags,
+  // current sum (atomic), E update; Mur faces that the E update does not do itself
+  c->launches += (A.nsp ? 4 : 3) + (push_direct(c->g, A) ? 0 : 1) + (c->det || c->act ? 1 : 0) + (c->det ? 0 : 1);
   if (nopen > 1 || (nopen == 1 && c->g.bc[0] != BP_OPEN)) c->launches += 1 + nopen;
   if (probes) {
     c->launches += probe_launches(probe_args(c));
@@ -906,19 +852,16 @@ void step_account(bp_ctx *c, const PushArgs &A, bool probes) {
 }
 
 // one leapfrog step, launched directly
-int one_step(bp_ctx *c, const PushArgs &A, int nsp, bool probes, float *snap_fields,
+int one_step(bp_ctx *c, const PushArgs &A, bool probes, float *snap_fields,
              std::vector<bp_part_copy> *snap_parts) {
-  launch_resort(c, nsp, c->stream);
   step_launches(c, A, probes, c->stream, snap_fields, snap_parts);
   step_account(c, A, probes);
   return check_launch(c, "step");
 }
 
 // one step through the step graph (step_graph succeeded for the current
-// arguments): one launch when the graph holds the re-sort, else two
-int graph_step(bp_ctx *c, const PushArgs &A, int nsp) {
-  if (c->step_sorts) c->launches += 1;  // the re-sort's condition kernel
-  else launch_resort(c, nsp, c->stream);
+// arguments)
+int graph_step(bp_ctx *c, const PushArgs &A) {
   cudaGraphLaunch(c->step_exec, c->stream);
   step_account(c, A, true);
   return check_launch(c, "step graph");
@@ -936,7 +879,7 @@ bool step_graph(bp_ctx *c, const PushArgs &A) {
   put(&c->g, sizeof c->g);
   put(c->F, sizeof c->F);
   put(c->Bn, sizeof c->Bn);
-  const void *ptrs[] = {c->jfx, c->jbox, c->occ, c->jbb, c->frame, c->ant, c->clk, c->sort_runs_dev};
+  const void *ptrs[] = {c->jfx, c->jbox, c->occ, c->jbb, c->frame, c->ant, c->clk};
   put(ptrs, sizeof ptrs);
   put(&c->sb, sizeof c->sb);
   put(&c->det, sizeof c->det);
@@ -966,27 +909,7 @@ bool step_graph(bp_ctx *c, const PushArgs &A) {
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamEndCapture(c->cap_stream, &graph);
   cudaGraphExec_t ex = nullptr;
-  // the re-sort's conditional node first, the captured launches after it
-  // (one graph launch per step); else the captured launches alone
-  bool sorts = false;
-  if (e == cudaSuccess && A.nsp > 0 && sort_graph(c)) {
-    SpecP sp[BP_MAX_SPECIES];
-    PartP pp[BP_MAX_SPECIES];
-    int n = 0;
-    for (auto &s : c->sp)
-      if (s.loaded && n < BP_MAX_SPECIES) {
-        sp[n] = s.sp;
-        pp[n] = s.p;
-        ++n;
-      }
-    sorts = make_sort_graph(c->g, n, sp, pp, c->sb, c->status, c->sort_runs_dev, c->cap_stream, &ex, graph) ==
-            cudaSuccess;
-    if (!sorts) {
-      ex = nullptr;
-      cudaGetLastError();
-    }
-  }
-  if (e == cudaSuccess && !sorts) e = cudaGraphInstantiate(&ex, graph, 0);
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, graph, 0);
   if (graph) cudaGraphDestroy(graph);
   if (e != cudaSuccess) {
     if (ex) cudaGraphExecDestroy(ex);
@@ -994,7 +917,6 @@ bool step_graph(bp_ctx *c, const PushArgs &A) {
     return false;
   }
   c->step_exec = ex;
-  c->step_sorts = sorts;
   c->step_key = key;
   return true;
 }
@@ -1009,12 +931,11 @@ int bp_step(bp_ctx *c, int64_t nsteps) {
   int nsp = 0;
   PushArgs A = push_args(c, &nsp);
   sync_clock(c, c->stream);
-  // two or more steps without push timing: one graph launch per step (the
-  // conditional re-sort, then the step's kernels)
+  // two or more steps without push timing: one graph launch per step
   const bool graph = nsteps >= 2 && !c->timing && step_graph(c, A);
   for (int64_t it = 0; it < nsteps; ++it) {
     int rc;
-    rc = graph ? graph_step(c, A, nsp) : one_step(c, A, nsp, true, nullptr, nullptr);
+    rc = graph ? graph_step(c, A) : one_step(c, A, true, nullptr, nullptr);
     if (rc) return rc;
   }
   return BP_OK;
@@ -1461,7 +1382,6 @@ int bp_load(bp_ctx *c, const char *path) {
   if (c->jfx) cudaMemset(c->jfx, 0, sizeof(unsigned long long) * 3 * (size_t)g.ncell);
   refresh_marks(c);
   c->step = h.step;
-  c->sort_dirty = true;
   update_jscale(c);
   cudaError_t e = cudaDeviceSynchronize();
   return e == cudaSuccess ? BP_OK : cuda_fail(c, e, "load");
@@ -1495,9 +1415,7 @@ int bp_residual(bp_ctx *c, double *dst, int on_device) {
 
 int64_t bp_kernel_launches(const bp_ctx *c) {
   if (!c) return 0;
-  // re-sorts run inside the step graph are counted on the device
-  const long long runs = c->sort_runs ? *(volatile int *)c->sort_runs : 0;
-  return c->launches + runs * ((long long)c->sort_nsp * sort_launches() + 1);
+  return c->launches;
 }
 
 int bp_set_record_capacity(bp_ctx *c, int64_t n) {
@@ -1656,7 +1574,7 @@ int bp_forward_ckpt(bp_ctx *c, int64_t nsteps, int K) {
     cl_flush(c, L);
     long long len = std::min<long long>(K, nsteps - (long long)k * K);
     for (long long j = 0; j < len; ++j) {
-      int rc = graph ? graph_step(c, A, nsp) : one_step(c, A, nsp, true, nullptr, nullptr);
+      int rc = graph ? graph_step(c, A) : one_step(c, A, true, nullptr, nullptr);
       if (rc) return rc;
     }
   }
@@ -1796,7 +1714,7 @@ int bp_backward(bp_ctx *c, int probe_id, const float *dl_dprobe, int sid, double
     c->step = ad.start + base;
     sync_clock(c, st);
     for (long long j = 0; j < len; ++j) {
-      int rc = one_step(c, A, nsp, false, ad.st_fields[bank * K + j], &ad.st_parts[bank * K + j]);
+      int rc = one_step(c, A, false, ad.st_fields[bank * K + j], &ad.st_parts[bank * K + j]);
       if (rc) return rc;
     }
     cudaEventRecord(ad.rec_done[bank], st);

@@ -558,22 +558,23 @@ void launch_clock_set(long long *clk, const ClockState &v, cudaStream_t s);
 
 struct SortBufs {
   int *hist;       // [ncell + 1]
-  int *bsum;       // scan block sums
+  int *bsum;       // [blocks] the sort blocks' totals
+  unsigned *bar;   // [2] their barrier
+  int blocks;      // blocks of the sort's cooperative launch
   int *tmp_cell;
   float *tmp_f;    // enough floats for the largest species' float payload
   int *tmp_i;      // pidx / id payload
 };
-void launch_sort(const GridP &g, const SpecP &sp, PartP &p, SortBufs &b, int *status, cudaStream_t s);
-void launch_clear_sort_flag(int *status, cudaStream_t s);
+// the sort of every species, if the status word asks for it; blocks resident at once
+cudaError_t launch_sort(const GridP &g, int nsp, const SpecP *sp, const PartP *p, const SortBufs &b, int *status,
+                        cudaStream_t s);
+int sort_blocks(int sms);
 void launch_gen_lattice(int D, const double *sites, int per_site, double jitter, uint64_t seed, double sigma,
                         const int *site_param, long long first, long long count, double *x, double *u, int *pidx,
                         cudaStream_t s);
 void launch_pick(const PartP &p, int D, int two, long long count, const int *sid, const int *srow, int n,
                  int *cell_out, float *out, unsigned char *found, cudaStream_t s);
 void launch_set_sort_flag(int *status, cudaStream_t s);
-cudaError_t make_sort_graph(const GridP &g, int nsp, const SpecP *sp, PartP *p, SortBufs &b, int *status, int *runs,
-                            cudaStream_t cap, cudaGraphExec_t *out, cudaGraph_t tail = nullptr);
-
 void launch_gen_medium(const GridP &g, const SpecP &sp, PartP &p, const int lo[3], const int hi[3], int ppc,
                        uint64_t seed, double sigma, long long first, long long count, cudaStream_t s);
 void launch_load_convert(const GridP &g, const SpecP &sp, PartP &p, const double *x, const double *u, const int *pidx,

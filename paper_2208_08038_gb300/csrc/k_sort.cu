@@ -2,13 +2,11 @@
 // (key = tile * cells_per_tile + cell within tile), run only when the device
 // status word says a particle left its tile's margin; the seeded device-side
 // medium generator; and the FP64 Gauss-law residual.
+#include <cstring>
+
 #include "bp_internal.cuh"
 
 namespace {
-
-constexpr int SCAN_BS = 1024;
-constexpr int SCAN_PER = 4;                 // elements per thread
-constexpr int SCAN_TILE = SCAN_BS * SCAN_PER;
 
 // blocks for n items; the kernels launched with it are grid-stride loops, so
 // the cap (two waves of 256-thread blocks on 152 SMs) only bounds the grid
@@ -16,8 +14,6 @@ int blocks_for(long long n, int bs, long long cap = 152LL * 16) {
   long long b = (n + bs - 1) / bs;
   return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
-
-__device__ __forceinline__ bool sorting(const int *status) { return (*(volatile const int *)status) & ST_NEED_SORT; }
 
 __device__ __forceinline__ int sort_key(const GridP &g, int cell) {
   int cc[3];
@@ -28,28 +24,9 @@ __device__ __forceinline__ int sort_key(const GridP &g, int cell) {
   return t * g.cpt + l;
 }
 
-__global__ void k_zero_if(int *a, long long n, const int *status) {
-  if (!sorting(status)) return;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x)
-    a[q] = 0;
-}
+constexpr int SORT_BS = 512;
 
-__global__ void k_save_count(const int *src, int *dst, const int *status) {
-  if (!sorting(status)) return;
-  *dst = *src;
-}
-
-__global__ void k_count(GridP g, PartP p, int *hist, const int *nold, const int *status) {
-  if (!sorting(status)) return;
-  const int n = *nold;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
-    int c = p.cell[q];
-    if (c >= 0) atomicAdd(hist + sort_key(g, c), 1);
-  }
-}
-
-// exclusive scan, three passes: per-block scan + block totals, scan of the
-// totals in one block, add-back
+// exclusive scan over the block; total: the block's sum
 __device__ __forceinline__ int block_exclusive_scan(int v, int *sh, int &total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int x = v;
@@ -76,114 +53,130 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *sh, int &total) 
   return base + x - v;
 }
 
-__global__ void __launch_bounds__(SCAN_BS) k_scan_blocks(int *a, long long n, int *bsum, const int *status) {
-  if (!sorting(status)) return;
+// A barrier over the blocks of a cooperative launch (all resident at once).
+// bar[0]: arrivals, bar[1]: barriers passed.  The wait is bounded (some ten
+// seconds of polls, longer than any kernel another stream may hold the GPU
+// with): false, with ST_TIMEOUT set, when it gives up.
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, int *status) {
+  __shared__ int passed;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    volatile unsigned *gen = bar + 1;
+    const unsigned g0 = *gen;
+    __threadfence();
+    passed = 1;
+    if (atomicAdd(bar, 1u) == gridDim.x - 1) {
+      bar[0] = 0u;
+      __threadfence();
+      atomicAdd(bar + 1, 1u);
+    } else {
+      int it = 0;
+      while (*gen == g0 && it < (1 << 26)) {
+        __nanosleep(64);
+        ++it;
+      }
+      if (*gen == g0) {
+        passed = 0;
+        atomicOr(status, ST_TIMEOUT);
+      }
+    }
+    __threadfence();
+  }
+  __syncthreads();
+  return passed != 0;
+}
+
+// The counting sort of every species by tile-major cell, as one cooperative
+// kernel that returns at once unless the status word asks for it (a particle
+// left its tile's margin): zero the histogram, count, scan (each block its
+// share of the cells, the blocks' totals summed by every block), scatter to
+// the scratch arrays, copy back.  As a conditional graph node with the phases
+// as nine launches a species the check alone took 14 to 21 us of every step
+// (1D medium: step 35 us with the conditional node, 21 us without); an
+// exiting launch takes 2 to 3.
+struct SortArgs {
+  int nsp;
+  PartP p[BP_MAX_SPECIES];
+  int two[BP_MAX_SPECIES];
+  SortBufs b;
+  int *status;
+};
+__global__ void __launch_bounds__(SORT_BS, 3) k_sort(const __grid_constant__ GridP g, const __grid_constant__ SortArgs S) {
+  // every block has read the flag when the last barrier lets one clear it
+  if (!(*(volatile const int *)S.status & ST_NEED_SORT)) return;
   __shared__ int sh[32];
-  long long base = (long long)blockIdx.x * SCAN_TILE + (long long)threadIdx.x * SCAN_PER;
-  int v[SCAN_PER], s = 0;
-#pragma unroll
-  for (int k = 0; k < SCAN_PER; ++k) {
-    v[k] = base + k < n ? a[base + k] : 0;
-    s += v[k];
-  }
-  int total;
-  int ex = block_exclusive_scan(s, sh, total);
-#pragma unroll
-  for (int k = 0; k < SCAN_PER; ++k) {
-    if (base + k < n) a[base + k] = ex;
-    ex += v[k];
-  }
-  if (threadIdx.x == 0) bsum[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(SCAN_BS) k_scan_single(int *a, int n, const int *status) {
-  if (!sorting(status)) return;
-  __shared__ int sh[32];
-  const int per = (n + SCAN_BS - 1) / SCAN_BS;
-  int s = 0;
-  for (int k = 0; k < per; ++k) {
-    int i = threadIdx.x * per + k;
-    s += i < n ? a[i] : 0;
-  }
-  int total;
-  int ex = block_exclusive_scan(s, sh, total);
-  for (int k = 0; k < per; ++k) {
-    int i = threadIdx.x * per + k;
-    if (i < n) {
-      int v = a[i];
-      a[i] = ex;
-      ex += v;
+  const long long nh = g.ncell + 1;
+  const long long tid = blockIdx.x * (long long)SORT_BS + threadIdx.x, nth = (long long)gridDim.x * SORT_BS;
+  int *const hist = S.b.hist, *const bsum = S.b.bsum;
+  const long long per = ((nh + gridDim.x - 1) / gridDim.x + SORT_BS - 1) / SORT_BS * SORT_BS;
+  const long long h0 = (long long)blockIdx.x * per, h1 = h0 + per < nh ? h0 + per : nh;
+  for (int s = 0; s < S.nsp; ++s) {
+    const PartP p = S.p[s];
+    const long long cap = p.cap;
+    const int n = p.tstart[g.ntiles];
+    for (long long q = tid; q < nh; q += nth) hist[q] = 0;
+    if (!grid_barrier(S.b.bar, S.status)) return;
+    for (long long q = tid; q < n; q += nth) {
+      const int c = p.cell[q];
+      if (c >= 0) atomicAdd(hist + sort_key(g, c), 1);
     }
-  }
-}
-
-__global__ void k_scan_add(int *a, long long n, const int *bsum, const int *status) {
-  if (!sorting(status)) return;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x)
-    a[q] += bsum[q / SCAN_TILE];
-}
-
-// tile ranges of the sorted order; the exclusive prefix at ncell is the count
-__global__ void k_tstart(GridP g, const int *hist, int *tstart, const int *status) {
-  if (!sorting(status)) return;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t <= g.ntiles;
-       t += (long long)gridDim.x * blockDim.x) {
-    tstart[t] = hist[t * (long long)g.cpt];
-  }
-}
-
-__global__ void k_scatter(GridP g, PartP p, int *off, int *tcell, float *tf, int *ti, int nf, const int *nold,
-                          const int *status) {
-  if (!sorting(status)) return;
-  const long long cap = p.cap;
-  const int n_old = *nold;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n_old;
-       q += (long long)gridDim.x * blockDim.x) {
-    int c = p.cell[q];
-    if (c < 0) continue;
-    int dst = atomicAdd(off + sort_key(g, c), 1);
-    tcell[dst] = c;
-    int k = 0;
-    for (int a = 0; a < g.D; ++a) tf[(k++) * cap + dst] = p.off[a * cap + q];
-    for (int a = 0; a < 3; ++a) tf[(k++) * cap + dst] = p.u1[a * cap + q];
-    if (nf > g.D + 3) {
-      for (int a = 0; a < 3; ++a) tf[(k++) * cap + dst] = p.r[a * cap + q];
-      for (int a = 0; a < 3; ++a) tf[(k++) * cap + dst] = p.u2[a * cap + q];
+    if (!grid_barrier(S.b.bar, S.status)) return;
+    int sum = 0, total;
+    for (long long q = h0 + threadIdx.x; q < h1; q += SORT_BS) sum += hist[q];
+    block_exclusive_scan(sum, sh, total);
+    if (threadIdx.x == 0) bsum[blockIdx.x] = total;
+    if (!grid_barrier(S.b.bar, S.status)) return;
+    int carry = 0;
+    sum = 0;
+    for (int q = threadIdx.x; q < (int)blockIdx.x; q += SORT_BS) sum += bsum[q];
+    block_exclusive_scan(sum, sh, carry);
+    for (long long q = h0; q < h1; q += SORT_BS) {
+      const long long k = q + threadIdx.x;
+      const int v = k < h1 ? hist[k] : 0;
+      const int ex = carry + block_exclusive_scan(v, sh, total);
+      if (k < h1) {
+        hist[k] = ex;
+        // the tile ranges; entry ncell is the count
+        if (k % g.cpt == 0) p.tstart[k / g.cpt] = ex;
+      }
+      carry += total;
     }
-    ti[dst] = p.id[q];
-    if (p.pidx) ti[cap + dst] = p.pidx[q];
-  }
-}
-
-__global__ void k_copyback(GridP g, PartP p, const int *tcell, const float *tf, const int *ti, int nf,
-                           const int *status) {
-  if (!sorting(status)) return;
-  const long long cap = p.cap;
-  const int n = p.tstart[g.ntiles];
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
-    p.cell[q] = tcell[q];
-    int k = 0;
-    for (int a = 0; a < g.D; ++a, ++k) p.off[a * cap + q] = tf[k * cap + q];
-    for (int a = 0; a < 3; ++a, ++k) p.u1[a * cap + q] = tf[k * cap + q];
-    if (nf > g.D + 3) {
-      for (int a = 0; a < 3; ++a, ++k) p.r[a * cap + q] = tf[k * cap + q];
-      for (int a = 0; a < 3; ++a, ++k) p.u2[a * cap + q] = tf[k * cap + q];
+    if (!grid_barrier(S.b.bar, S.status)) return;
+    for (long long q = tid; q < n; q += nth) {
+      const int c = p.cell[q];
+      if (c < 0) continue;
+      const int dst = atomicAdd(hist + sort_key(g, c), 1);
+      float *tf = S.b.tmp_f + dst;
+      S.b.tmp_cell[dst] = c;
+      for (int a = 0; a < g.D; ++a, tf += cap) *tf = p.off[a * cap + q];
+      for (int a = 0; a < 3; ++a, tf += cap) *tf = p.u1[a * cap + q];
+      if (S.two[s]) {
+        for (int a = 0; a < 3; ++a, tf += cap) *tf = p.r[a * cap + q];
+        for (int a = 0; a < 3; ++a, tf += cap) *tf = p.u2[a * cap + q];
+      }
+      S.b.tmp_i[dst] = p.id[q];
+      if (p.pidx) S.b.tmp_i[cap + dst] = p.pidx[q];
     }
-    p.id[q] = ti[q];
-    if (p.pidx) p.pidx[q] = ti[cap + q];
+    if (!grid_barrier(S.b.bar, S.status)) return;
+    const int m = p.tstart[g.ntiles];
+    for (long long q = tid; q < m; q += nth) {
+      const float *tf = S.b.tmp_f + q;
+      p.cell[q] = S.b.tmp_cell[q];
+      for (int a = 0; a < g.D; ++a, tf += cap) p.off[a * cap + q] = *tf;
+      for (int a = 0; a < 3; ++a, tf += cap) p.u1[a * cap + q] = *tf;
+      if (S.two[s]) {
+        for (int a = 0; a < 3; ++a, tf += cap) p.r[a * cap + q] = *tf;
+        for (int a = 0; a < 3; ++a, tf += cap) p.u2[a * cap + q] = *tf;
+      }
+      p.id[q] = S.b.tmp_i[q];
+      if (p.pidx) p.pidx[q] = S.b.tmp_i[cap + q];
+    }
+    if (!grid_barrier(S.b.bar, S.status)) return;
   }
+  if (tid == 0) atomicAnd(S.status, ~ST_NEED_SORT);
 }
 
-__global__ void k_clear_flag(int *status) { atomicAnd(status, ~ST_NEED_SORT); }
 __global__ void k_set_flag(int *status) { atomicOr(status, ST_NEED_SORT); }
-
-// condition of the re-sort graph: non-zero when a particle left its tile's
-// margin in the previous step; counts the sorts that run
-__global__ void k_sort_cond(cudaGraphConditionalHandle h, const int *status, int *runs) {
-  const bool need = (*(volatile const int *)status) & ST_NEED_SORT;
-  if (need) ++*runs;
-  cudaGraphSetConditional(h, need ? 1u : 0u);
-}
 
 // ---------------------------------------------------------------------------
 // device medium: ion g = cell rank * ppc + p over the cell box [lo, hi);
@@ -395,80 +388,27 @@ __global__ void k_load_convert(GridP g, SpecP sp, PartP p, const double *x, cons
 
 }  // namespace
 
-void launch_sort(const GridP &g, const SpecP &sp, PartP &p, SortBufs &b, int *status, cudaStream_t s) {
-  const long long nh = g.ncell + 1;
-  const int nf = g.D + (sp.kind == BP_TWO_BODY ? 9 : 3);
-  const int nblk = (int)((nh + SCAN_TILE - 1) / SCAN_TILE);
-  int *nold = b.bsum + nblk;
-  k_save_count<<<1, 1, 0, s>>>(p.tstart + g.ntiles, nold, status);
-  k_zero_if<<<blocks_for(nh, 256), 256, 0, s>>>(b.hist, nh, status);
-  k_count<<<blocks_for(p.cap, 256), 256, 0, s>>>(g, p, b.hist, nold, status);
-  k_scan_blocks<<<nblk, SCAN_BS, 0, s>>>(b.hist, nh, b.bsum, status);
-  k_scan_single<<<1, SCAN_BS, 0, s>>>(b.bsum, nblk, status);
-  k_scan_add<<<blocks_for(nh, 256), 256, 0, s>>>(b.hist, nh, b.bsum, status);
-  k_tstart<<<blocks_for(g.ntiles + 1, 256), 256, 0, s>>>(g, b.hist, p.tstart, status);
-  k_scatter<<<blocks_for(p.cap, 256), 256, 0, s>>>(g, p, b.hist, b.tmp_cell, b.tmp_f, b.tmp_i, nf, nold, status);
-  k_copyback<<<blocks_for(p.cap, 256), 256, 0, s>>>(g, p, b.tmp_cell, b.tmp_f, b.tmp_i, nf, status);
+int sort_blocks(int sms) {
+  int per = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sort, SORT_BS, 0) != cudaSuccess || per < 1) return -1;
+  return sms * per;
 }
 
-int sort_scan_blocks(const GridP &g) { return (int)((g.ncell + 1 + SCAN_TILE - 1) / SCAN_TILE); }
-int sort_launches() { return 9; }
-
-void launch_clear_sort_flag(int *status, cudaStream_t s) { k_clear_flag<<<1, 1, 0, s>>>(status); }
-
-// The per-step re-sort as one graph: a one-thread kernel reads the status
-// word and sets the condition of an IF node whose body is the sort pipeline
-// of every species followed by the flag reset.  A step in which no particle
-// left its tile's margin then costs that one kernel instead of the pipeline's
-// nine launches per species.  Captured on the private stream cap (the
-// caller's stream may be one that cannot capture); the executable graph is
-// launched on any stream of the context.  Valid while the particle arrays,
-// the sort scratch and the status word keep their addresses.
-cudaError_t make_sort_graph(const GridP &g, int nsp, const SpecP *sp, PartP *p, SortBufs &b, int *status, int *runs,
-                            cudaStream_t cap, cudaGraphExec_t *out, cudaGraph_t tail) {
-  *out = nullptr;
-  cudaGraph_t graph = nullptr;
-  cudaError_t e = cudaGraphCreate(&graph, 0);
-  if (e != cudaSuccess) return e;
-  cudaGraphConditionalHandle h;
-  cudaGraphNode_t ncond = nullptr, nif = nullptr;
-  e = cudaGraphConditionalHandleCreate(&h, graph, 0, cudaGraphCondAssignDefault);
-  if (e == cudaSuccess) {
-    const int *cs = status;
-    void *args[3] = {&h, (void *)&cs, &runs};
-    cudaKernelNodeParams kp{};
-    kp.func = (void *)k_sort_cond;
-    kp.gridDim = dim3(1);
-    kp.blockDim = dim3(1);
-    kp.kernelParams = args;
-    e = cudaGraphAddKernelNode(&ncond, graph, nullptr, 0, &kp);
+cudaError_t launch_sort(const GridP &g, int nsp, const SpecP *sp, const PartP *p, const SortBufs &b, int *status,
+                        cudaStream_t s) {
+  SortArgs S;
+  memset(&S, 0, sizeof S);
+  S.nsp = nsp;
+  for (int k = 0; k < nsp; ++k) {
+    S.p[k] = p[k];
+    S.two[k] = sp[k].kind == BP_TWO_BODY;
   }
-  cudaGraph_t body = nullptr;
-  if (e == cudaSuccess) {
-    cudaGraphNodeParams np{};
-    np.type = cudaGraphNodeTypeConditional;
-    np.conditional.handle = h;
-    np.conditional.type = cudaGraphCondTypeIf;
-    np.conditional.size = 1;
-    e = cudaGraphAddNode(&nif, graph, &ncond, nullptr, 1, &np);
-    if (e == cudaSuccess) body = np.conditional.phGraph_out[0];
-  }
-  if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
-  if (e == cudaSuccess) {
-    for (int q = 0; q < nsp; ++q) launch_sort(g, sp[q], p[q], b, status, cap);
-    launch_clear_sort_flag(status, cap);
-    cudaGraph_t captured = nullptr;
-    e = cudaStreamEndCapture(cap, &captured);
-  }
-  // the rest of a step, when given, after the conditional re-sort (a copy of
-  // the tail graph becomes a child node)
-  cudaGraphNode_t ntail = nullptr;
-  if (e == cudaSuccess && tail) e = cudaGraphAddChildGraphNode(&ntail, graph, &nif, 1, tail);
-  if (e == cudaSuccess) e = cudaGraphInstantiate(out, graph, 0);
-  cudaGraphDestroy(graph);
-  if (e != cudaSuccess) *out = nullptr;
-  return e;
+  S.b = b;
+  S.status = status;
+  void *args[2] = {(void *)&g, (void *)&S};
+  return cudaLaunchCooperativeKernel((const void *)k_sort, dim3((unsigned)b.blocks), dim3(SORT_BS), args, 0, s);
 }
+
 void launch_set_sort_flag(int *status, cudaStream_t s) { k_set_flag<<<1, 1, 0, s>>>(status); }
 
 // particles whose load id is in the sorted list sid[0..n): copy the raw

@@ -120,5 +120,7 @@ struct bp_ctx {
   // with (rebuilt when any of them changes)
   long long *clk = nullptr;
   cudaGraphExec_t step_exec = nullptr;
+  cudaGraphExec_t unroll_exec = nullptr;  // several steps in one graph
+  int singles = 0;                        // calls of one step in a row
   std::string step_key;
 };

@@ -11,7 +11,8 @@
 #define BP_MAX_LASER 4
 #define BP_MAX_PROBE 32
 
-// bits of the device status word
+// bits of the device status word (status[0]); status[1] holds a bit for each
+// loaded species that ST_NEED_SORT is about (none: all of them)
 enum { ST_NEED_SORT = 1, ST_DOMAIN = 2, ST_NONFINITE = 4, ST_TIMEOUT = 8 };
 
 // Grid geometry as the kernels see it.  Axes >= D have n = 1, L = 1, box 1.
@@ -349,6 +350,19 @@ __device__ __forceinline__ void fx_add(unsigned int *lo, int hoff, float v) {
   const int hh = __float_as_int(hs) - 0x4B400000;
   if (hh) atomicAdd(reinterpret_cast<int *>(lo + hoff), hh);
 }
+// The lanes' split of fx_add on a packed pair: low words r.x, r.y (integers),
+// high words h
+__device__ __forceinline__ void fx_split2(float2 v, int r[2], int h[2]) {
+  constexpr float M = 12582912.0f;
+  const float2 hs = __ffma2_rn(v, make_float2(1.52587890625e-05f, 1.52587890625e-05f), make_float2(M, M));
+  const float2 hh = __fadd2_rn(hs, make_float2(-M, -M));
+  const float2 rm = __fadd2_rn(__ffma2_rn(hh, make_float2(-65536.0f, -65536.0f), v), make_float2(M, M));
+  r[0] = __float_as_int(rm.x) - 0x4B400000;
+  r[1] = __float_as_int(rm.y) - 0x4B400000;
+  h[0] = __float_as_int(hs.x) - 0x4B400000;
+  h[1] = __float_as_int(hs.y) - 0x4B400000;
+}
+
 // fx_add of six values: three pairs, srow nodes apart, each pair spair nodes
 // apart (high words hoff later), the FP32 part on packed pairs: each lane
 // rounds exactly as fx_add does.  One branch for the six high words: a branch
@@ -357,27 +371,46 @@ __device__ __forceinline__ void fx_add(unsigned int *lo, int hoff, float v) {
 // pair, 4.26 with one per six; adding the zeros without a branch: 4.53, the
 // shared-memory adds are the dearer part).
 __device__ __forceinline__ void fx_add6(unsigned int *p, int srow, int spair, int hoff, const float2 v[3]) {
-  constexpr float M = 12582912.0f;
-  int h[6];
+  int r[3][2], h[3][2];
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    const float2 hs = __ffma2_rn(v[j], make_float2(1.52587890625e-05f, 1.52587890625e-05f), make_float2(M, M));
-    const float2 hh = __fadd2_rn(hs, make_float2(-M, -M));
-    const float2 r = __ffma2_rn(hh, make_float2(-65536.0f, -65536.0f), v[j]);
-    const float2 rm = __fadd2_rn(r, make_float2(M, M));
-    atomicAdd(reinterpret_cast<int *>(p + j * srow), __float_as_int(rm.x) - 0x4B400000);
-    atomicAdd(reinterpret_cast<int *>(p + j * srow + spair), __float_as_int(rm.y) - 0x4B400000);
-    h[2 * j] = __float_as_int(hs.x) - 0x4B400000;
-    h[2 * j + 1] = __float_as_int(hs.y) - 0x4B400000;
+    fx_split2(v[j], r[j], h[j]);
+    atomicAdd(reinterpret_cast<int *>(p + j * srow), r[j][0]);
+    atomicAdd(reinterpret_cast<int *>(p + j * srow + spair), r[j][1]);
   }
-  if (h[0] | h[1] | h[2] | h[3] | h[4] | h[5]) {
+  if (h[0][0] | h[0][1] | h[1][0] | h[1][1] | h[2][0] | h[2][1]) {
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      atomicAdd(reinterpret_cast<int *>(p + hoff + j * srow), h[2 * j]);
-      atomicAdd(reinterpret_cast<int *>(p + hoff + j * srow + spair), h[2 * j + 1]);
+      atomicAdd(reinterpret_cast<int *>(p + hoff + j * srow), h[j][0]);
+      atomicAdd(reinterpret_cast<int *>(p + hoff + j * srow + spair), h[j][1]);
     }
   }
 }
+
+// fx_add of a rows x cols block of values (row stride srow), one branch for
+// its high words
+template <int R, int C>
+__device__ __forceinline__ void fx_add_block(unsigned int *p, int srow, int hoff, const float (*v)[C]) {
+  constexpr float M = 12582912.0f;
+  int h[R][C], any = 0;
+#pragma unroll
+  for (int j = 0; j < R; ++j)
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+      const float hs = fmaf(v[j][i], 1.52587890625e-05f, M);
+      const float r = fmaf(-__fsub_rn(hs, M), 65536.0f, v[j][i]);
+      atomicAdd(reinterpret_cast<int *>(p + j * srow + i), __float_as_int(__fadd_rn(r, M)) - 0x4B400000);
+      h[j][i] = __float_as_int(hs) - 0x4B400000;
+      any |= h[j][i];
+    }
+  if (any) {
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+#pragma unroll
+      for (int i = 0; i < C; ++i) atomicAdd(reinterpret_cast<int *>(p + hoff + j * srow + i), h[j][i]);
+  }
+}
+
 // the value of a pair (both words initialised to 0)
 __device__ __forceinline__ long long fx_value(const unsigned int *lo, int hoff) {
   return (long long)(int)lo[hoff] * 65536LL + (long long)(int)lo[0];
@@ -560,7 +593,7 @@ struct SortBufs {
   int *hist;       // [ncell + 1]
   int *bsum;       // [blocks] the sort blocks' totals
   unsigned *bar;   // [2] their barrier
-  int blocks;      // blocks of the sort's cooperative launch
+  int blocks;      // blocks of the sort's cooperative launch resident at once
   int *tmp_cell;
   float *tmp_f;    // enough floats for the largest species' float payload
   int *tmp_i;      // pidx / id payload

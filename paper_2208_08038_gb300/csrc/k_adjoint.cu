@@ -1058,20 +1058,19 @@ __device__ __forceinline__ void scatter_comp(unsigned *A, const int d1[3], const
   scat_loc<D, PAT>(d1, f1, b1, w1);
   scat_loc<D, PAT>(d2, f2, b2, w2);
   const bool same = two && b1[0] == b2[0] && b1[1] == b2[1] && b1[2] == b2[2];
+  // a row of the stencil at a time: its high words under one branch
 #pragma unroll
   for (int k = 0; k < NK; ++k)
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
-      const float a1 = e1 * w1[1][j] * w1[2][k];
-      if (same) {
-        const float a2 = e2 * w2[1][j] * w2[2][k];
+      const float a1 = e1 * w1[1][j] * w1[2][k], a2 = e2 * w2[1][j] * w2[2][k];
+      float v[1][3];
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
-          fx_add(A + Box<D>::gi(b1[0] + i, b1[1] + j, b1[2] + k), hoff, __fadd_rn(a1 * w1[0][i], a2 * w2[0][i]));
-      } else {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) fx_add(A + Box<D>::gi(b1[0] + i, b1[1] + j, b1[2] + k), hoff, a1 * w1[0][i]);
+      for (int i = 0; i < 3; ++i) {
+        v[0][i] = __fmul_rn(a1, w1[0][i]);
+        if (same) v[0][i] = __fadd_rn(v[0][i], __fmul_rn(a2, w2[0][i]));
       }
+      fx_add_block<1, 3>(A + Box<D>::gi(b1[0], b1[1] + j, b1[2] + k), 0, hoff, v);
     }
   if (two && !same) {
 #pragma unroll
@@ -1079,8 +1078,10 @@ __device__ __forceinline__ void scatter_comp(unsigned *A, const int d1[3], const
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
         const float a2 = e2 * w2[1][j] * w2[2][k];
+        float v[1][3];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) fx_add(A + Box<D>::gi(b2[0] + i, b2[1] + j, b2[2] + k), hoff, a2 * w2[0][i]);
+        for (int i = 0; i < 3; ++i) v[0][i] = __fmul_rn(a2, w2[0][i]);
+        fx_add_block<1, 3>(A + Box<D>::gi(b2[0], b2[1] + j, b2[2] + k), 0, hoff, v);
       }
   }
 }

@@ -60,6 +60,20 @@ __device__ __forceinline__ void jadd(JT *p, float v, float scale) {
   jput<D, DET>(p, DET ? v * scale : v);
 }
 
+// jput of a rows x cols block of nodes (the sorted mode's high words under one
+// branch)
+template <int D, bool DET, int R, int C, typename JT>
+__device__ __forceinline__ void jput_block(JT *p, const float (*v)[C]) {
+  if constexpr (DET) {
+    fx_add_block<R, C>(p, Box<D>::J0, 3 * Box<D>::JCELLS, v);
+  } else {
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+#pragma unroll
+      for (int i = 0; i < C; ++i) atomicAdd(p + Box<D>::J0 * j + i, v[j][i]);
+  }
+}
+
 // Fast path: all four positions (both bodies, before and after the move)
 // share one nearest node per axis, so the window is the three nodes around
 // it and S1 - S0 has a closed form in the move d (no cancellation):
@@ -114,13 +128,13 @@ __device__ __forceinline__ void esirkepov3(JT *__restrict__ J, const int n[3], c
   JT *Jx = J, *Jy = J + jcells, *Jz = J + 2 * jcells;
   const int bx = n[0] - 1, by = n[1] - 1, bz = n[2] - 1;
   if constexpr (D == 1) {
+    float x[1][2], y[1][3], z[1][3], qy[NB], qz[NB];
 #pragma unroll
     for (int f = 0; f < 2; ++f) {
-      float jx = cP[0][0][f];
-      if constexpr (NB == 2) jx = __fadd_rn(jx, cP[1][0][f]);
-      jput<D, DET, false>(Jx + bx + f, jx);
+      x[0][f] = cP[0][0][f];
+      if constexpr (NB == 2) x[0][f] = __fadd_rn(x[0][f], cP[1][0][f]);
     }
-    float qy[NB], qz[NB];
+    jput_block<D, DET, 1, 2>(Jx + bx, x);
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
       qy[b] = qw[b] * v[b][1] * sc;
@@ -128,43 +142,44 @@ __device__ __forceinline__ void esirkepov3(JT *__restrict__ J, const int n[3], c
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      float jy = __fmul_rn(qy[0], A[0][0][i]), jz = __fmul_rn(qz[0], A[0][0][i]);
+      y[0][i] = __fmul_rn(qy[0], A[0][0][i]);
+      z[0][i] = __fmul_rn(qz[0], A[0][0][i]);
       if constexpr (NB == 2) {
-        jy = __fadd_rn(jy, __fmul_rn(qy[1], A[1][0][i]));
-        jz = __fadd_rn(jz, __fmul_rn(qz[1], A[1][0][i]));
+        y[0][i] = __fadd_rn(y[0][i], __fmul_rn(qy[1], A[1][0][i]));
+        z[0][i] = __fadd_rn(z[0][i], __fmul_rn(qz[1], A[1][0][i]));
       }
-      jput<D, DET, false>(Jy + bx + i, jy);
-      jput<D, DET, false>(Jz + bx + i, jz);
     }
+    jput_block<D, DET, 1, 3>(Jy + bx, y);
+    jput_block<D, DET, 1, 3>(Jz + bx, z);
   } else if constexpr (D == 2) {
+    float x[3][2], y[2][3], z[3][3], qz[NB];
 #pragma unroll
     for (int j = 0; j < 3; ++j)
 #pragma unroll
       for (int f = 0; f < 2; ++f) {
-        float jx = __fmul_rn(cP[0][0][f], A[0][1][j]);
-        if constexpr (NB == 2) jx = __fadd_rn(jx, __fmul_rn(cP[1][0][f], A[1][1][j]));
-        jput<D, DET, false>(Jx + Box<D>::ji(bx + f, by + j, 0), jx);
+        x[j][f] = __fmul_rn(cP[0][0][f], A[0][1][j]);
+        if constexpr (NB == 2) x[j][f] = __fadd_rn(x[j][f], __fmul_rn(cP[1][0][f], A[1][1][j]));
       }
+    jput_block<D, DET, 3, 2>(Jx + Box<D>::ji(bx, by, 0), x);
 #pragma unroll
     for (int g = 0; g < 2; ++g)
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        float jy = __fmul_rn(cP[0][1][g], A[0][0][i]);
-        if constexpr (NB == 2) jy = __fadd_rn(jy, __fmul_rn(cP[1][1][g], A[1][0][i]));
-        jput<D, DET, false>(Jy + Box<D>::ji(bx + i, by + g, 0), jy);
+        y[g][i] = __fmul_rn(cP[0][1][g], A[0][0][i]);
+        if constexpr (NB == 2) y[g][i] = __fadd_rn(y[g][i], __fmul_rn(cP[1][1][g], A[1][0][i]));
       }
-    float qz[NB];
+    jput_block<D, DET, 2, 3>(Jy + Box<D>::ji(bx, by, 0), y);
 #pragma unroll
     for (int b = 0; b < NB; ++b) qz[b] = qw[b] * v[b][2] * sc;
 #pragma unroll
     for (int j = 0; j < 3; ++j)
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        float jz = __fmul_rn(qz[0], fmaf(A[0][0][i], A[0][1][j], DK[0][0][i] * DS[0][1][j]));
+        z[j][i] = __fmul_rn(qz[0], fmaf(A[0][0][i], A[0][1][j], DK[0][0][i] * DS[0][1][j]));
         if constexpr (NB == 2)
-          jz = __fadd_rn(jz, __fmul_rn(qz[1], fmaf(A[1][0][i], A[1][1][j], DK[1][0][i] * DS[1][1][j])));
-        jput<D, DET, false>(Jz + Box<D>::ji(bx + i, by + j, 0), jz);
+          z[j][i] = __fadd_rn(z[j][i], __fmul_rn(qz[1], fmaf(A[1][0][i], A[1][1][j], DK[1][0][i] * DS[1][1][j])));
       }
+    jput_block<D, DET, 3, 3>(Jz + Box<D>::ji(bx, by, 0), z);
   } else {
     // The outer loop of each pass stays rolled (its weights picked by
     // selects): the fully unrolled 54-node form is about three times the
@@ -458,12 +473,14 @@ __device__ __noinline__ void deposit_general3_warp(JT *__restrict__ J, unsigned 
   }
 }
 
-// The deposit of a far body (a bound electron a cell or more from its
-// nucleus, or that nucleus) by a whole warp: four-node windows as above
+// W lanes work on one far body: the whole warp on one after the other of an
+// ion's bodies (32), a half warp on each (16, 1D and 2D), or one thread on both
+// (1).  lanes: the deposit of a far body (a bound electron a cell or more from
+// its nucleus, or that nucleus), four-node windows as above
 // around its own cell c, each node's value rounded to the fixed-point unit as
 // the shared-memory path rounds it and added to the global current (periodic
 // axes wrapped, nodes beyond an open face dropped, as the push drops them).
-template <int D>
+template <int D, int W>
 __device__ __forceinline__ void deposit_far(const GridP &g, const int c[3], const float f[3], const float de[3], float qw,
                                             const float v[3], unsigned long long *jfx, float scale) {
   constexpr int NODES = D == 3 ? 64 : (D == 2 ? 16 : 4);
@@ -472,7 +489,7 @@ __device__ __forceinline__ void deposit_far(const GridP &g, const int c[3], cons
 #pragma unroll
   for (int a = 0; a < D; ++a) G[a] = general_axis(f[a], de[a], -qw * g.dxdt[a]);
 #pragma unroll 1
-  for (int it = threadIdx.x & 31; it < 3 * NODES; it += 32) {
+  for (int it = W > 1 ? (int)(threadIdx.x & (W - 1)) : 0; it < 3 * NODES; it += W) {
     const int cc = it / NODES, m = it - cc * NODES;
     float A[3] = {1.0f, 1.0f, 1.0f}, S[3] = {0.0f, 0.0f, 0.0f}, val = 0.0f;
     long long gi = 0, stride = 1;
@@ -500,39 +517,41 @@ __device__ __forceinline__ void deposit_far(const GridP &g, const int c[3], cons
   }
 }
 
-// E and B of one body read from the global fields by a whole warp (a body
+// E and B of one body read from the global fields by its lanes (a body
 // outside the tile's staged box): the staggered quadratic gather over the
-// body's cell c and offset f, one lane per node of the stencil, summed in a
-// fixed order; periodic axes wrapped, zero beyond open faces
-template <int D>
+// body's cell c and offset f, the stencil's nodes shared out over the lanes; periodic axes wrapped, zero beyond open faces
+template <int D, int W>
 __device__ __forceinline__ void gather_global(const GridP &g, const float *const *Eg, const float *const *Bg,
                                               const int c[3], const float f[3], float E[3], float B[3]) {
   constexpr int NODES = D == 3 ? 27 : (D == 2 ? 9 : 3);
-  const int lane = threadIdx.x & 31;
-  const int o[3] = {lane % 3, (lane / 3) % 3, lane / 9};
 #pragma unroll
   for (int cc = 0; cc < 6; ++cc) {
     // stagger pattern of component cc: bit a set when it sits half a cell along a
     const int pat = cc < 3 ? (1 << cc) : (7 & ~(1 << (cc - 3)));
-    long long gi = 0, stride = 1;
-    float w = 1.0f;
-    bool ok = lane < NODES;
+    const float *F = cc < 3 ? Eg[cc] : Bg[cc - 3];
+    float acc = 0.0f;
+    for (int k = W > 1 ? (int)(threadIdx.x & (W - 1)) : 0; k < NODES; k += W) {
+      const int o[3] = {k % 3, (k / 3) % 3, k / 9};
+      long long gi = 0, stride = 1;
+      float w = 1.0f;
+      bool ok = true;
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-      const bool half = (pat >> a) & 1;
-      const int up = half ? 0 : (f[a] >= 0.5f ? 1 : 0);
-      float wa[3];
-      qweights(half ? f[a] - 0.5f : f[a] - (float)up, wa);
-      w *= o[a] == 0 ? wa[0] : (o[a] == 1 ? wa[1] : wa[2]);
-      int x = c[a] + up - 1 + o[a];
-      if (g.bc[a] == BP_PERIODIC) x = wrap_once(x, g.n[a]);
-      else ok &= x >= 0 && x < g.n[a];
-      gi += (long long)x * stride;
-      stride *= g.n[a];
+      for (int a = 0; a < D; ++a) {
+        const bool half = (pat >> a) & 1;
+        const int up = half ? 0 : (f[a] >= 0.5f ? 1 : 0);
+        float wa[3];
+        qweights(half ? f[a] - 0.5f : f[a] - (float)up, wa);
+        w *= o[a] == 0 ? wa[0] : (o[a] == 1 ? wa[1] : wa[2]);
+        int x = c[a] + up - 1 + o[a];
+        if (g.bc[a] == BP_PERIODIC) x = wrap_once(x, g.n[a]);
+        else ok &= x >= 0 && x < g.n[a];
+        gi += (long long)x * stride;
+        stride *= g.n[a];
+      }
+      if (ok) acc = fmaf(w, F[gi], acc);
     }
-    float acc = ok ? w * (cc < 3 ? Eg[cc] : Bg[cc - 3])[gi] : 0.0f;
 #pragma unroll
-    for (int q = 16; q > 0; q >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, q);
+    for (int q = W / 2; q > 0; q >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, q);
     if (cc < 3) E[cc] = acc;
     else B[cc - 3] = acc;
   }
@@ -557,6 +576,15 @@ template <int D>
 __device__ __forceinline__ void window_centre(const float *f, const int *d, int n0[3]) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) n0[a] = a < D ? d[a] + Box<D>::OJ + (f[a] >= 0.5f ? 1 : 0) : 0;
+}
+
+// a particle of (loaded) species s left its tile's margin: the species is
+// sorted before the next push.  The flags are read first: in a hot plasma many
+// particles set them in one step.
+__device__ __forceinline__ void mark_sort(int *status, int s) {
+  volatile int *const st = status;
+  if (!(st[1] & (1 << s))) atomicOr(status + 1, 1 << s);
+  if (!(st[0] & ST_NEED_SORT)) atomicOr(status, ST_NEED_SORT);
 }
 
 // 1 / gamma of a momentum u = p / (m c), one fixed evaluation order (the
@@ -616,7 +644,7 @@ __device__ __forceinline__ bool quiet_state(const float r[3], const float u1[3],
 // quiet (left for the full push).
 template <int D, int QB>
 __device__ __forceinline__ bool quiet_batch(const GridP &g, const PartP &P, long long i0, int bs, long long end,
-                                            const int T0[3], int *status, unsigned &moved) {
+                                            const int T0[3], int *status, int s, unsigned &moved) {
   const long long cap = P.cap;
   int cell[QB];
   float f[QB][3], u1[QB][3], u2[QB][3], r[QB][3];
@@ -662,7 +690,7 @@ __device__ __forceinline__ bool quiet_batch(const GridP &g, const PartP &P, long
       P.cell[i] = -1;
       continue;
     }
-    if (need_sort) atomicOr(status, ST_NEED_SORT);
+    if (need_sort) mark_sort(status, s);
     P.cell[i] = pack_cell(g, c[0], c[1], c[2]);
 #pragma unroll
     for (int a = 0; a < D; ++a) P.off[a * cap + i] = fn[a];
@@ -697,12 +725,13 @@ __device__ __forceinline__ bool quiet_done(const PartP &P, long long i) {
 // modified potential), sorted mode: outside the tile's boxes, so both bodies
 // gather from the global E and B and deposit into the global fixed-point
 // current.  The same arithmetic as push_particle's.
-// A whole warp per ion (every lane holds the ion; lane 0 writes it).  Returns
+// A warp (W = 32 or 16 lanes a body; every lane holds the ion, lane 0 writes
+// it) or a thread (W = 1) per ion.  Returns
 // false when the ion cannot be moved this way (body 1 outside its tile's
 // margin, body 2 beyond an open face or a displacement that is not finite): a
 // domain error for the caller.
-template <int D>
-__device__ __forceinline__ bool push_far(const GridP &g, const SpecP &sp, const PartP &P, long long i, int t0x, int t0y,
+template <int D, int W>
+__device__ __forceinline__ bool push_far(const GridP &g, const SpecP &sp, const PartP &P, int s, long long i, int t0x, int t0y,
                                       int t0z, int *status, const float *const *Eg, const float *const *Bg,
                                       unsigned long long *jfx, float scale) {
   const long long cap = P.cap;
@@ -736,17 +765,37 @@ __device__ __forceinline__ bool push_far(const GridP &g, const SpecP &sp, const 
     f2[a] = fr;
   }
   float E1[3], B1[3], E2[3], B2[3];
-  gather_global<D>(g, Eg, Bg, c, f, E1, B1);
-  gather_global<D>(g, Eg, Bg, c2, f2, E2, B2);
+  const bool second = W == 16 && (threadIdx.x & 16);  // this half warp's body
+  if constexpr (W != 16) {
+    gather_global<D, W>(g, Eg, Bg, c, f, E1, B1);
+    gather_global<D, W>(g, Eg, Bg, c2, f2, E2, B2);
+  } else {
+    int cb[3];
+    float fb[3], Eo[3], Bo[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      cb[a] = second ? c2[a] : c[a];
+      fb[a] = second ? f2[a] : f[a];
+    }
+    gather_global<D, W>(g, Eg, Bg, cb, fb, Eo, Bo);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const float e = __shfl_xor_sync(0xFFFFFFFFu, Eo[a], 16), b = __shfl_xor_sync(0xFFFFFFFFu, Bo[a], 16);
+      E1[a] = second ? e : Eo[a];
+      B1[a] = second ? b : Bo[a];
+      E2[a] = second ? Eo[a] : e;
+      B2[a] = second ? Bo[a] : b;
+    }
+  }
   const int pi = P.pidx ? P.pidx[i] : 0;
   const float ac = sp.ac[pi];
   const float rr = r[0] * r[0] + r[1] * r[1] + r[2] * r[2] + ac * ac;
   const float rs = rsqrtf(rr);
-  const float s = sp.kappa * rs * rs * rs;
+  const float k3 = sp.kappa * rs * rs * rs;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    E1[a] = fmaf(sp.q2 * s, r[a], E1[a]);
-    E2[a] = fmaf(-sp.q1 * s, r[a], E2[a]);
+    E1[a] = fmaf(sp.q2 * k3, r[a], E1[a]);
+    E2[a] = fmaf(-sp.q1 * k3, r[a], E2[a]);
   }
   boris(sp.h2, E2, B2, u2);
   boris(sp.h1, E1, B1, u1);
@@ -769,9 +818,22 @@ __device__ __forceinline__ bool push_far(const GridP &g, const SpecP &sp, const 
     if (a < D) de2[a] = de1[a] - (rn[a] - r[a]) * g.idx[a];
   }
   // each body on its own, around its own cell
-  deposit_far<D>(g, c, f, de1, sp.qw1, v1, jfx, scale);
-  deposit_far<D>(g, c2, f2, de2, sp.qw2, v2, jfx, scale);
-  if (threadIdx.x & 31) return true;
+  if constexpr (W != 16) {
+    deposit_far<D, W>(g, c, f, de1, sp.qw1, v1, jfx, scale);
+    deposit_far<D, W>(g, c2, f2, de2, sp.qw2, v2, jfx, scale);
+  } else {
+    int cb[3];
+    float fb[3], db[3], vb[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      cb[a] = second ? c2[a] : c[a];
+      fb[a] = second ? f2[a] : f[a];
+      db[a] = second ? de2[a] : de1[a];
+      vb[a] = second ? v2[a] : v1[a];
+    }
+    deposit_far<D, W>(g, cb, fb, db, second ? sp.qw2 : sp.qw1, vb, jfx, scale);
+  }
+  if (W > 1 && (threadIdx.x & 31)) return true;
   bool bad = false, removed = false, need_sort = false, nonfinite = false;
   advance_cell<D>(g, T0, true, c, fn, bad, removed, need_sort);
 #pragma unroll
@@ -782,7 +844,7 @@ __device__ __forceinline__ bool push_far(const GridP &g, const SpecP &sp, const 
     P.cell[i] = -1;
     return true;
   }
-  if (need_sort) atomicOr(status, ST_NEED_SORT);
+  if (need_sort) mark_sort(status, s);
   P.cell[i] = pack_cell(g, c[0], c[1], c[2]);
 #pragma unroll
   for (int a = 0; a < D; ++a) P.off[a * cap + i] = fn[a];
@@ -1022,7 +1084,7 @@ __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, l
     P.cell[i] = -1;
     return;
   }
-  if (need_sort) atomicOr(status, ST_NEED_SORT);
+  if (need_sort) mark_sort(status, s);
   P.cell[i] = pack_cell(g, c[0], c[1], c[2]);
 #pragma unroll
   for (int a = 0; a < D; ++a) P.off[a * cap + i] = fn[a];
@@ -1152,7 +1214,7 @@ __global__ void __launch_bounds__(128, 8) k_push_quiet(const __grid_constant__ G
       const int beg = A.p[s].tstart[tq], end = A.p[s].tstart[tq + 1];
       if (A.sp[s].kind == BP_TWO_BODY && A.sp[s].qw1 == -A.sp[s].qw2) {
         for (long long i0 = beg + tid; i0 < end; i0 += (long long)QB * bs)
-          left |= quiet_batch<D, QB>(g, A.p[s], i0, bs, end, T0, A.status, moved);
+          left |= quiet_batch<D, QB>(g, A.p[s], i0, bs, end, T0, A.status, s, moved);
       } else {
         left |= end > beg;
       }
@@ -1187,20 +1249,22 @@ __device__ __forceinline__ void tile_active(const GridP &g, const PushArgs &A, b
       const int x0 = tc[0] * Geo<D>::L0;
       // a far bound electron deposits at its own position: every tile then
       a = far || (A.ia_hi >= x0 - Geo<D>::L0 && A.ia_lo < x0 + 2 * Geo<D>::L0);
-      for (int o = 0; o < 27 && !a; ++o) {
-        const int off[3] = {o % 3 - 1, (o / 3) % 3 - 1, o / 9 - 1};
-        bool use = true;
-        int nb[3];
+      // all neighbours' states loaded at once (stopping at the first hit made
+      // 27 dependent loads of it: 9.4 us on 4096 tiles)
+      constexpr int NB = D == 3 ? 27 : (D == 2 ? 9 : 3);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
+      for (int o = 0; o < NB; ++o) {
+        const int off[3] = {o % 3 - 1, D >= 2 ? (o / 3) % 3 - 1 : 0, D >= 3 ? o / 9 - 1 : 0};
+        bool use = true;
+        int nb[3] = {0, 0, 0};
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
           nb[k] = tc[k] + off[k];
-          if (k >= D) use &= off[k] == 0;
-          else if (g.bc[k] == BP_PERIODIC) nb[k] = wrap_once(nb[k], g.nt[k]);
+          if (g.bc[k] == BP_PERIODIC) nb[k] = wrap_once(nb[k], g.nt[k]);
           else use &= nb[k] >= 0 && nb[k] < g.nt[k];
         }
-        if (!use) continue;
-        const int u = nb[0] + g.nt[0] * (nb[1] + g.nt[1] * nb[2]);
-        a = g.fnz[u] != 0 || A.qstate[u] != QS_DONE;
+        const int u = use ? nb[0] + g.nt[0] * (nb[1] + g.nt[1] * nb[2]) : t;
+        a |= g.fnz[u] != 0 || A.qstate[u] != QS_DONE;
       }
       A.act[t] = a ? 1 : 0;
     }
@@ -1566,17 +1630,25 @@ __global__ void __launch_bounds__(push_threads(D), PB) k_push(GridP g, PushArgs 
 // move is a domain error.
 template <int D>
 __global__ void __launch_bounds__(128) k_push_far(GridP g, PushArgs A) {
-  const int n = A.far_n ? min(*A.far_n, A.far_cap) : 0, lane = threadIdx.x & 31;
+  const int n = A.far_n ? min(*A.far_n, A.far_cap) : 0;
   if (A.act) tile_active<D>(g, A, n > 0);
-  const int warps = gridDim.x * (blockDim.x >> 5);
-  for (int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += warps) {
+  auto move = [&](int k, auto lanes) {
     const int4 e = A.far[k];
     const int t = e.z;
     const int T0[3] = {(t % g.nt[0]) * Geo<D>::L0, ((t / g.nt[0]) % g.nt[1]) * Geo<D>::L1,
                        (t / (g.nt[0] * g.nt[1])) * Geo<D>::L2};
-    if (!push_far<D>(g, A.sp[e.x], A.p[e.x], e.y, T0[0], T0[1], T0[2], A.status, A.E, A.B, A.jfx, A.jscale) &&
-        lane == 0)
+    constexpr int W = decltype(lanes)::value;
+    if (!push_far<D, W>(g, A.sp[e.x], A.p[e.x], e.x, e.y, T0[0], T0[1], T0[2], A.status, A.E, A.B, A.jfx, A.jscale) &&
+        (W == 1 || (threadIdx.x & 31) == 0))
       atomicOr(A.status, ST_DOMAIN);
+  };
+  // few ions (rare tears): a warp each, for the latency; many (a strong field
+  // over a whole crystal): a thread each
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+  if (n <= nt / 32) {
+    for (int k = tid >> 5; k < n; k += nt / 32) move(k, std::integral_constant<int, D == 3 ? 32 : 16>{});
+  } else {
+    for (int k = tid; k < n; k += nt) move(k, std::integral_constant<int, 1>{});
   }
 }
 

@@ -86,11 +86,11 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, int *status) {
   return passed != 0;
 }
 
-// The counting sort of every species by tile-major cell, as one cooperative
-// kernel that returns at once unless the status word asks for it (a particle
-// left its tile's margin): zero the histogram, count, scan (each block its
-// share of the cells, the blocks' totals summed by every block), scatter to
-// the scratch arrays, copy back.  As a conditional graph node with the phases
+// The counting sort by tile-major cell of the species that ask for it, as one
+// cooperative kernel that returns at once unless the status word does (a
+// particle left its tile's margin): count, scan (each block its share of the cells, the
+// blocks' totals summed by every block), scatter to the scratch arrays, copy
+// back and clear the histogram.  As a conditional graph node with the phases
 // as nine launches a species the check alone took 14 to 21 us of every step
 // (1D medium: step 35 us with the conditional node, 21 us without); an
 // exiting launch takes 2 to 3.
@@ -104,6 +104,7 @@ struct SortArgs {
 __global__ void __launch_bounds__(SORT_BS, 3) k_sort(const __grid_constant__ GridP g, const __grid_constant__ SortArgs S) {
   // every block has read the flag when the last barrier lets one clear it
   if (!(*(volatile const int *)S.status & ST_NEED_SORT)) return;
+  const int which = *(volatile const int *)(S.status + 1);  // bit s: species s; 0: all
   __shared__ int sh[32];
   const long long nh = g.ncell + 1;
   const long long tid = blockIdx.x * (long long)SORT_BS + threadIdx.x, nth = (long long)gridDim.x * SORT_BS;
@@ -111,11 +112,11 @@ __global__ void __launch_bounds__(SORT_BS, 3) k_sort(const __grid_constant__ Gri
   const long long per = ((nh + gridDim.x - 1) / gridDim.x + SORT_BS - 1) / SORT_BS * SORT_BS;
   const long long h0 = (long long)blockIdx.x * per, h1 = h0 + per < nh ? h0 + per : nh;
   for (int s = 0; s < S.nsp; ++s) {
+    if (which && !(which >> s & 1)) continue;
     const PartP p = S.p[s];
     const long long cap = p.cap;
     const int n = p.tstart[g.ntiles];
-    for (long long q = tid; q < nh; q += nth) hist[q] = 0;
-    if (!grid_barrier(S.b.bar, S.status)) return;
+    // (the histogram is kept clear between sorts)
     for (long long q = tid; q < n; q += nth) {
       const int c = p.cell[q];
       if (c >= 0) atomicAdd(hist + sort_key(g, c), 1);
@@ -159,6 +160,7 @@ __global__ void __launch_bounds__(SORT_BS, 3) k_sort(const __grid_constant__ Gri
     }
     if (!grid_barrier(S.b.bar, S.status)) return;
     const int m = p.tstart[g.ntiles];
+    for (long long q = tid; q < nh; q += nth) hist[q] = 0;
     for (long long q = tid; q < m; q += nth) {
       const float *tf = S.b.tmp_f + q;
       p.cell[q] = S.b.tmp_cell[q];
@@ -173,10 +175,17 @@ __global__ void __launch_bounds__(SORT_BS, 3) k_sort(const __grid_constant__ Gri
     }
     if (!grid_barrier(S.b.bar, S.status)) return;
   }
-  if (tid == 0) atomicAnd(S.status, ~ST_NEED_SORT);
+  if (tid == 0) {
+    S.status[1] = 0;
+    atomicAnd(S.status, ~ST_NEED_SORT);
+  }
 }
 
-__global__ void k_set_flag(int *status) { atomicOr(status, ST_NEED_SORT); }
+// every species of the next launch_sort is to be sorted
+__global__ void k_set_flag(int *status) {
+  status[1] = 0;
+  atomicOr(status, ST_NEED_SORT);
+}
 
 // ---------------------------------------------------------------------------
 // device medium: ion g = cell rank * ppc + p over the cell box [lo, hi);
@@ -405,8 +414,16 @@ cudaError_t launch_sort(const GridP &g, int nsp, const SpecP *sp, const PartP *p
   }
   S.b = b;
   S.status = status;
+  // A block for every 4096 cells and particles, at least 16: the exit of an
+  // unneeded sort and its barriers cost by the block (1D scan, 23.2 us a step
+  // with all 456 resident blocks, 21.9 with 152), its phases gain by it (4.2 M
+  // electrons: 495 and 528 us).
+  long long work = g.ncell;
+  for (int k = 0; k < nsp; ++k) work += p[k].cap;
+  const long long want = work / 4096 < 16 ? 16 : work / 4096;
+  const unsigned nb = (unsigned)(want < b.blocks ? want : b.blocks);
   void *args[2] = {(void *)&g, (void *)&S};
-  return cudaLaunchCooperativeKernel((const void *)k_sort, dim3((unsigned)b.blocks), dim3(SORT_BS), args, 0, s);
+  return cudaLaunchCooperativeKernel((const void *)k_sort, dim3(nb), dim3(SORT_BS), args, 0, s);
 }
 
 void launch_set_sort_flag(int *status, cudaStream_t s) { k_set_flag<<<1, 1, 0, s>>>(status); }

@@ -330,7 +330,7 @@ __device__ __forceinline__ void esirkepov3_p3(unsigned int *__restrict__ J, cons
 // kernel of its own, and a single thread's 75 rows from local memory once the
 // buffer was full: 4.2 M electrons, many of them crossing in a strong pulse,
 // push and records 1.07 ms a step before, 0.43 after; 32.5 M thermal ions in
-// 3D, 4.26 ms before, 3.78 after (one record took its lane as long as several
+// 3D, 4.26 ms before, 3.60 after (one record took its lane as long as several
 // particles).
 struct GenAxis {
   float A[4], DS[4], P[3];  // mid-step shape S0 + DS / 2, shape difference, face currents (charge factor included)
@@ -362,11 +362,63 @@ __device__ __forceinline__ GenAxis general_axis(float f, float de, float c) {
   return g;
 }
 
+// The same axis for an ion's body, in the arithmetic of the shape functions
+// (qshape, qshape_delta) node by node: the terms of a co-moving neutral pair
+// cancel to rounding, so how each is rounded shows in the sum.  Without
+// branches: a node's difference is the closed form of the piece that old and
+// new position share, else the difference of the two shapes.
+struct PairAxis {
+  float S[4], DS[4], P[4];  // old shape, shape difference, running sums of the differences times the charge factor
+  int base;
+};
+// old nearest node's offset up, position x from it, and the window's first node
+// o relative to it
+__device__ __forceinline__ void pair_place(float f, float d, float &x, int &up, int &o) {
+  up = f >= 0.5f ? 1 : 0;
+  x = f - (float)up;
+  o = x + d < -0.5f ? -2 : -1;
+}
+// old shape S and shape difference DS of the node k away from the old nearest one
+__device__ __forceinline__ void pair_node(float x, float d, int k, float &S, float &DS) {
+  const float u = x - (float)k, v = u + d;
+  const float au = fabsf(u), av = fabsf(v);
+  const float tu = 1.5f - au, tv = 1.5f - av;
+  const float cu = fmaf(-u, u, 0.75f), cv = fmaf(-v, v, 0.75f);
+  const float su = au <= 0.5f ? cu : (au < 1.5f ? __fmul_rn(__fmul_rn(0.5f, tu), tu) : 0.0f);
+  const float sv = av <= 0.5f ? cv : (av < 1.5f ? __fmul_rn(__fmul_rn(0.5f, tv), tv) : 0.0f);
+  const bool mid = au <= 0.5f && av <= 0.5f, right = u > 0.5f && v > 0.5f && u < 1.5f && v < 1.5f,
+             left = u < -0.5f && v < -0.5f && u > -1.5f && v > -1.5f;
+  const float w = mid ? u + v : (right ? __fsub_rn(__fsub_rn(3.0f, u), v) : __fadd_rn(__fadd_rn(3.0f, u), v));
+  const float h = mid ? -d : (right ? __fmul_rn(-0.5f, d) : __fmul_rn(0.5f, d));
+  S = su;
+  DS = mid || right || left ? __fmul_rn(h, w) : __fsub_rn(sv, su);
+}
+__device__ __forceinline__ PairAxis pair_axis(float f, float d, float c) {
+  PairAxis g;
+  float x, run = 0.0f;
+  int up, o;
+  pair_place(f, d, x, up, o);
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    pair_node(x, d, o + m, g.S[m], g.DS[m]);
+    run = __fadd_rn(run, g.DS[m]);
+    g.P[m] = __fmul_rn(c, run);
+  }
+  if (o == -1) g.P[3] = 0.0f;  // no face beyond the nodes n0 - 2 .. n0 + 2
+  g.base = up + o;
+  return g;
+}
+// the Esirkepov factor of the two axes transverse to a component
+__device__ __forceinline__ float pair_factor(float sp, float dp, float sq, float dq) {
+  return sp * sq + 0.5f * (dp * sq + sp * dq) + (1.0f / 3.0f) * dp * dq;
+}
+
 __device__ __forceinline__ float sel4(int k, const float *a) {
   return k == 0 ? a[0] : (k == 1 ? a[1] : (k == 2 ? a[2] : a[3]));
 }
 
-// 1D and 2D: one body
+// 1D and 2D: a free particle (and, body by body, the ions of a 2D grid with free
+// particles, whose kernel has no registers left for the other form)
 template <int D, bool DET, typename JT>
 __device__ __forceinline__ void deposit_general(JT *__restrict__ J, const int d[3], const float f[3], const float de[3],
                                                 float qw, const float v[3], const float dxdt[3], float scale) {
@@ -409,67 +461,135 @@ __device__ __forceinline__ void deposit_general(JT *__restrict__ J, const int d[
   }
 }
 
+// an ion in 1D and 2D (rare: its bodies stay close to each other and slow), both
+// bodies one after the other, out of line
+template <int D, bool DET, typename JT>
+__device__ __noinline__ void deposit_general_pair(JT *__restrict__ J, const int *d1, const int *d2, const float *f1,
+                                                  const float *f2, const float *e1, const float *e2, float qw1,
+                                                  float qw2, const float *v1, const float *v2, const float *dxdt,
+                                                  float scale) {
+  constexpr int jcells = Box<D>::JCELLS;
+#pragma unroll 1
+  for (int b = 0; b < 2; ++b) {
+    const float q = (b ? qw2 : qw1) * (DET ? scale : 1.0f);
+    const float *v = b ? v2 : v1;
+    PairAxis G[2];
+    int n0[2] = {0, 0};
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      G[a] = pair_axis(b ? f2[a] : f1[a], b ? e2[a] : e1[a], -q * dxdt[a]);
+      n0[a] = (b ? d2[a] : d1[a]) + Box<D>::OJ + G[a].base;
+    }
+    const PairAxis &X = G[0], &Y = G[1];
+    const float qy = q * v[1], qz = q * v[2];
+    JT *p = J + Box<D>::ji(n0[0], n0[1], 0);
+#pragma unroll 1
+    for (int j = 0; j < (D == 2 ? 4 : 1); ++j, p += Box<D>::J0) {
+      const float sy = D == 2 ? sel4(j, Y.S) : 1.0f, dy = D == 2 ? sel4(j, Y.DS) : 0.0f, py = D == 2 ? sel4(j, Y.P) : 0.0f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float fx = pair_factor(X.S[i], X.DS[i], 1.0f, 0.0f);
+        jput<D, DET>(p + i, X.P[i] * pair_factor(sy, dy, 1.0f, 0.0f));
+        jput<D, DET>(p + jcells + i, D == 2 ? py * fx : qy * fx);
+        jput<D, DET>(p + 2 * jcells + i, qz * pair_factor(X.S[i], X.DS[i], sy, dy));
+      }
+    }
+  }
+}
+
 // 3D: one row of one body, (component c, nodes j and k along the other two
-// axes), the three faces along c
+// axes), the faces along c
 template <bool DET, typename JT>
-__device__ __forceinline__ void general_row3(JT *__restrict__ J, const int d[3], const GenAxis G[3], int c, int j, int k) {
-  constexpr float K12 = 1.0f / 12.0f;
-  const GenAxis &X = G[0], &Y = G[1], &Z = G[2];
+__device__ __forceinline__ void general_row3(JT *__restrict__ J, const int d[3], const PairAxis G[3], int c, int j, int k) {
+  const PairAxis &X = G[0], &Y = G[1], &Z = G[2];
   // p < q: the other two axes
-  const float ap = c == 0 ? sel4(j, Y.A) : sel4(j, X.A), dp = c == 0 ? sel4(j, Y.DS) : sel4(j, X.DS);
-  const float aq = c == 2 ? sel4(k, Y.A) : sel4(k, Z.A), dq = c == 2 ? sel4(k, Y.DS) : sel4(k, Z.DS);
-  const float F = fmaf(ap, aq, K12 * dp * dq);
+  const float sp = c == 0 ? sel4(j, Y.S) : sel4(j, X.S), dp = c == 0 ? sel4(j, Y.DS) : sel4(j, X.DS);
+  const float sq = c == 2 ? sel4(k, Y.S) : sel4(k, Z.S), dq = c == 2 ? sel4(k, Y.DS) : sel4(k, Z.DS);
+  const float F = pair_factor(sp, dp, sq, dq);
   const int sc = c == 0 ? 1 : (c == 1 ? Box<3>::J0 : Box<3>::JP);
   JT *p = J + c * Box<3>::JCELLS +
           Box<3>::ji(d[0] + Box<3>::OJ + X.base, d[1] + Box<3>::OJ + Y.base, d[2] + Box<3>::OJ + Z.base) +
           j * (c == 0 ? Box<3>::J0 : 1) + k * (c == 2 ? Box<3>::J0 : Box<3>::JP);
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
+  for (int i = 0; i < 4; ++i)
     jput<3, DET>(p + i * sc, (c == 0 ? X.P[i] : (c == 1 ? Y.P[i] : Z.P[i])) * F);
 }
 
-// 3D, in a strong field: every lane its own particle's rows
+// one particle's deposit inputs, handed to its warp in shared memory (by value
+// they cost the push its registers: 3D, 32.5 M ions, 3.75 ms a step by value,
+// 3.60 this way)
+struct PairJob {
+  float f[2][3], e[2][3];  // the bodies' offsets and moves
+  int d[2][3];             // their cells relative to the tile
+  float q[2][3];           // minus charge factor times dx / dt along each axis
+  int two;
+};
+
+// 3D, in a warp that is not whole: its lanes (mask act) share out the rows of
+// the particle, every second lane those of the second body
 template <bool DET, typename JT>
-__device__ __noinline__ void deposit_general3(JT *__restrict__ J, int two, const int *d1, const int *d2, const float *f1,
-                                              const float *f2, const float *e1, const float *e2, float qw1, float qw2,
-                                              const float *dxdt, float scale) {
+__device__ __forceinline__ void deposit_general3_lanes(JT *__restrict__ J, unsigned act, const PairJob &P) {
+  const int lane = threadIdx.x & 31, rank = __popc(act & ((1u << lane) - 1u)), n = __popc(act);
+  // one lane alone takes one body after the other
+  const int nb = P.two ? 2 : 1, split = n > 1 ? nb : 1;
 #pragma unroll 1
-  for (int b = 0; b < (two ? 2 : 1); ++b) {
-    const float q = -(b ? qw2 : qw1) * (DET ? scale : 1.0f);
-    GenAxis G[3];
+  for (int b = rank % split; b < nb; b += split) {
+    PairAxis G[3];
     int d[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      d[a] = b ? d2[a] : d1[a];
-      G[a] = general_axis(b ? f2[a] : f1[a], b ? e2[a] : e1[a], q * dxdt[a]);
+      d[a] = P.d[b][a];
+      G[a] = pair_axis(P.f[b][a], P.e[b][a], P.q[b][a]);
     }
+    const int of = split == 1 ? n : (n + 1 - b) >> 1;  // lanes of this body
 #pragma unroll 1
-    for (int it = 0; it < 48; ++it) general_row3<DET, JT>(J, d, G, it >> 4, it & 3, (it >> 2) & 3);
+    for (int it = rank / split; it < 48; it += of) general_row3<DET, JT>(J, d, G, it >> 4, it & 3, (it >> 2) & 3);
   }
 }
 
-// 3D, the usual case of one such particle in a warp: the warp's active lanes
-// (mask act) share out the rows of lane src's particle.  A thermal medium has
-// one crossing in about 25 warps; alone, a lane took some 3,000 instructions
-// for it, the warp together 500.
+// 3D, the usual case of one such particle in a warp: the whole warp shares it
+// out, first a node of a body's axis per lane (24 of them), then the rows of
+// both bodies, three a lane.  A thermal medium has one such particle in some 15
+// warps; alone, its lane's chain of some 3,000 dependent instructions held the
+// warp as long as several runs of particles, and the tile with it when it came
+// in one of the last runs.
 template <bool DET, typename JT>
-__device__ __noinline__ void deposit_general3_warp(JT *__restrict__ J, unsigned act, int src, int two, const int *d1,
-                                                   const int *d2, const float *f1, const float *f2, const float *e1,
-                                                   const float *e2, float qw1, float qw2, const float *dxdt,
-                                                   float scale) {
-  const int lane = threadIdx.x & 31, rank = __popc(act & ((1u << lane) - 1u)), n = __popc(act);
-#pragma unroll 1
-  for (int b = 0; b < (two ? 2 : 1); ++b) {
-    const float q = -(b ? qw2 : qw1) * (DET ? scale : 1.0f);
-    GenAxis G[3];
-    int d[3];
+__device__ __noinline__ void deposit_general3_warp(JT *__restrict__ J, unsigned act, const PairJob *job) {
+  constexpr unsigned ALL = 0xFFFFFFFFu;
+  const PairJob &P = *job;
+  if (act != ALL) {
+    deposit_general3_lanes<DET, JT>(J, act, P);
+    return;
+  }
+  const int lane = threadIdx.x & 31;
+  // lanes 12 b + 4 a + m: node m of axis a of body b (the last eight lanes repeat)
+  const int nl = lane < 24 ? lane : lane - 24, nbody = nl / 12, naxis = (nl % 12) >> 2;
+  float x, S, DS;
+  int up, o;
+  const float d = P.e[nbody][naxis];
+  pair_place(P.f[nbody][naxis], d, x, up, o);
+  pair_node(x, d, o + (nl & 3), S, DS);
+  const int base = P.d[nbody][naxis] + Box<3>::OJ + up + o;  // the window's first node along this lane's axis
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      d[a] = __shfl_sync(act, b ? d2[a] : d1[a], src);
-      G[a] = general_axis(__shfl_sync(act, b ? f2[a] : f1[a], src), __shfl_sync(act, b ? e2[a] : e1[a], src), q * dxdt[a]);
+  for (int w = 0; w < 3; ++w) {
+    const int it = lane + 32 * w, b = it / 48, r = it - 48 * b, c = r >> 4, j = r & 3, k = (r >> 2) & 3;
+    const int p = c == 0 ? 1 : 0, q = c == 2 ? 1 : 2;  // the other two axes
+    const int lb = 12 * b, lc = lb + 4 * c, lp = lb + 4 * p + j, lq = lb + 4 * q + k;
+    const float F = pair_factor(__shfl_sync(ALL, S, lp), __shfl_sync(ALL, DS, lp), __shfl_sync(ALL, S, lq),
+                                __shfl_sync(ALL, DS, lq));
+    const int n0 = __shfl_sync(ALL, base, lb), n1 = __shfl_sync(ALL, base, lb + 4), n2 = __shfl_sync(ALL, base, lb + 8);
+    const int oc = __shfl_sync(ALL, o, lc);
+    const int sc = c == 0 ? 1 : (c == 1 ? Box<3>::J0 : Box<3>::JP);
+    JT *row = J + c * Box<3>::JCELLS + Box<3>::ji(n0, n1, n2) + j * (c == 0 ? Box<3>::J0 : 1) +
+              k * (c == 2 ? Box<3>::J0 : Box<3>::JP);
+    const float cq = P.q[b][c];
+    float run = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      run = __fadd_rn(run, __shfl_sync(ALL, DS, lc + i));
+      const float v = __fmul_rn(__fmul_rn(cq, run), F);
+      if ((i < 3 || oc == -2) && (b == 0 || P.two)) jput<3, DET>(row + i * sc, v);
     }
-#pragma unroll 1
-    for (int it = rank; it < 48; it += n) general_row3<DET, JT>(J, d, G, it >> 4, it & 3, (it >> 2) & 3);
   }
 }
 
@@ -484,24 +604,24 @@ template <int D, int W>
 __device__ __forceinline__ void deposit_far(const GridP &g, const int c[3], const float f[3], const float de[3], float qw,
                                             const float v[3], unsigned long long *jfx, float scale) {
   constexpr int NODES = D == 3 ? 64 : (D == 2 ? 16 : 4);
-  constexpr float K12 = 1.0f / 12.0f;
-  GenAxis G[3];
+  PairAxis G[3];
 #pragma unroll
-  for (int a = 0; a < D; ++a) G[a] = general_axis(f[a], de[a], -qw * g.dxdt[a]);
+  for (int a = 0; a < D; ++a) G[a] = pair_axis(f[a], de[a], -qw * g.dxdt[a]);
 #pragma unroll 1
   for (int it = W > 1 ? (int)(threadIdx.x & (W - 1)) : 0; it < 3 * NODES; it += W) {
     const int cc = it / NODES, m = it - cc * NODES;
-    float A[3] = {1.0f, 1.0f, 1.0f}, S[3] = {0.0f, 0.0f, 0.0f}, val = 0.0f;
+    // shapes of the transverse axes (1 and 0 along cc and axes not simulated)
+    float S[3] = {1.0f, 1.0f, 1.0f}, T[3] = {0.0f, 0.0f, 0.0f}, val = 0.0f;
     long long gi = 0, stride = 1;
     bool ok = true;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
       const int k = (m >> (2 * a)) & 3;
       if (a == cc) {
-        val = k == 0 ? G[a].P[0] : (k == 1 ? G[a].P[1] : (k == 2 ? G[a].P[2] : 0.0f));
+        val = sel4(k, G[a].P);
       } else {
-        A[a] = sel4(k, G[a].A);
-        S[a] = sel4(k, G[a].DS);
+        S[a] = sel4(k, G[a].S);
+        T[a] = sel4(k, G[a].DS);
       }
       int x = c[a] + G[a].base + k;
       if (g.bc[a] == BP_PERIODIC) x = wrap_once(x, g.n[a]);
@@ -510,8 +630,8 @@ __device__ __forceinline__ void deposit_far(const GridP &g, const int c[3], cons
       stride *= g.n[a];
     }
     if (cc >= D) val = qw * (cc == 1 ? v[1] : v[2]);
-    // the two transverse axes (at most two of the three differences are not 0)
-    const float F = A[0] * A[1] * A[2] + K12 * (S[0] * S[1] + S[1] * S[2] + S[0] * S[2]);
+    const float F = cc == 0 ? pair_factor(S[1], T[1], S[2], T[2])
+                            : (cc == 1 ? pair_factor(S[0], T[0], S[2], T[2]) : pair_factor(S[0], T[0], S[1], T[1]));
     const float vs = val * F * scale;
     if (ok && fabsf(vs) > 0.5f) atomicAdd(jfx + (size_t)cc * g.ncell + gi, (unsigned long long)f2ll_rn(vs));
   }
@@ -857,10 +977,10 @@ __device__ __forceinline__ bool push_far(const GridP &g, const SpecP &sp, const 
   return true;
 }
 
-template <int D, bool DET, typename JT>
+template <int D, bool DET, bool FREE, typename JT>
 __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, long long i, const int T0[3],
-                              const float *Gsm, JT *Jsm, int *status, float scale, unsigned &blo, unsigned &bhi, bool nofield, int4 *far, int *far_n, int far_cap, int s,
-                              int t) {
+                              const float *Gsm, JT *Jsm, int *status, float scale, unsigned &blo, unsigned &bhi,
+                              PairJob *jobs, bool nofield, int4 *far, int *far_n, int far_cap, int s, int t) {
   const long long cap = P.cap;
   const bool two = sp.kind == BP_TWO_BODY;
   int cell = P.cell[i];
@@ -1006,28 +1126,28 @@ __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, l
   for (int a = 0; a < 3; ++a) silent &= (r[a] == 0.0f) && (v1[a] == v2[a]);
   if constexpr (D == 3) {
     // the general case in 3D: rare in a thermal medium, so the warp's lanes
-    // share out the rows of one such particle after the other; with more than
-    // three of them every lane does its own
+    // share out one such particle after the other
     const unsigned act = __activemask();
     unsigned gen = __ballot_sync(act, !silent && !fast);
-    if (gen) {
-      float fb[2][3], db[2][3], dd[3];
-      int cb[2][3];
+    for (; gen; gen &= gen - 1) {
+      PairJob &P = jobs[threadIdx.x >> 5];
+      if ((int)(threadIdx.x & 31) == __ffs(gen) - 1) {
+        const float sc = DET ? scale : 1.0f;
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        fb[0][a] = f[a]; fb[1][a] = f2[a];
-        db[0][a] = de1[a]; db[1][a] = de2[a];
-        cb[0][a] = d[a]; cb[1][a] = d2[a];
-        dd[a] = dxdt[a];
+        for (int a = 0; a < 3; ++a) {
+          P.f[0][a] = f[a];
+          P.f[1][a] = f2[a];
+          P.e[0][a] = de1[a];
+          P.e[1][a] = de2[a];
+          P.d[0][a] = d[a];
+          P.d[1][a] = d2[a];
+          P.q[0][a] = -(sp.qw1 * sc) * dxdt[a];
+          P.q[1][a] = -(sp.qw2 * sc) * dxdt[a];
+        }
+        P.two = two;
       }
-      if (__popc(gen) > 3) {
-        if (!silent && !fast)
-          deposit_general3<DET, JT>(Jsm, two, cb[0], cb[1], fb[0], fb[1], db[0], db[1], sp.qw1, sp.qw2, dd, scale);
-      } else {
-        for (; gen; gen &= gen - 1)
-          deposit_general3_warp<DET, JT>(Jsm, act, __ffs(gen) - 1, two, cb[0], cb[1], fb[0], fb[1], db[0], db[1],
-                                         sp.qw1, sp.qw2, dd, scale);
-      }
+      __syncwarp(act);
+      deposit_general3_warp<DET, JT>(Jsm, act, &P);
       __syncwarp(act);
     }
   }
@@ -1050,7 +1170,8 @@ __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, l
       else esirkepov3<D, DET, 1>(Jsm, nn, xi, dd, qw, vv, dxdt, scale);
       bb_add<D>(blo, bhi, nn, 1, 1);
     } else {
-      if constexpr (D < 3) {
+      if constexpr (D == 2 && FREE) {
+        // body by body
 #pragma unroll 1
         for (int b = 0; b < (two ? 2 : 1); ++b) {
           float fb[3], db[3], vb[3];
@@ -1063,6 +1184,23 @@ __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, l
             cb[a] = b ? d2[a] : d[a];
           }
           deposit_general<D, DET, JT>(Jsm, cb, fb, db, b ? sp.qw2 : sp.qw1, vb, dxdt, scale);
+        }
+      } else if constexpr (D < 3) {
+        if (two) {
+          float fb[2][3], db[2][3], vb[2][3], dd[3];
+          int cb[2][3];
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            fb[0][a] = f[a]; fb[1][a] = f2[a];
+            db[0][a] = de1[a]; db[1][a] = de2[a];
+            vb[0][a] = v1[a]; vb[1][a] = v2[a];
+            cb[0][a] = d[a]; cb[1][a] = d2[a];
+            dd[a] = dxdt[a];
+          }
+          deposit_general_pair<D, DET, JT>(Jsm, cb[0], cb[1], fb[0], fb[1], db[0], db[1], sp.qw1, sp.qw2, vb[0], vb[1], dd,
+                                           scale);
+        } else if constexpr (D == 1) {
+          deposit_general<D, DET, JT>(Jsm, d, f, de1, sp.qw1, v1, dxdt, scale);
         }
       }
       int n0[3];
@@ -1415,7 +1553,7 @@ __device__ __forceinline__ void stage_done(const GridP &g, const PushArgs &A, co
 }
 
 // one tile of the push (the block's work for tile t)
-template <int D, bool DET, typename AfterLoop>
+template <int D, bool DET, bool FREE, typename AfterLoop>
 __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, const TmaMaps &T, const int t,
                                           const unsigned char qs, unsigned long long *bar, unsigned &phase, bool &failed,
                                           AfterLoop &&after_loop) {
@@ -1450,6 +1588,7 @@ __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, con
   // reading every staged value to find it cost 1% of the 3D push)
   const bool nofield = qs != QS_PUSH;
   __shared__ int run;
+  __shared__ PairJob jobs[D == 3 ? push_threads(D) / 32 : 1];  // a warp's general-case particle (3D)
   __shared__ unsigned sbb[6];
   if (tid < 6) sbb[tid] = tid < 3 ? 0xFFFFFFFFu : 0u;
   unsigned blo = 0xFFFFFFFFu, bhi = 0u;
@@ -1489,8 +1628,8 @@ __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, con
       if (k < n && !(moved && quiet_done(A.p[s], i))) {
         const int kn = at(rn);
         if (kn < n) prefetch_particle<D>(A.p[s], beg + kn, two);
-        push_particle<D, DET, JT>(g, A.sp[s], A.p[s], i, T0, Gsm, Jsm, A.status, A.jscale, blo,
-                                  bhi, nofield, A.far, A.far_n, A.far_cap, s, t);
+        push_particle<D, DET, FREE, JT>(g, A.sp[s], A.p[s], i, T0, Gsm, Jsm, A.status, A.jscale, blo, bhi, jobs,
+                                        nofield, A.far, A.far_n, A.far_cap, s, t);
         ++pushed;
       }
       r = rn;
@@ -1616,7 +1755,7 @@ __global__ void __launch_bounds__(push_threads(D), PB) k_push(GridP g, PushArgs 
   };
   grab(true);
   for (int t = next; t >= 0; t = next) {
-    push_tile<D, DET>(g, A, T, t, qs, &bar, phase, failed, [&]() { grab(false); });
+    push_tile<D, DET, PB == 3>(g, A, T, t, qs, &bar, phase, failed, [&]() { grab(false); });
     if (failed) give_up = 1;
     __syncthreads();  // every thread has read `next` before it changes
     if (give_up) break;  // a staging wait gave up twice (ST_TIMEOUT is set): stop

@@ -795,7 +795,7 @@ ProbeArgs probe_args(const bp_ctx *c) {
 // work.  When snap_fields is given, E^n and B^n (after the first half step)
 // and the particle state before the push are copied there; with push timing
 // on, events bracket the push.
-void step_launches(bp_ctx *c, const PushArgs &A, bool probes, cudaStream_t st, float *snap_fields,
+void step_launches(bp_ctx *c, PushArgs A, bool probes, cudaStream_t st, float *snap_fields,
                    std::vector<bp_part_copy> *snap_parts) {
   const GridP &g = c->g;
   float *E[3] = {c->F[0], c->F[1], c->F[2]}, *B[3] = {c->F[3], c->F[4], c->F[5]}, *J[3] = {c->F[6], c->F[7], c->F[8]};
@@ -806,10 +806,19 @@ void step_launches(bp_ctx *c, const PushArgs &A, bool probes, cudaStream_t st, f
   const bool direct = push_direct(g, A);
   // re-sort when a particle left its tile margin in the previous step
   if (A.nsp) launch_sort(g, A.nsp, A.sp, A.p, c->sb, c->status, st);
-  launch_yee_b(g, B, c->Bn, cE, 0.5f * g.dt, c->jfx, A, direct ? ant : none, c->act, st);
+  // a snapshot's E^n and B^n are written by the B update itself (1D, 2D: the
+  // push then reads B^n there; in 3D its tensor maps are those of Bn)
+  const bool store = snap_fields && g.D < 3;
+  float *sE[3] = {}, *Bn[3] = {c->Bn[0], c->Bn[1], c->Bn[2]};
+  for (int k = 0; k < 3 && store; ++k) {
+    sE[k] = snap_fields + (size_t)k * g.ncell;
+    Bn[k] = snap_fields + (size_t)(3 + k) * g.ncell;
+    A.B[k] = Bn[k];
+  }
+  launch_yee_b(g, B, Bn, cE, 0.5f * g.dt, c->jfx, A, direct ? ant : none, c->act, store ? sE : nullptr, st);
   if (snap_fields) {
     CopyList L;
-    for (int k = 0; k < 6; ++k)
+    for (int k = 0; k < 6 && !store; ++k)
       cl_add(c, L, k < 3 ? c->F[k] : c->Bn[k - 3], snap_fields + (size_t)k * g.ncell, sizeof(float) * g.ncell);
     int q = 0;
     for (auto &s : c->sp)
@@ -1752,12 +1761,16 @@ int bp_backward(bp_ctx *c, int probe_id, const float *dl_dprobe, int sid, double
         launch_adj_inject(ad.lamE[P.comp], P.nodes, P.npts, ad.dl + n * P.npts, as);
         c->launches++;
       }
-      // E update with Mur faces, transposed (H is clear: zeroed before the
-      // first reverse step, then by the previous step's B transpose)
-      launch_adj_e(g, ad.lamE, ad.H, ad.lamB, ad.lamJ, as);
-      for (int k = 0; k < 3; ++k) std::swap(ad.lamE[k], ad.H[k]);
+      std::vector<PartP> pp;
+      for (size_t q = 0; q < c->sp.size(); ++q) pp.push_back(ad.st_parts[bank * K + j][q].p);
+      // E update with Mur faces, transposed, and the step's work list
+      const bool inplace = adj_e_inplace(g);
+      launch_adj_e(g, ad.lamE, ad.H, ad.lamB, ad.lamJ, (int)c->sp.size(), pp.data(), bufs, as);
+      // the result is in H (clear: zeroed before the first reverse step, then
+      // by the previous step's B transpose)
+      for (int k = 0; k < 3 && !inplace; ++k) std::swap(ad.lamE[k], ad.H[k]);
       // B^{n+1/2} = B^n - dt/2 curl E^n; clears H (the old E adjoint) for the next step
-      launch_adj_b(g, ad.lamE, ad.lamB, 0.5f * g.dt, ad.H, as);
+      launch_adj_b(g, ad.lamE, ad.lamB, 0.5f * g.dt, inplace ? nullptr : ad.H, inplace, as);
       // particles, with E^n, B^n and the particle state stored for step n
       const float *En[3], *Bn[3], *lJ[3] = {ad.lamJ[0], ad.lamJ[1], ad.lamJ[2]};
       const float *sf = ad.st_fields[bank * K + j];
@@ -1765,17 +1778,16 @@ int bp_backward(bp_ctx *c, int probe_id, const float *dl_dprobe, int sid, double
         En[k] = sf + (size_t)k * g.ncell;
         Bn[k] = sf + (size_t)(3 + k) * g.ncell;
       }
-      std::vector<PartP> pp;
-      for (size_t q = 0; q < c->sp.size(); ++q) pp.push_back(ad.st_parts[bank * K + j][q].p);
       launch_adj_push(g, (int)c->sp.size(), sps.data(), pp.data(), xbs.data(), acbs.data(), ebs.data(), caps.data(), En,
                       Bn, lJ, bufs, ad.lamE, ad.lamB, ad.status, as);
       // B^n = B^{n-1/2} - dt/2 curl E^n
-      launch_adj_b(g, ad.lamE, ad.lamB, 0.5f * g.dt, nullptr, as);
-      // E transpose and its Mur passes (one per pass and open axis), two B
-      // transposes, work list, particle adjoint, scatter, fixed-point sum
+      launch_adj_b(g, ad.lamE, ad.lamB, 0.5f * g.dt, nullptr, false, as);
+      // E transpose (with Mur passes, one per pass and open axis, and the work
+      // list apart unless in place), two B transposes, particle adjoint,
+      // scatter, fixed-point sum
       int nopen = 0;
       for (int a = 0; a < g.D; ++a) nopen += g.bc[a] == BP_OPEN;
-      c->launches += 1 + nopen * nopen + 2 + 4;
+      c->launches += (inplace ? 1 : 2 + nopen * nopen) + 2 + 3;
       int rc = check_launch(c, "backward step");
       if (rc) return rc;
     }

@@ -553,8 +553,11 @@ int push_prepare(const GridP &g, int det, int blocks[2]);
 // = B^n - h curl E (the same curl).  Clears the fixed-point current jfx (may be
 // null) and the push's counters of a, and runs the antenna of ant.
 // act (per tile, optional): tiles to update; the others keep zero E, B, J.
+// sE (optional): E^n copied there and Bn an array that is not kept zero in the
+// other tiles (both are then written everywhere).
 void launch_yee_b(const GridP &g, float *const B[3], float *const Bn[3], const float *const E[3], float h,
-                  unsigned long long *jfx, const PushArgs &a, const AntArgs &ant, const unsigned char *act, cudaStream_t s);
+                  unsigned long long *jfx, const PushArgs &a, const AntArgs &ant, const unsigned char *act,
+                  float *const sE[3], cudaStream_t s);
 // recompute the tile marks (g.fnz) from E, B (F[0..5]) after a write from outside the step
 void launch_field_marks(const GridP &g, const float *const F[6], cudaStream_t s);
 // E <- E + dt (curl B - J) with Mur faces; advances the clock's step number.
@@ -617,7 +620,6 @@ void launch_divE_minus(const GridP &g, const float *const E[3], double *R, cudaS
 
 // adjoint
 void launch_adj_inject(float *lam, const long long *nodes, long long npts, const float *dl, cudaStream_t s);
-void launch_adj_e(const GridP &g, float *G[3], float *H[3], float *lamB[3], float *lamJ[3], cudaStream_t s);
 // device-to-device copies of whole 4-byte-word arrays, issued as one kernel
 struct CopyList {
   static constexpr int MAX = 32;
@@ -627,8 +629,6 @@ struct CopyList {
   long long words[MAX];
 };
 void launch_copy_many(const CopyList &L, int sms, cudaStream_t s);
-// zero (optional): three arrays cleared on the way
-void launch_adj_b(const GridP &g, float *lamE[3], float *lamB[3], float h, float *zero[3], cudaStream_t s);
 size_t adj_push_smem(int D);
 constexpr int kAdjChunk = 256;  // particles per work item of the particle adjoint
 int adj_prepare(int D, int *push_blocks, int *scat_blocks);
@@ -644,6 +644,14 @@ struct AdjBufs {
   int chunk;                // particles per work item
   int push_blocks, scat_blocks;
 };
+// The E update transposed, and the step's work list.  Where adj_e_inplace says
+// so, G (the E adjoint) is only read, H is not used and the next launch_adj_b
+// does the open faces (faces); else G is consumed and the result is in H.
+bool adj_e_inplace(const GridP &g);
+void launch_adj_e(const GridP &g, float *G[3], float *H[3], float *lamB[3], float *lamJ[3], int nsp, const PartP *p,
+                  const AdjBufs &b, cudaStream_t s);
+// zero (optional): three arrays cleared on the way
+void launch_adj_b(const GridP &g, float *lamE[3], float *lamB[3], float h, float *zero[3], bool faces, cudaStream_t s);
 void launch_adj_push(const GridP &g, int nsp, const SpecP *sp, const PartP *p, float *const xb[], double *const acb[],
                      float *const eb[], const long long *cap, const float *const E[3], const float *const B[3],
                      const float *const lamJ[3], const AdjBufs &b, float *lamE[3], float *lamB[3], int *status,

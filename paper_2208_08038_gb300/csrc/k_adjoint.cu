@@ -135,8 +135,123 @@ __device__ __forceinline__ float g_up_a4(const GridP &g, const float4 &Gu, int c
   return e_int<D>(g, comp, x) ? el(Gu, i) : 0.0f;
 }
 
-// interior E update transposed: H += G (interior and exterior nodes),
-// lamJ = -dt G (interior), lamB += dt curl_B^T (G on interior nodes)
+// The Mur nodes of the x faces transposed, where x is the only open axis.  A face
+// node and its inward neighbour lie in one group of four cells: of the E adjoint
+// G, v = G[face] goes to the neighbour's new value (G[adj] + km v, used by the
+// interior transposes) and to the old values (adj + v, face - km v).
+struct FaceX {
+  int on;
+  float km;
+};
+// the neighbour's value before the interior transposes (components y and z)
+__device__ __forceinline__ void face_in(const GridP &g, const FaceX &F, int c0, float4 &G) {
+  if (!F.on) return;
+  if (c0 == 0) G.y = fmaf(F.km, G.x, G.y);
+  if (c0 + 4 == g.n[0]) G.z = fmaf(F.km, G.w, G.z);
+}
+// the adjoint of the old E (the interior nodes' passes through)
+__device__ __forceinline__ void face_out(const GridP &g, const FaceX &F, int c0, float4 &G) {
+  if (!F.on) return;
+  face_in(g, F, c0, G);
+  if (c0 == 0) {
+    G.y = G.x + G.y;
+    G.x = -(F.km * G.x);
+  }
+  if (c0 + 4 == g.n[0]) {
+    G.z = G.w + G.z;
+    G.w = -(F.km * G.w);
+  }
+}
+
+// the work list's inputs, for the blocks that build it
+struct WorkIn {
+  int nsp, chunk, cap, blocks;
+  const int *tstart[BP_MAX_SPECIES];
+  int *n;
+  int4 *item;
+};
+// one thread per tile and species: the chunks of its particles appended
+__device__ __forceinline__ void list_work(const GridP &g, const WorkIn &W) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= g.ntiles * W.nsp) return;
+  const int t = q % g.ntiles, s = q / g.ntiles;
+  const int beg = W.tstart[s][t], end = W.tstart[s][t + 1];
+  if (end <= beg) return;
+  const int m = (end - beg + W.chunk - 1) / W.chunk;
+  const int at = atomicAdd(W.n, m);
+  for (int k = 0; k < m && at + k < W.cap; ++k)
+    W.item[at + k] = make_int4(t, s, beg + k * W.chunk, min(beg + (k + 1) * W.chunk, end));
+}
+
+// interior E update transposed, with open faces on x alone or none: lamJ = -dt G
+// (interior), lamB += dt curl_B^T (G on interior nodes).  The E adjoint itself
+// only changes at the faces, which the next B transpose does (k_adj_b), so no
+// second E array is written and cleared: 48 B per cell instead of 72 and 12.
+// The first blocks build the step's work list.
+template <int D>
+__global__ void __launch_bounds__(128) k_adj_ex(GridP g, const float *G0, const float *G1, const float *G2, float *B0,
+                                                float *B1, float *B2, float *J0, float *J1, float *J2, FaceX F,
+                                                const __grid_constant__ WorkIn W) {
+  if ((int)blockIdx.x < W.blocks) {
+    list_work(g, W);
+    return;
+  }
+  Cell4 C;
+  if (!row_cell4<D>(g, C, (int)blockIdx.x - W.blocks)) return;
+  const long long q = C.q;
+  const float dt = g.dt;
+  const float4 g0 = ld4(G0 + q);
+  float4 g1 = ld4(G1 + q), g2 = ld4(G2 + q);
+  const float g1n = G1[q + C.up[0]], g2n = G2[q + C.up[0]];  // x neighbours of the last cell (never a face's)
+  float4 g2y = g2, g0y = g0, g1z = g1, g0z = g0;
+  if (D >= 2) {
+    g2y = ld4(G2 + q + C.up[1]);
+    g0y = ld4(G0 + q + C.up[1]);
+  }
+  if (D >= 3) {
+    g1z = ld4(G1 + q + C.up[2]);
+    g0z = ld4(G0 + q + C.up[2]);
+  }
+  face_in(g, F, C.c[0], g1);
+  face_in(g, F, C.c[0], g2);
+  if (D >= 2) face_in(g, F, C.c[0], g2y);
+  if (D >= 3) face_in(g, F, C.c[0], g1z);
+  {
+    const float4 gg[3] = {g0, g1, g2};
+    float *J[3] = {J0, J1, J2};
+#pragma unroll
+    for (int comp = 0; comp < 3; ++comp) {
+      float4 j;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int x[3] = {C.c[0] + i, C.c[1], C.c[2]};
+        set_el(j, i, e_int<D>(g, comp, x) ? -dt * el(gg[comp], i) : 0.0f);
+      }
+      st4(J[comp] + q, j);
+    }
+  }
+  float4 b0 = ld4(B0 + q), b1 = ld4(B1 + q), b2 = ld4(B2 + q);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float bx = 0.0f, by = 0.0f, bz = 0.0f;
+    if (D >= 3) bx += (g_here4<D>(g, g1, 1, C.c, i) - g_up_a4<D>(g, g1z, 1, C.c, i, 2)) * g.idx[2];
+    if (D >= 2) bx -= (g_here4<D>(g, g2, 2, C.c, i) - g_up_a4<D>(g, g2y, 2, C.c, i, 1)) * g.idx[1];
+    if (D >= 3) by -= (g_here4<D>(g, g0, 0, C.c, i) - g_up_a4<D>(g, g0z, 0, C.c, i, 2)) * g.idx[2];
+    by += (g_here4<D>(g, g2, 2, C.c, i) - g_up_x4<D>(g, g2, g2n, 2, C.c, i)) * g.idx[0];
+    if (D >= 2) bz += (g_here4<D>(g, g0, 0, C.c, i) - g_up_a4<D>(g, g0y, 0, C.c, i, 1)) * g.idx[1];
+    bz -= (g_here4<D>(g, g1, 1, C.c, i) - g_up_x4<D>(g, g1, g1n, 1, C.c, i)) * g.idx[0];
+    set_el(b0, i, el(b0, i) + dt * bx);
+    set_el(b1, i, el(b1, i) + dt * by);
+    set_el(b2, i, el(b2, i) + dt * bz);
+  }
+  st4(B0 + q, b0);
+  st4(B1 + q, b1);
+  st4(B2 + q, b2);
+}
+
+// interior E update transposed, open faces on other axes (after k_adj_mur):
+// H += G (interior and exterior nodes), lamJ = -dt G (interior), lamB += dt
+// curl_B^T (G on interior nodes)
 template <int D>
 __global__ void __launch_bounds__(128) k_adj_e(GridP g, const float *G0, const float *G1, const float *G2, float *H0,
                                                float *H1, float *H2, float *B0, float *B1, float *B2, float *J0,
@@ -224,11 +339,12 @@ __device__ __forceinline__ float b_dn_a4(const GridP &g, const float4 &Bd, int p
 
 // B <- B - h curl E transposed: E adjoint -= h curl_E^T (B adjoint on
 // non-exterior B nodes); the B adjoint itself passes through.  Z0..Z2, when
-// given, are cleared on the way (the buffer the next E transpose fills).
+// given, are cleared on the way (the buffer the next E transpose fills).  F: the
+// x faces' part of the E transpose first (see k_adj_ex).
 template <int D>
 __global__ void __launch_bounds__(128) k_adj_b(GridP g, float *E0, float *E1, float *E2, const float *B0,
                                                const float *B1, const float *B2, float h, float *Z0, float *Z1,
-                                               float *Z2) {
+                                               float *Z2, FaceX F) {
   Cell4 C;
   if (!row_cell4<D>(g, C)) return;
   const long long q = C.q;
@@ -244,6 +360,8 @@ __global__ void __launch_bounds__(128) k_adj_b(GridP g, float *E0, float *E1, fl
     b0z = ld4(B0 + q + C.dn[2]);
   }
   float4 e0 = ld4(E0 + q), e1 = ld4(E1 + q), e2 = ld4(E2 + q);
+  face_out(g, F, C.c[0], e1);
+  face_out(g, F, C.c[0], e2);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     float ex = 0.0f, ey = 0.0f, ez = 0.0f;
@@ -278,6 +396,16 @@ __device__ __forceinline__ float dqshape(float x) {
   return 0.0f;
 }
 
+// x / b for a normal b with its correctly rounded reciprocal r: a quotient
+// estimate and one correction by its exact remainder, correctly rounded
+// (Markstein, "Computation of elementary functions on the IBM RISC System/6000
+// processor", IBM J. Res. Dev. 34, 1990, theorem 8) while x r and the remainder
+// do not underflow
+__device__ __forceinline__ float quot(float x, float b, float r) {
+  const float q = __fmul_rn(x, r);
+  return fmaf(fmaf(-b, q, x), r, q);
+}
+
 // reverse of boris(): given the adjoint of the pushed momentum, the adjoints
 // of the old momentum, E and B
 __device__ __forceinline__ void boris_adj(float h, const float E[3], const float B[3], const float u0[3], const float ubn[3],
@@ -286,11 +414,18 @@ __device__ __forceinline__ void boris_adj(float h, const float E[3], const float
 #pragma unroll
   for (int a = 0; a < 3; ++a) um[a] = u0[a] + h * E[a];
   float gm = sqrtf(1.0f + um[0] * um[0] + um[1] * um[1] + um[2] * um[2]);
+  // One division each for gamma, gamma^2 and 1 + t^2, the quotients from their
+  // reciprocals (quot: the same bits).  A zero field component sent each of the
+  // 16 divisions of a body down the division's out-of-line path: 35 of them were
+  // a quarter of the reversed push's instructions (2D, 524 k ions: 107 us
+  // before, 72 with this and one staging per tile).
+  const float ig = 1.0f / gm, gm2 = gm * gm, ig2 = 1.0f / gm2;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) t[a] = h * B[a] / gm;
+  for (int a = 0; a < 3; ++a) t[a] = quot(h * B[a], gm, ig);
   float t2 = t[0] * t[0] + t[1] * t[1] + t[2] * t[2];
+  const float dt2 = 1.0f + t2, it = 1.0f / dt2;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) sv[a] = 2.0f * t[a] / (1.0f + t2);
+  for (int a = 0; a < 3; ++a) sv[a] = quot(2.0f * t[a], dt2, it);
   c1[0] = um[0] + (um[1] * t[2] - um[2] * t[1]);
   c1[1] = um[1] + (um[2] * t[0] - um[0] * t[2]);
   c1[2] = um[2] + (um[0] * t[1] - um[1] * t[0]);
@@ -313,18 +448,17 @@ __device__ __forceinline__ void boris_adj(float h, const float E[3], const float
   tb[1] = cb[2] * um[0] - cb[0] * um[2];
   tb[2] = cb[0] * um[1] - cb[1] * um[0];
   float ts = t[0] * sb[0] + t[1] * sb[1] + t[2] * sb[2];
-  float i1 = 1.0f / (1.0f + t2);
 #pragma unroll
-  for (int a = 0; a < 3; ++a) tb[a] += 2.0f * sb[a] * i1 - 4.0f * t[a] * ts * i1 * i1;
+  for (int a = 0; a < 3; ++a) tb[a] += 2.0f * sb[a] * it - 4.0f * t[a] * ts * it * it;
   float gmb = 0.0f;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    Bb[a] = h * tb[a] / gm;
-    gmb -= h * B[a] * tb[a] / (gm * gm);
+    Bb[a] = quot(h * tb[a], gm, ig);
+    gmb -= quot(h * B[a] * tb[a], gm2, ig2);
   }
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    umb[a] += um[a] * gmb / gm;
+    umb[a] += quot(um[a] * gmb, gm, ig);
     ub0[a] = umb[a];
     Eb[a] += h * umb[a];
   }
@@ -653,6 +787,9 @@ __device__ void adj_particle(const GridP &g, const SpecP &sp, const PartP &P, Ad
   const int cell = P.cell[i];
   if (cell < 0) return;
   const int id = P.id[i];
+  // the carried adjoints, by load id, wanted after the gather and the deposit
+#pragma unroll
+  for (int a = 0; a < 12; ++a) asm volatile("prefetch.global.L1 [%0];" ::"l"(S.xb + a * S.cap + id));
   int c[3];
   unpack_cell(g, cell, c);
   float f[3] = {0.0f, 0.0f, 0.0f}, r[3] = {0.0f, 0.0f, 0.0f}, u1[3], u2[3] = {0.0f, 0.0f, 0.0f};
@@ -874,18 +1011,7 @@ __device__ void adj_particle(const GridP &g, const SpecP &sp, const PartP &P, Ad
   }
 }
 
-// one thread per tile and species: the chunks of its particles appended
-__global__ void k_adj_work(GridP g, AdjArgs A, AdjWork W, int chunk) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= g.ntiles * A.nsp) return;
-  const int t = q % g.ntiles, s = q / g.ntiles;
-  const int beg = A.p[s].tstart[t], end = A.p[s].tstart[t + 1];
-  if (end <= beg) return;
-  const int m = (end - beg + chunk - 1) / chunk;
-  const int at = atomicAdd(W.n, m);
-  for (int k = 0; k < m && at + k < W.cap; ++k)
-    W.item[at + k] = make_int4(t, s, beg + k * chunk, min(beg + (k + 1) * chunk, end));
-}
+__global__ void k_adj_work(GridP g, const __grid_constant__ WorkIn W) { list_work(g, W); }
 
 // The staged boxes of tile t: E^n, B^n (gather box) and the J adjoint, as
 // per-thread asynchronous 4-byte copies (zero fill outside open faces),
@@ -960,8 +1086,8 @@ __host__ __device__ constexpr int adj_box_floats() {
   return 6 * Box<D>::GCELLS + 3 * Box<D>::JCELLS;
 }
 
-// the reversed push of the step's work items, round-robin over the
-// resident blocks
+// the reversed push of the step's work items, shared out over the resident
+// blocks
 template <int D>
 __global__ void __launch_bounds__(256, D == 3 ? 1 : 2) k_adj_push(GridP g, AdjArgs A, AdjWork W) {
   using BX = Box<D>;
@@ -972,32 +1098,41 @@ __global__ void __launch_bounds__(256, D == 3 ? 1 : 2) k_adj_push(GridP g, AdjAr
   const int tid = threadIdx.x, bs = blockDim.x;
   const int nw = min(*W.n, W.cap);
   float emax = 0.0f;
-  int w = blockIdx.x, cur = 0, T0[3], Tn[3];
-  if (w < nw) {
+  // each block a contiguous range of items: the chunks of a tile follow each
+  // other in the list, and its boxes are staged once for those a block takes
+  int w = (int)((long long)nw * blockIdx.x / gridDim.x), cur = 0, T0[3], Tn[3];
+  const int w1 = (int)((long long)nw * (blockIdx.x + 1) / gridDim.x);
+  if (w < w1) {
     int4 it = W.item[w];
     adj_stage<D>(g, A, it.x, T0, buf, buf + 6 * GC);
+    bool staged = true;  // the current boxes were staged for this item
     for (;;) {
-      const int wn = w + (int)gridDim.x;
-      const bool more = wn < nw;
-      const int4 nx = more ? W.item[wn] : make_int4(0, 0, 0, 0);
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      __syncthreads();  // the current boxes have landed; the other set is no longer read
+      const bool more = w + 1 < w1;
+      const int4 nx = more ? W.item[w + 1] : make_int4(0, 0, 0, 0);
+      const bool other = more && nx.x != it.x;
+      if (staged) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();  // the current boxes have landed; the other set is no longer read
+      }
       float *Gsm = buf + cur * BOX;
-      if (NB == 2 && more) adj_stage<D>(g, A, nx.x, Tn, buf + (cur ^ 1) * BOX, buf + (cur ^ 1) * BOX + 6 * GC);
+      if (NB == 2 && other) adj_stage<D>(g, A, nx.x, Tn, buf + (cur ^ 1) * BOX, buf + (cur ^ 1) * BOX + 6 * GC);
       const int s = it.y;
       for (long long i = it.z + tid; i < it.w; i += bs)
         adj_particle<D>(g, A.sp[s], A.p[s], A.st[s], i, T0, Gsm, Gsm + 6 * GC, stash, emax);
       if (!more) break;
-      if (NB == 1) {
+      if (NB == 1 && other) {
         __syncthreads();  // every thread is done with the set before it is restaged
         adj_stage<D>(g, A, nx.x, Tn, buf, buf + 6 * GC);
       }
+      staged = other;
+      if (other) {
+        T0[0] = Tn[0];
+        T0[1] = Tn[1];
+        T0[2] = Tn[2];
+        if (NB == 2) cur ^= 1;
+      }
       it = nx;
-      w = wn;
-      T0[0] = Tn[0];
-      T0[1] = Tn[1];
-      T0[2] = Tn[2];
-      if (NB == 2) cur ^= 1;
+      ++w;
     }
   }
   // non-negative floats order like their bit patterns
@@ -1103,17 +1238,28 @@ __global__ void __launch_bounds__(256) k_adj_scatter(GridP g, ScatArgs S, AdjWor
   if (blockIdx.x == 0 && tid == 0) *S.kst = k;
   __shared__ int sbb[6];  // the chunk's body cells (box coordinates): lowest, highest per axis
   for (int q = tid; q < 12 * GC; q += bs) A[q] = 0u;
-  for (int w = blockIdx.x; w < nw; w += gridDim.x) {
+  // A block takes a contiguous range of items and flushes its box once for the
+  // chunks of a tile that follow each other (at most 64: a node's low word
+  // holds 2^16 adds).
+  const int w1 = (int)((long long)nw * (blockIdx.x + 1) / gridDim.x);
+  int lo[3], hi[3], chunks = 0;
+  for (int w = (int)((long long)nw * blockIdx.x / gridDim.x); w < w1; ++w) {
     const int4 it = W.item[w];
     const int t = it.x, s = it.y;
     const int tc[3] = {t % g.nt[0], (t / g.nt[0]) % g.nt[1], t / (g.nt[0] * g.nt[1])};
     const int T0[3] = {tc[0] * Geo<D>::L0, tc[1] * Geo<D>::L1, tc[2] * Geo<D>::L2};
-    if (tid < 3) {
-      sbb[tid] = 1 << 30;
-      sbb[3 + tid] = -(1 << 30);
+    if (chunks == 0) {
+      if (tid < 3) {
+        sbb[tid] = 1 << 30;
+        sbb[3 + tid] = -(1 << 30);
+      }
+      __syncthreads();  // the box is clear (the previous flush cleared what it read)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        lo[a] = 1 << 30;
+        hi[a] = -(1 << 30);
+      }
     }
-    __syncthreads();  // the box is clear (the previous item's flush cleared what it read)
-    int lo[3] = {1 << 30, 1 << 30, 1 << 30}, hi[3] = {-(1 << 30), -(1 << 30), -(1 << 30)};
     const PartP &P = S.p[s];
     const bool two = S.sp[s].kind == BP_TWO_BODY;
     const long long cap = P.cap, ec = S.ecap[s];
@@ -1156,6 +1302,8 @@ __global__ void __launch_bounds__(256) k_adj_scatter(GridP g, ScatArgs S, AdjWor
       scatter_comp<D, 5>(A + 4 * GC, d, f, e[4], d2, f2, e[10], two);
       scatter_comp<D, 3>(A + 5 * GC, d, f, e[5], d2, f2, e[11], two);
     }
+    if (++chunks < 64 && w + 1 < w1 && W.item[w + 1].x == t) continue;
+    chunks = 0;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
       const int l = __reduce_min_sync(0xFFFFFFFFu, lo[a]), h = __reduce_max_sync(0xFFFFFFFFu, hi[a]);
@@ -1284,25 +1432,62 @@ void launch_adj_inject(float *lam, const long long *nodes, long long npts, const
   k_adj_inject<<<blocks_for(npts, 256), 256, 0, s>>>(lam, nodes, npts, dl);
 }
 
-void launch_adj_e(const GridP &g, float *G[3], float *H[3], float *lamB[3], float *lamJ[3], cudaStream_t s) {
-  int nopen = 0;
-  for (int a = 0; a < g.D; ++a) nopen += g.bc[a] == BP_OPEN;
-  for (int p = nopen; p >= 1; --p)
-    for (int a = 0; a < g.D; ++a)
-      if (g.bc[a] == BP_OPEN)
-        k_adj_mur<<<blocks_for(4 * (g.ncell / g.n[a]), 256), 256, 0, s>>>(g, G[0], G[1], G[2], H[0], H[1], H[2], a, p);
-  const int nb = row_blocks4(g, 128);
-  if (g.D == 1) k_adj_e<1><<<nb, 128, 0, s>>>(g, G[0], G[1], G[2], H[0], H[1], H[2], lamB[0], lamB[1], lamB[2], lamJ[0], lamJ[1], lamJ[2]);
-  else if (g.D == 2) k_adj_e<2><<<nb, 128, 0, s>>>(g, G[0], G[1], G[2], H[0], H[1], H[2], lamB[0], lamB[1], lamB[2], lamJ[0], lamJ[1], lamJ[2]);
-  else k_adj_e<3><<<nb, 128, 0, s>>>(g, G[0], G[1], G[2], H[0], H[1], H[2], lamB[0], lamB[1], lamB[2], lamJ[0], lamJ[1], lamJ[2]);
+// whether the E transpose needs no second E array: open faces on x alone, or none
+bool adj_e_inplace(const GridP &g) {
+  for (int a = 1; a < g.D; ++a)
+    if (g.bc[a] == BP_OPEN) return false;
+  return true;
+}
+static FaceX face_x(const GridP &g, bool on) {
+  return FaceX{on && g.bc[0] == BP_OPEN ? 1 : 0, (g.dt - g.dx[0]) / (g.dt + g.dx[0])};
+}
+static WorkIn work_in(const GridP &g, int nsp, const PartP *p, const AdjBufs &b, int threads) {
+  WorkIn W;
+  memset(&W, 0, sizeof W);
+  W.nsp = nsp;
+  W.chunk = b.chunk;
+  W.cap = b.work_cap;
+  W.n = b.nwork;
+  W.item = b.work;
+  for (int k = 0; k < nsp; ++k) W.tstart[k] = p[k].tstart;
+  W.blocks = (g.ntiles * nsp + threads - 1) / threads;
+  return W;
 }
 
-void launch_adj_b(const GridP &g, float *lamE[3], float *lamB[3], float h, float *zero[3], cudaStream_t s) {
+void launch_adj_e(const GridP &g, float *G[3], float *H[3], float *lamB[3], float *lamJ[3], int nsp, const PartP *p,
+                  const AdjBufs &b, cudaStream_t s) {
+  const int nb = row_blocks4(g, 128);
+  if (adj_e_inplace(g)) {
+    const FaceX F = face_x(g, true);
+    const WorkIn W = work_in(g, nsp, p, b, 128);
+#define ADJ_EX(DD)                                                                                                      \
+  k_adj_ex<DD><<<nb + W.blocks, 128, 0, s>>>(g, G[0], G[1], G[2], lamB[0], lamB[1], lamB[2], lamJ[0], lamJ[1], lamJ[2], \
+                                             F, W)
+    if (g.D == 1) ADJ_EX(1);
+    else if (g.D == 2) ADJ_EX(2);
+    else ADJ_EX(3);
+#undef ADJ_EX
+    return;
+  }
+  int nopen = 0;
+  for (int a = 0; a < g.D; ++a) nopen += g.bc[a] == BP_OPEN;
+  for (int p_ = nopen; p_ >= 1; --p_)
+    for (int a = 0; a < g.D; ++a)
+      if (g.bc[a] == BP_OPEN)
+        k_adj_mur<<<blocks_for(4 * (g.ncell / g.n[a]), 256), 256, 0, s>>>(g, G[0], G[1], G[2], H[0], H[1], H[2], a, p_);
+  if (g.D == 2) k_adj_e<2><<<nb, 128, 0, s>>>(g, G[0], G[1], G[2], H[0], H[1], H[2], lamB[0], lamB[1], lamB[2], lamJ[0], lamJ[1], lamJ[2]);
+  else k_adj_e<3><<<nb, 128, 0, s>>>(g, G[0], G[1], G[2], H[0], H[1], H[2], lamB[0], lamB[1], lamB[2], lamJ[0], lamJ[1], lamJ[2]);
+  const WorkIn W = work_in(g, nsp, p, b, 256);
+  k_adj_work<<<W.blocks, 256, 0, s>>>(g, W);
+}
+
+void launch_adj_b(const GridP &g, float *lamE[3], float *lamB[3], float h, float *zero[3], bool faces, cudaStream_t s) {
   const int nb = row_blocks4(g, 128);
   float *z0 = zero ? zero[0] : nullptr, *z1 = zero ? zero[1] : nullptr, *z2 = zero ? zero[2] : nullptr;
-  if (g.D == 1) k_adj_b<1><<<nb, 128, 0, s>>>(g, lamE[0], lamE[1], lamE[2], lamB[0], lamB[1], lamB[2], h, z0, z1, z2);
-  else if (g.D == 2) k_adj_b<2><<<nb, 128, 0, s>>>(g, lamE[0], lamE[1], lamE[2], lamB[0], lamB[1], lamB[2], h, z0, z1, z2);
-  else k_adj_b<3><<<nb, 128, 0, s>>>(g, lamE[0], lamE[1], lamE[2], lamB[0], lamB[1], lamB[2], h, z0, z1, z2);
+  const FaceX F = face_x(g, faces && adj_e_inplace(g));
+  if (g.D == 1) k_adj_b<1><<<nb, 128, 0, s>>>(g, lamE[0], lamE[1], lamE[2], lamB[0], lamB[1], lamB[2], h, z0, z1, z2, F);
+  else if (g.D == 2) k_adj_b<2><<<nb, 128, 0, s>>>(g, lamE[0], lamE[1], lamE[2], lamB[0], lamB[1], lamB[2], h, z0, z1, z2, F);
+  else k_adj_b<3><<<nb, 128, 0, s>>>(g, lamE[0], lamE[1], lamE[2], lamB[0], lamB[1], lamB[2], h, z0, z1, z2, F);
 }
 
 // box sets, then the 256 threads' slices of gather derivatives (12 D floats each)
@@ -1345,16 +1530,14 @@ int adj_prepare(int D, int *push_blocks, int *scat_blocks) {
 template <int D>
 void adj_launch_all(const GridP &g, const AdjArgs &A, const ScatArgs &S, const AdjWork &W, const AdjBufs &b,
                     float *lamE[3], float *lamB[3], cudaStream_t s) {
-  const int nq = g.ntiles * A.nsp;
-  k_adj_work<<<(nq + 255) / 256, 256, 0, s>>>(g, A, W, b.chunk);
   k_adj_push<D><<<b.push_blocks, 256, adj_push_smem(D), s>>>(g, A, W);
   k_adj_scatter<D><<<b.scat_blocks, 256, adj_scatter_smem(D), s>>>(g, S, W);
   k_adj_fxsum<D><<<g.ntiles, 256, 0, s>>>(g, b.lfx, b.dirty, b.kst, lamE[0], lamE[1], lamE[2], lamB[0], lamB[1],
                                            lamB[2], b.emax, b.nwork);
 }
 
-// the particle adjoint of one step: the work list, the reversed push with
-// the position derivatives of the gather (k_adj_push), the field-adjoint
+// the particle adjoint of one step (its work list built by launch_adj_e): the
+// reversed push with the position derivatives of the gather (k_adj_push), the field-adjoint
 // scatter (k_adj_scatter), then its sum into lamE, lamB (k_adj_fxsum)
 void launch_adj_push(const GridP &g, int nsp, const SpecP *sp, const PartP *p, float *const xb[], double *const acb[],
                      float *const eb[], const long long *cap, const float *const E[3], const float *const B[3],

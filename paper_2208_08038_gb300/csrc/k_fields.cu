@@ -75,7 +75,8 @@ __global__ void __launch_bounds__(128) k_yee_b(const __grid_constant__ GridP g, 
                                                const float *__restrict__ Ex, const float *__restrict__ Ey,
                                                const float *__restrict__ Ez, float h, unsigned long long *jfx,
                                                int *tile_n, int *tile_ctr, int *far_n,
-                                               const unsigned char *__restrict__ act, const __grid_constant__ AntArgs ant) {
+                                               const unsigned char *__restrict__ act, float *S0, float *S1, float *S2,
+                                               const __grid_constant__ AntArgs ant) {
   int block = (int)blockIdx.x;
   if (ANT) {
     if (block < ant.blocks) {
@@ -91,8 +92,19 @@ __global__ void __launch_bounds__(128) k_yee_b(const __grid_constant__ GridP g, 
   }
   Cell4 C;
   if (!row_cell4<D>(g, C, block)) return;
-  if (act && !act[tile_of(g, C.c)]) return;  // E and B zero around the tile: B stays zero
   const long long q = C.q;
+  if (act && !act[tile_of(g, C.c)]) {  // E and B zero around the tile: B stays zero
+    if (S0) {
+      const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      st4(S0 + q, z);
+      st4(S1 + q, z);
+      st4(S2 + q, z);
+      st4(Nx + q, z);
+      st4(Ny + q, z);
+      st4(Nz + q, z);
+    }
+    return;
+  }
   const float4 ex = ld4(Ex + q), ey = ld4(Ey + q), ez = ld4(Ez + q);
   const float eyn = Ey[q + C.up[0]], ezn = Ez[q + C.up[0]];  // x neighbours of the last cell
   float4 ezy = ez, exy = ex, eyz = ey, exz = ex;
@@ -135,6 +147,11 @@ __global__ void __launch_bounds__(128) k_yee_b(const __grid_constant__ GridP g, 
       if (D >= 2) d -= (el(exy, i) - exi) * g.idx[1];
       half(nz, bz, i, d);
     }
+  }
+  if (S0) {
+    st4(S0 + q, ex);
+    st4(S1 + q, ey);
+    st4(S2 + q, ez);
   }
   st4(Nx + q, nx);
   st4(Ny + q, ny);
@@ -615,11 +632,13 @@ AntArgs antenna_args(const GridP &g, const LaserP *las, int nlas, const long lon
 }
 
 void launch_yee_b(const GridP &g, float *const B[3], float *const Bn[3], const float *const E[3], float h,
-                  unsigned long long *jfx, const PushArgs &a, const AntArgs &ant, const unsigned char *act, cudaStream_t s) {
+                  unsigned long long *jfx, const PushArgs &a, const AntArgs &ant, const unsigned char *act,
+                  float *const sE[3], cudaStream_t s) {
   const int nb = row_blocks4(g, 128);
+  float *s0 = sE ? sE[0] : nullptr, *s1 = sE ? sE[1] : nullptr, *s2 = sE ? sE[2] : nullptr;
 #define YEE_B(DD, AA)                                                                                               \
   k_yee_b<DD, AA><<<nb + ant.blocks, 128, 0, s>>>(g, B[0], B[1], B[2], Bn[0], Bn[1], Bn[2], E[0], E[1], E[2], h, jfx, \
-                                                  a.tile_n, a.tile_ctr, a.far_n, act, ant)
+                                                  a.tile_n, a.tile_ctr, a.far_n, act, s0, s1, s2, ant)
   if (ant.blocks) {
     if (g.D == 1) YEE_B(1, true);
     else if (g.D == 2) YEE_B(2, true);

@@ -325,7 +325,7 @@ int bp_create(const bp_grid_desc *gd, const bp_allocator *al, void *stream, bp_c
   }
   c->tile_ctr = (int *)dalloc(c, sizeof(int));
   c->tile_list = (int *)dalloc(c, sizeof(int) * g.ntiles);
-  c->tile_n = (int *)dalloc(c, sizeof(int));
+  c->tile_n = (int *)dalloc(c, 2 * sizeof(int));
   c->status = (int *)dalloc(c, sizeof(int) * 4);
   c->work = (unsigned long long *)dalloc(c, sizeof(unsigned long long) * 2);
   c->clk = (long long *)dalloc(c, sizeof(long long) * kClockWords);

@@ -135,7 +135,8 @@ struct PushArgs {
   unsigned char *qstate;   // [ntiles] what the quiet-tile pass left to the push
   unsigned long long *jfx; // [3][ncell] sorted deposit: the current in 64-bit fixed point (two's complement)
   int *tile_list;          // [ntiles] tiles the quiet-tile pass left for the push
-  int *tile_n;             // their number (cleared before the quiet-tile pass)
+  int *tile_n;             // their number (cleared before the quiet-tile pass); then the number of tiles with few
+                           // ions, which stand at the list's end (k_push_few)
   int *tile_ctr;           // the push's next list entry (cleared before each launch)
   int *status;
   float jscale, jinv;      // fixed-point scale (sorted deposit), power of two

@@ -34,10 +34,11 @@ __device__ __forceinline__ void make_loc(const int d[3], const float f[3], Loc &
 // one field component with stagger pattern PAT (bit a: half cell along a)
 // at two bodies; loads are shared when both stencils start at the same node
 // for every active lane of the warp (a warp-uniform choice: both forms give
-// the same sums, and a uniform branch keeps the warp from running both)
+// the same sums, and a uniform branch keeps the warp from running both).  rs:
+// row stride in 2D
 template <int D, int PAT>
 __device__ __forceinline__ void gather_comp(const float *__restrict__ G, const Loc &A, const Loc &Bo, float &oa,
-                                            float &ob) {
+                                            float &ob, int rs = Box<D>::GR) {
   int ba[3], bb[3];
   const float *wa[3];
   const float *wb[3];
@@ -60,7 +61,7 @@ __device__ __forceinline__ void gather_comp(const float *__restrict__ G, const L
       float pa = 0.0f, pb = 0.0f;
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
-        const float *row = G + Box<D>::gi(ba[0], ba[1] + j, ba[2] + k);
+        const float *row = G + (D == 2 ? ba[0] + rs * (ba[1] + j) : Box<D>::gi(ba[0], ba[1] + j, ba[2] + k));
         float ra = 0.0f, rb = 0.0f;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
@@ -80,8 +81,8 @@ __device__ __forceinline__ void gather_comp(const float *__restrict__ G, const L
       float pa = 0.0f, pb = 0.0f;
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
-        const float *ra_ = G + Box<D>::gi(ba[0], ba[1] + j, ba[2] + k);
-        const float *rb_ = G + Box<D>::gi(bb[0], bb[1] + j, bb[2] + k);
+        const float *ra_ = G + (D == 2 ? ba[0] + rs * (ba[1] + j) : Box<D>::gi(ba[0], ba[1] + j, ba[2] + k));
+        const float *rb_ = G + (D == 2 ? bb[0] + rs * (bb[1] + j) : Box<D>::gi(bb[0], bb[1] + j, bb[2] + k));
         float ra = 0.0f, rb = 0.0f;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
@@ -109,6 +110,18 @@ __device__ __forceinline__ void gather_all(const float *G, const Loc &A, const L
   gather_comp<D, 6>(G + 3 * gc, A, Bo, Ba[0], Bb[0]);
   gather_comp<D, 5>(G + 4 * gc, A, Bo, Ba[1], Bb[1]);
   gather_comp<D, 3>(G + 5 * gc, A, Bo, Ba[2], Bb[2]);
+}
+
+// the same from the global 2D fields: E and B at the box's origin, rows rs apart
+__device__ __forceinline__ void gather_all_few(const float *const E[3], const float *const B[3], long long at, int rs,
+                                               const Loc &A, const Loc &Bo, float Ea[3], float Ba[3], float Eb[3],
+                                               float Bb[3]) {
+  gather_comp<2, 1>(E[0] + at, A, Bo, Ea[0], Eb[0], rs);
+  gather_comp<2, 2>(E[1] + at, A, Bo, Ea[1], Eb[1], rs);
+  gather_comp<2, 4>(E[2] + at, A, Bo, Ea[2], Eb[2], rs);
+  gather_comp<2, 6>(B[0] + at, A, Bo, Ba[0], Bb[0], rs);
+  gather_comp<2, 5>(B[1] + at, A, Bo, Ba[1], Bb[1], rs);
+  gather_comp<2, 3>(B[2] + at, A, Bo, Ba[2], Bb[2], rs);
 }
 
 // ---------------------------------------------------------------------------

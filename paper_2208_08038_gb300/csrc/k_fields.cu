@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(128) k_yee_b(const __grid_constant__ GridP g, 
     block -= ant.blocks;
   }
   if (block == 0 && threadIdx.x == 0) {
-    *tile_n = 0;
+    tile_n[0] = tile_n[1] = 0;
     *tile_ctr = 0;
     if (far_n) *far_n = 0;
   }

@@ -7,6 +7,7 @@
 //   k_push_quiet  tiles whose neighbourhood never held a field (the field
 //                 kernels' tile marks): their co-moving neutral ions only
 //                 drift; the other tiles go on a list for the push,
+//   k_push_few    2D grids with few ions: the tiles with few, without a box,
 //   k_push        persistent blocks walk that list; per tile:
 //     1. stage E and B of the tile plus halo in shared memory (FP32, by
 //        asynchronous copies issued while the block finishes the previous
@@ -40,13 +41,28 @@ __host__ __device__ constexpr int push_threads(int D) { return D == 3 ? 512 : 25
 // and the blocks per SM its registers are held to (see k_push)
 __host__ __device__ constexpr int push_pb(int D, bool free_sp) { return D == 2 ? (free_sp ? 3 : 2) : 1; }
 
+// Where a deposit goes: the tile's box in shared memory, or (tiles with few
+// ions in 2D, sorted mode) straight to the global fixed-point current, whose row and
+// component strides are the grid's.
+template <int D>
+struct BoxStride {
+  static constexpr int row = Box<D>::J0, comp = Box<D>::JCELLS;
+};
+struct GridStride {
+  int row;
+  long long comp;
+};
+using fx64 = unsigned long long;  // a node of the global fixed-point current
+
 // add v (already in fixed-point units in the sorted mode) to a current node:
 // sorted mode, the exact fixed-point add fx_add (low words of the box, high
 // words 3 * JCELLS entries later); atomic mode, an FP32 shared atomic.  Zero
 // contributions are skipped where SKIP0.
 template <int D, bool DET, bool SKIP0 = true, typename JT>
 __device__ __forceinline__ void jput(JT *p, float v) {
-  if constexpr (DET) {
+  if constexpr (std::is_same<JT, fx64>::value) {
+    if (fabsf(v) > 0.5f) atomicAdd(p, (fx64)f2ll_rn(v));
+  } else if constexpr (DET) {
     if (SKIP0 && fabsf(v) <= 0.5f) return;
     fx_add(p, 3 * Box<D>::JCELLS, v);
   } else {
@@ -62,9 +78,14 @@ __device__ __forceinline__ void jadd(JT *p, float v, float scale) {
 
 // jput of a rows x cols block of nodes (the sorted mode's high words under one
 // branch)
-template <int D, bool DET, int R, int C, typename JT>
-__device__ __forceinline__ void jput_block(JT *p, const float (*v)[C]) {
-  if constexpr (DET) {
+template <int D, bool DET, int R, int C, typename JT, typename ST>
+__device__ __forceinline__ void jput_block(JT *p, const float (*v)[C], const ST &st) {
+  if constexpr (std::is_same<JT, fx64>::value) {
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+#pragma unroll
+      for (int i = 0; i < C; ++i) jput<D, DET>(p + (long long)st.row * j + i, v[j][i]);
+  } else if constexpr (DET) {
     fx_add_block<R, C>(p, Box<D>::J0, 3 * Box<D>::JCELLS, v);
   } else {
 #pragma unroll
@@ -86,11 +107,10 @@ __device__ __forceinline__ void jput_block(JT *p, const float (*v)[C]) {
 // carry the fixed-point scale (a power of two, so the products round
 // exactly as unscaled ones).  The two bodies' terms are added without FMA
 // contraction so that a neutral pair moving together cancels exactly.
-template <int D, bool DET, int NB, typename JT>
+template <int D, bool DET, int NB, typename JT, typename ST = BoxStride<D>>
 __device__ __forceinline__ void esirkepov3(JT *__restrict__ J, const int n[3], const float (*xi)[3],
                                            const float (*de)[3], const float *qw, const float (*v)[3],
-                                           const float dxdt[3], float scale) {
-  constexpr int jcells = Box<D>::JCELLS;
+                                           const float dxdt[3], float scale, const ST &st = ST()) {
   constexpr float K12 = 1.0f / 12.0f;
   const float sc = DET ? scale : 1.0f;
   float A[NB][3][3], DS[NB][3][3], DK[NB][3][3], cP[NB][3][2];
@@ -125,7 +145,7 @@ __device__ __forceinline__ void esirkepov3(JT *__restrict__ J, const int n[3], c
         cP[b][a][0] = cP[b][a][1] = 0.0f;
       }
     }
-  JT *Jx = J, *Jy = J + jcells, *Jz = J + 2 * jcells;
+  JT *Jx = J, *Jy = J + st.comp, *Jz = J + 2 * st.comp;
   const int bx = n[0] - 1, by = n[1] - 1, bz = n[2] - 1;
   if constexpr (D == 1) {
     float x[1][2], y[1][3], z[1][3], qy[NB], qz[NB];
@@ -134,7 +154,7 @@ __device__ __forceinline__ void esirkepov3(JT *__restrict__ J, const int n[3], c
       x[0][f] = cP[0][0][f];
       if constexpr (NB == 2) x[0][f] = __fadd_rn(x[0][f], cP[1][0][f]);
     }
-    jput_block<D, DET, 1, 2>(Jx + bx, x);
+    jput_block<D, DET, 1, 2>(Jx + bx, x, st);
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
       qy[b] = qw[b] * v[b][1] * sc;
@@ -149,8 +169,8 @@ __device__ __forceinline__ void esirkepov3(JT *__restrict__ J, const int n[3], c
         z[0][i] = __fadd_rn(z[0][i], __fmul_rn(qz[1], A[1][0][i]));
       }
     }
-    jput_block<D, DET, 1, 3>(Jy + bx, y);
-    jput_block<D, DET, 1, 3>(Jz + bx, z);
+    jput_block<D, DET, 1, 3>(Jy + bx, y, st);
+    jput_block<D, DET, 1, 3>(Jz + bx, z, st);
   } else if constexpr (D == 2) {
     float x[3][2], y[2][3], z[3][3], qz[NB];
 #pragma unroll
@@ -160,7 +180,7 @@ __device__ __forceinline__ void esirkepov3(JT *__restrict__ J, const int n[3], c
         x[j][f] = __fmul_rn(cP[0][0][f], A[0][1][j]);
         if constexpr (NB == 2) x[j][f] = __fadd_rn(x[j][f], __fmul_rn(cP[1][0][f], A[1][1][j]));
       }
-    jput_block<D, DET, 3, 2>(Jx + Box<D>::ji(bx, by, 0), x);
+    jput_block<D, DET, 3, 2>(Jx + (bx + (long long)st.row * by), x, st);
 #pragma unroll
     for (int g = 0; g < 2; ++g)
 #pragma unroll
@@ -168,7 +188,7 @@ __device__ __forceinline__ void esirkepov3(JT *__restrict__ J, const int n[3], c
         y[g][i] = __fmul_rn(cP[0][1][g], A[0][0][i]);
         if constexpr (NB == 2) y[g][i] = __fadd_rn(y[g][i], __fmul_rn(cP[1][1][g], A[1][0][i]));
       }
-    jput_block<D, DET, 2, 3>(Jy + Box<D>::ji(bx, by, 0), y);
+    jput_block<D, DET, 2, 3>(Jy + (bx + (long long)st.row * by), y, st);
 #pragma unroll
     for (int b = 0; b < NB; ++b) qz[b] = qw[b] * v[b][2] * sc;
 #pragma unroll
@@ -179,7 +199,7 @@ __device__ __forceinline__ void esirkepov3(JT *__restrict__ J, const int n[3], c
         if constexpr (NB == 2)
           z[j][i] = __fadd_rn(z[j][i], __fmul_rn(qz[1], fmaf(A[1][0][i], A[1][1][j], DK[1][0][i] * DS[1][1][j])));
       }
-    jput_block<D, DET, 3, 3>(Jz + Box<D>::ji(bx, by, 0), z);
+    jput_block<D, DET, 3, 3>(Jz + (bx + (long long)st.row * by), z, st);
   } else {
     // The outer loop of each pass stays rolled (its weights picked by
     // selects): the fully unrolled 54-node form is about three times the
@@ -463,12 +483,11 @@ __device__ __forceinline__ void deposit_general(JT *__restrict__ J, const int d[
 
 // an ion in 1D and 2D (rare: its bodies stay close to each other and slow), both
 // bodies one after the other, out of line
-template <int D, bool DET, typename JT>
+template <int D, bool DET, typename JT, typename ST = BoxStride<D>>
 __device__ __noinline__ void deposit_general_pair(JT *__restrict__ J, const int *d1, const int *d2, const float *f1,
                                                   const float *f2, const float *e1, const float *e2, float qw1,
                                                   float qw2, const float *v1, const float *v2, const float *dxdt,
-                                                  float scale) {
-  constexpr int jcells = Box<D>::JCELLS;
+                                                  float scale, const ST st = ST()) {
 #pragma unroll 1
   for (int b = 0; b < 2; ++b) {
     const float q = (b ? qw2 : qw1) * (DET ? scale : 1.0f);
@@ -482,16 +501,16 @@ __device__ __noinline__ void deposit_general_pair(JT *__restrict__ J, const int 
     }
     const PairAxis &X = G[0], &Y = G[1];
     const float qy = q * v[1], qz = q * v[2];
-    JT *p = J + Box<D>::ji(n0[0], n0[1], 0);
+    JT *p = J + (n0[0] + (long long)st.row * (D == 2 ? n0[1] : 0));
 #pragma unroll 1
-    for (int j = 0; j < (D == 2 ? 4 : 1); ++j, p += Box<D>::J0) {
+    for (int j = 0; j < (D == 2 ? 4 : 1); ++j, p += st.row) {
       const float sy = D == 2 ? sel4(j, Y.S) : 1.0f, dy = D == 2 ? sel4(j, Y.DS) : 0.0f, py = D == 2 ? sel4(j, Y.P) : 0.0f;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const float fx = pair_factor(X.S[i], X.DS[i], 1.0f, 0.0f);
         jput<D, DET>(p + i, X.P[i] * pair_factor(sy, dy, 1.0f, 0.0f));
-        jput<D, DET>(p + jcells + i, D == 2 ? py * fx : qy * fx);
-        jput<D, DET>(p + 2 * jcells + i, qz * pair_factor(X.S[i], X.DS[i], sy, dy));
+        jput<D, DET>(p + st.comp + i, D == 2 ? py * fx : qy * fx);
+        jput<D, DET>(p + 2 * st.comp + i, qz * pair_factor(X.S[i], X.DS[i], sy, dy));
       }
     }
   }
@@ -977,10 +996,14 @@ __device__ __forceinline__ bool push_far(const GridP &g, const SpecP &sp, const 
   return true;
 }
 
-template <int D, bool DET, bool FREE, typename JT>
+// JT fx64: fields and current are the global arrays (A.E, A.B at `at`; Jsm the
+// current at the box's origin, strides st)
+template <int D, bool DET, bool FREE, typename JT, typename ST = BoxStride<D>>
 __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, long long i, const int T0[3],
                               const float *Gsm, JT *Jsm, int *status, float scale, unsigned &blo, unsigned &bhi,
-                              PairJob *jobs, bool nofield, int4 *far, int *far_n, int far_cap, int s, int t) {
+                              PairJob *jobs, bool nofield, int4 *far, int *far_n, int far_cap, int s, int t,
+                              const PushArgs *A = nullptr, long long at = 0, const ST &st = ST()) {
+  constexpr bool GLOBAL = std::is_same<JT, fx64>::value;
   const long long cap = P.cap;
   const bool two = sp.kind == BP_TWO_BODY;
   int cell = P.cell[i];
@@ -1052,7 +1075,8 @@ __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, l
       Loc L1, L2;
       make_loc<D>(d, f, L1);
       make_loc<D>(two ? d2 : d, two ? f2 : f, L2);
-      gather_all<D>(Gsm, L1, L2, E1, B1, E2, B2);
+      if constexpr (GLOBAL) gather_all_few(A->E, A->B, at, st.row, L1, L2, E1, B1, E2, B2);
+      else gather_all<D>(Gsm, L1, L2, E1, B1, E2, B2);
     }
   }
   float v1[3], v2[3] = {0.0f, 0.0f, 0.0f};
@@ -1166,8 +1190,8 @@ __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, l
       if constexpr (D == 3 && DET) {
         if (two) esirkepov3_p3(Jsm, nn, xi, dd, qw, dxdt, scale);
         else esirkepov3<D, DET, 1>(Jsm, nn, xi, dd, qw, vv, dxdt, scale);
-      } else if (two) esirkepov3<D, DET, 2>(Jsm, nn, xi, dd, qw, vv, dxdt, scale);
-      else esirkepov3<D, DET, 1>(Jsm, nn, xi, dd, qw, vv, dxdt, scale);
+      } else if (two) esirkepov3<D, DET, 2>(Jsm, nn, xi, dd, qw, vv, dxdt, scale, st);
+      else esirkepov3<D, DET, 1>(Jsm, nn, xi, dd, qw, vv, dxdt, scale, st);
       bb_add<D>(blo, bhi, nn, 1, 1);
     } else {
       if constexpr (D == 2 && FREE) {
@@ -1198,7 +1222,7 @@ __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, l
             dd[a] = dxdt[a];
           }
           deposit_general_pair<D, DET, JT>(Jsm, cb[0], cb[1], fb[0], fb[1], db[0], db[1], sp.qw1, sp.qw2, vb[0], vb[1], dd,
-                                           scale);
+                                           scale, st);
         } else if constexpr (D == 1) {
           deposit_general<D, DET, JT>(Jsm, d, f, de1, sp.qw1, v1, dxdt, scale);
         }
@@ -1298,8 +1322,29 @@ __device__ __forceinline__ bool near_mark(const GridP &g, int t, int lane) {
   return use && g.fnz[nb[0] + g.nt[0] * (nb[1] + g.nt[1] * nb[2])] != 0;
 }
 
+// Tiles of at most FEW ions go to k_push_few when their boxes lie within the
+// grid (no wrap, no open face to look out for).  1024 x 1024 cells, ions at
+// random places, step by box and from the global arrays: 133 and 71 us with 8
+// ions a tile, 149 and 93 with 48, 154 and 104 with 64, 172 and 139 with 128;
+// but ions that sit close together add to the same nodes, one after the other
+// in L2 (128 a tile in 4 x 4 cells: 303 us a step, 312), so it stops at 64.
+constexpr int FEW = 64;
 template <int D>
-__global__ void __launch_bounds__(128, 8) k_push_quiet(const __grid_constant__ GridP g, PushArgs A, int qt,
+__device__ __forceinline__ bool box_inside(const GridP &g, int t) {
+  const int tc[3] = {t % g.nt[0], (t / g.nt[0]) % g.nt[1], t / (g.nt[0] * g.nt[1])};
+  using BX = Box<D>;
+  constexpr int L[3] = {Geo<D>::L0, Geo<D>::L1, Geo<D>::L2}, GN[3] = {BX::G0, BX::G1, BX::G2}, JN[3] = {BX::J0, BX::J1, BX::J2};
+  bool in = true;
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    const int x = tc[a] * L[a];
+    in &= x >= BX::OG && x - BX::OG + GN[a] <= g.n[a] && x >= BX::OJ && x - BX::OJ + JN[a] <= g.n[a];
+  }
+  return in;
+}
+
+template <int D>
+__global__ void __launch_bounds__(128, 8) k_push_quiet(const __grid_constant__ GridP g, PushArgs A, int qt, int few,
                                                        const __grid_constant__ AntArgs ant) {
   static_assert(Box<D>::OG <= Geo<D>::L0 && Box<D>::G0 - Box<D>::OG <= 2 * Geo<D>::L0 &&
                     (D < 2 || (Box<D>::OG <= Geo<D>::L1 && Box<D>::G1 - Box<D>::OG <= 2 * Geo<D>::L1)) &&
@@ -1320,14 +1365,16 @@ __global__ void __launch_bounds__(128, 8) k_push_quiet(const __grid_constant__ G
   const int t = ((int)blockIdx.x - ant.blocks) * qt + warp;
   if (tid == 0) nquiet = 0;
   bool marked = false, occupied = false;
+  int ions = 0;
   if (warp < qt && t < g.ntiles) {
     marked = near_mark<D>(g, t, lane);
     // a tile without particles has nothing to push or deposit, whatever its
     // fields: done here, so the push neither stages its fields nor visits it
-    if (lane < A.nsp) occupied = A.p[lane].tstart[t + 1] > A.p[lane].tstart[t];
+    if (lane < A.nsp) ions = A.p[lane].tstart[t + 1] - A.p[lane].tstart[t];
   }
   marked = __any_sync(0xFFFFFFFFu, marked);
-  occupied = __any_sync(0xFFFFFFFFu, occupied);
+  ions = __reduce_add_sync(0xFFFFFFFFu, ions);
+  occupied = ions > 0;
   __syncthreads();  // nquiet cleared
   if (warp < qt && t < g.ntiles && lane == 0) {
     if (!occupied) {
@@ -1335,7 +1382,8 @@ __global__ void __launch_bounds__(128, 8) k_push_quiet(const __grid_constant__ G
       A.occ[t] = 0;
     } else if (marked) {
       A.qstate[t] = QS_PUSH;
-      A.tile_list[atomicAdd(A.tile_n, 1)] = t;
+      if (few && ions <= FEW && box_inside<D>(g, t)) A.tile_list[g.ntiles - 1 - atomicAdd(A.tile_n + 1, 1)] = t;
+      else A.tile_list[atomicAdd(A.tile_n, 1)] = t;
     } else {
       quiet[atomicAdd(&nquiet, 1)] = t;  // each quiet tile is drifted alone: their order changes nothing
     }
@@ -1764,6 +1812,37 @@ __global__ void __launch_bounds__(push_threads(D), PB) k_push(GridP g, PushArgs 
   if (next >= 0 && qs == QS_PUSH) stage_done<D>(g, A, T, next, qs, &bar, phase, failed);
 }
 
+// 2D, sorted mode: the tiles with few ions, a warp each and a lane per ion,
+// straight from the global fields to the global current, in the arithmetic of
+// the tile push (the current's integer adds give the same bits in any order).
+// Bound by the chain of one ion's gather, push and deposit; for a few ions the
+// box push adds the staging of 2,400 field values, the clearing of the current
+// box and its flush, with two blocks per SM: the 1,600 ions of a Bragg crystal
+// on 2048 x 2048 cells, step 233 us before, 160 after.
+__global__ void __launch_bounds__(128, 4) k_push_few(GridP g, PushArgs A) {
+  using BX = Box<2>;
+  const int lane = threadIdx.x & 31, n = A.tile_n[1];
+  const GridStride st = {g.n[0], (long long)g.ncell};
+  unsigned pushed = 0;
+  for (int k = (int)(blockIdx.x * 4 + (threadIdx.x >> 5)); k < n; k += (int)gridDim.x * 4) {
+    const int t = A.tile_list[g.ntiles - 1 - k];
+    const int T0[3] = {(t % g.nt[0]) * Geo<2>::L0, (t / g.nt[0]) * Geo<2>::L1, 0};
+    const long long at = (T0[0] - BX::OG) + (long long)g.n[0] * (T0[1] - BX::OG);
+    fx64 *J = A.jfx + ((T0[0] - BX::OJ) + (long long)g.n[0] * (T0[1] - BX::OJ));
+    for (int s = 0; s < A.nsp; ++s) {
+      const int end = A.p[s].tstart[t + 1];
+      for (int i = A.p[s].tstart[t] + lane; i < end; i += 32) {
+        unsigned blo = 0xFFFFFFFFu, bhi = 0u;
+        push_particle<2, true, false, fx64, GridStride>(g, A.sp[s], A.p[s], i, T0, nullptr, J, A.status, A.jscale, blo, bhi,
+                                                        nullptr, false, A.far, A.far_n, A.far_cap, s, t, &A, at, st);
+        ++pushed;
+      }
+      __syncwarp();
+    }
+  }
+  if (A.work) count_work(A.work, pushed);
+}
+
 // Sorted mode: the ions the push listed as far (a bound electron a cell or
 // more from its nucleus), each moved by push_far; anything push_far cannot
 // move is a domain error.
@@ -1798,12 +1877,26 @@ int push_variant(const GridP &g, const PushArgs &a) {
   return g.D == 2 && free_sp ? 1 : 0;
 }
 
+// Whether a 2D step launches k_push_few: two-body ions only, less than 8 a tile
+// on average.  Where no tile has few ions the launch is lost (a dense slab in a
+// wide grid, 16 ions a tile on average: adjoint cycle 53.4 ms without it, 55.1
+// with), and the host knows no more of the tiles than the average.
+bool push_few(const GridP &g, const PushArgs &a) {
+  if (push_variant(g, a)) return false;
+  long long ions = 0;
+  for (int k = 0; k < a.nsp; ++k) ions += a.p[k].cap;
+  return ions < 8LL * g.ntiles;
+}
+
 template <int D, bool DET>
 void launch_one(const GridP &g, const PushArgs &a, const TmaMaps &tm, const AntArgs &ant, cudaStream_t s) {
   const bool direct = push_direct(g, a);
   if (!direct) {
     const int qt = g.ntiles >= 8192 ? 4 : 1;  // tiles per quiet-pass block
-    k_push_quiet<D><<<(g.ntiles + qt - 1) / qt + ant.blocks, 128, 0, s>>>(g, a, qt, ant);
+    const bool few = D == 2 && DET && push_few(g, a);
+    k_push_quiet<D><<<(g.ntiles + qt - 1) / qt + ant.blocks, 128, 0, s>>>(g, a, qt, few, ant);
+    if constexpr (D == 2 && DET)
+      if (few) k_push_few<<<a.sms * 4, 128, 0, s>>>(g, a);
   }
   const size_t smem = push_smem_bytes(g, DET);
   // as many persistent blocks as the device holds at once (worked out per

@@ -85,6 +85,12 @@ int check_launch(bp_ctx *c, const char *what) {
 // A node of a tile box then holds the exact sum of up to 2^26 such maximal
 // contributions, and a quantum is about 1e-11 of the largest one (below the
 // FP32 rounding of the contributions themselves).
+// every tile updated, and its current cleared and formed, until the next push
+// recomputes the flags
+void reset_active(bp_ctx *c) {
+  if (c->act) cudaMemsetAsync(c->act, ACT_ALL, (size_t)c->g.ntiles, c->stream);
+}
+
 // the tile marks of the push's field-box test, recomputed from E and B
 // after they were written from outside the step (state file, caller,
 // checkpoint)
@@ -92,8 +98,7 @@ void refresh_marks(bp_ctx *c) {
   const float *F[6] = {c->F[0], c->F[1], c->F[2], c->F[3], c->F[4], c->F[5]};
   launch_field_marks(c->g, F, c->stream);
   c->launches += 1;
-  // every tile active until the next push recomputes the flags
-  if (c->act) cudaMemsetAsync(c->act, 1, (size_t)c->g.ntiles, c->stream);
+  reset_active(c);
 }
 
 void update_jscale(bp_ctx *c) {
@@ -321,7 +326,7 @@ int bp_create(const bp_grid_desc *gd, const bp_allocator *al, void *stream, bp_c
   if (g.ntiles >= 1024) {
     c->act = (unsigned char *)dalloc(c, g.ntiles);
     c->act_n = (unsigned long long *)dalloc(c, 2 * sizeof(unsigned long long));
-    if (c->act) cudaMemsetAsync(c->act, 1, (size_t)g.ntiles, c->stream);
+    reset_active(c);
   }
   c->tile_ctr = (int *)dalloc(c, sizeof(int));
   c->tile_list = (int *)dalloc(c, sizeof(int) * g.ntiles);
@@ -1035,6 +1040,7 @@ int bp_write_field(bp_ctx *c, int comp, const float *src, int on_device) {
   cudaError_t e = cudaMemcpyAsync(c->F[comp], src, sizeof(float) * c->g.ncell,
                                   on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess && comp < 6) refresh_marks(c);
+  else if (e == cudaSuccess) reset_active(c);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   return e == cudaSuccess ? BP_OK : cuda_fail(c, e, "write field");
 }
@@ -1507,7 +1513,7 @@ int bp_reset(bp_ctx *c) {
   cudaStream_t st = c->stream;
   for (int k = 0; k < 9; ++k) cudaMemsetAsync(c->F[k], 0, sizeof(float) * c->g.ncell, st);
   cudaMemsetAsync(c->g.fnz, 0, (size_t)c->g.ntiles, st);
-  if (c->act) cudaMemsetAsync(c->act, 1, (size_t)c->g.ntiles, st);
+  reset_active(c);
   if (c->jfx) cudaMemsetAsync(c->jfx, 0, sizeof(unsigned long long) * 3 * (size_t)c->g.ncell, st);
   cudaMemsetAsync(c->status, 0, sizeof(int) * 4, st);
   c->step = 0;

@@ -123,6 +123,14 @@ struct PartP {
   long long cap;
 };
 
+// What the field kernels do in a tile (tile_active):
+//   ACT_ON     E and B are updated,
+//   ACT_J      the step's deposits or antennas can reach the tile,
+//   ACT_CLEAR  they cannot, but the J of an earlier step is to be zeroed,
+//   ACT_STALE  not updated; an earlier step's J stands.
+// Before the first step and after a write from outside: ACT_ON | ACT_J.
+constexpr unsigned char ACT_ON = 1, ACT_J = 2, ACT_CLEAR = 4, ACT_STALE = 8, ACT_ALL = ACT_ON | ACT_J;
+
 struct PushArgs {
   int nsp;
   SpecP sp[BP_MAX_SPECIES];
@@ -144,7 +152,7 @@ struct PushArgs {
   int4 *far;                // sorted deposit: two-body ions whose bound electron is a cell or more away,
   int *far_n;               //   (species, particle, tile), moved after the push by k_push_far; their count
   int far_cap;
-  unsigned char *act;       // [ntiles] tiles the field kernels update this step (null: all), set by k_push_far
+  unsigned char *act;       // [ntiles] ACT_* flags of a step (null: every tile is updated with its current), set by k_push_far
   unsigned long long *act_n; // their number, summed over the steps; the steps
   int ia_lo, ia_hi;         // the antenna planes' x range
   int push_blocks[2];       // persistent push blocks for this grid on this device (see push_prepare)

@@ -93,7 +93,8 @@ __global__ void __launch_bounds__(128) k_yee_b(const __grid_constant__ GridP g, 
   Cell4 C;
   if (!row_cell4<D>(g, C, block)) return;
   const long long q = C.q;
-  if (act && !act[tile_of(g, C.c)]) {  // E and B zero around the tile: B stays zero
+  const unsigned char on = act ? act[tile_of(g, C.c)] : ACT_ALL;
+  if (!(on & ACT_ON)) {  // E and B zero around the tile: B stays zero
     if (S0) {
       const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       st4(S0 + q, z);
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(128) k_yee_b(const __grid_constant__ GridP g, 
   st4(Bx + q, bx);
   st4(By + q, by);
   st4(Bz + q, bz);
-  if (jfx) {
+  if (jfx && (on & ACT_J)) {
     const ulonglong2 z = make_ulonglong2(0ull, 0ull);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -221,10 +222,18 @@ __global__ void __launch_bounds__(128) k_yee_e(GridP g, float *Ex, float *Ey, fl
   if (blockIdx.x == 0 && threadIdx.x == 0) clk[0] += 1;
   Cell4 C;
   if (!row_cell4<D>(g, C)) return;
-  if (act && !act[tile_of(g, C.c)]) return;  // no field and no current around the tile: E stays zero
+  const unsigned char on = act ? act[tile_of(g, C.c)] : ACT_ALL;
+  if (!(on & ACT_ON)) return;  // no field and no current around the tile: E stays zero
   const long long q = C.q;
   float4 jx, jy, jz;
-  if constexpr (FX) {
+  if (FX && !(on & ACT_J)) {
+    jx = jy = jz = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (on & ACT_CLEAR) {
+      st4(Jx + q, jx);
+      st4(Jy + q, jy);
+      st4(Jz + q, jz);
+    }
+  } else if constexpr (FX) {
     const long long nc = g.ncell;
     const ulonglong2 *px = reinterpret_cast<const ulonglong2 *>(jfx + q);
     const ulonglong2 *py = reinterpret_cast<const ulonglong2 *>(jfx + nc + q);

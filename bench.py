@@ -213,7 +213,7 @@ def run_e2e(wl, n_ion, mode, steps, rank, world, dist=None):
                     "copy overlapping the next steps); context creation included"}
 
 
-BRAGG_BYTES_CELL = 168  # per cell and step: 2 B half steps (36 B), E step (72 B), clearing the current (24 B)
+BRAGG_BYTES_CELL = 84  # per cell and step: both B half steps 48 B, E step 36 B (near ions 60 B more for the current)
 
 
 def updated_cells(act_tiles, act_steps, ncell, ntiles, steps):
@@ -298,8 +298,8 @@ def run_neutral_1d(steps, warmup):
             "steps": f"{warmup}..{warmup + steps}", "ms_per_step": ms / steps,
             "ion_pushes_per_s": len(sp.x) * steps / (ms * 1e-3), "push_ms_per_launch": push_ms / max(push_n, 1),
             "gpu_launches_per_step": launches / steps, "ms_per_step_launched_directly": ms_direct / steps,
-            "bound": "kernel launches (a few microseconds of work per kernel): each step is one graph "
-                     "launch (the conditional re-sort, then the step's kernels)"}
+            "bound": "kernel launches (a few microseconds of work per kernel): eight steps are one "
+                     "graph launch"}
 
 
 def run_adjoint_ratio(steps=400, K=20, reps=3):
@@ -383,7 +383,7 @@ def fp32_peak_tflops(sm_mhz, sms=None):
 
 
 def push_roofline(full, quiet, launches, push_ms, ncell, hbm, hbm_src, sm_max, sms=None):
-    """Roofline of the push launch (k_push_quiet + k_push + k_records) over a
+    """Roofline of the push launch (k_push_quiet + k_push + k_push_far) over a
     timed window: `full` and `quiet` are the device-counted full pushes and
     quiet drifts of the window's `launches` push launches, `push_ms` their
     summed CUDA-event time.  FP32 operations (the binding roof) from the full
@@ -402,7 +402,7 @@ def push_roofline(full, quiet, launches, push_ms, ncell, hbm, hbm_src, sm_max, s
         traffic = (full * TRAFFIC_FULL_ION + quiet * TRAFFIC_QUIET_ION) / per
     return {"bound": "alu", "achieved": achieved_tf, "peak": fp32_peak, "unit": "TFLOP/s",
             "frac": achieved_tf / fp32_peak, "traffic": traffic, "traffic_unit": "bytes per launch",
-            "window": "late", "kernel": "push launch: k_push_quiet<3> + k_push<3,sorted> + k_records<3>",
+            "window": "late", "kernel": "push launch: k_push_quiet<3> + k_push<3,sorted> + k_push_far<3>",
             "peak_source": f"FP32 lanes: {sms} SMs x 128 x 2 flops x {sm_max:.0f} MHz (max SM clock)",
             "flops_per_full_push": FLOPS_FULL_ION,
             "limiter": "instruction issue (ncu on the small 3D case with a field in every tile)",
@@ -413,7 +413,7 @@ def push_roofline(full, quiet, launches, push_ms, ncell, hbm, hbm_src, sm_max, s
 def timed_window(ctx, steps, stream, time_push=True):
     """CUDA-event time of `steps` steps, with the push launches timed and
     their work counted on the device (time_push); without push timing the
-    steps replay the library's graph of a step."""
+    steps replay the library's graphs of the step."""
     import torch
     ctx.time_push(time_push)
     launches0 = ctx.kernel_launches()

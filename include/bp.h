@@ -192,9 +192,10 @@ int bp_add_probe(bp_ctx *ctx, int comp, const int64_t *nodes, int64_t npts, int6
  * Sec. 3.1 -- Maxwell's equations with the vacuum permittivity.  Returns
  * BP_ERR_ARG for n_steps < 0; kernel problems (a particle off its tile's
  * reach, a non-finite momentum) surface at the next bp_sync.  With two or
- * more steps and push timing off, the steps replay a CUDA graph of one step
- * (captured on first use and again whenever a launch argument has changed:
- * particle arrays, lasers, probes, parameters); single steps and timed steps
+ * more steps and push timing off, the steps replay CUDA graphs of eight steps
+ * and of one (captured on first use and again whenever a launch argument has
+ * changed: particle arrays, lasers, probes, parameters); so do single steps
+ * from the third such call in a row.  Other single steps and timed steps
  * launch the same kernels directly, with the same results bit for bit. */
 int bp_step(bp_ctx *ctx, int64_t n_steps);
 
@@ -366,7 +367,7 @@ int64_t bp_kernel_launches(const bp_ctx *ctx);
 
 /* Per-kernel CUDA-event timing of the push/deposit launches: when enabled,
  * bp_step records events around each push launch (and launches directly,
- * not through the step graph); bp_push_time returns
+ * not through the step graphs); bp_push_time returns
  * the summed milliseconds and launch count since the last reset (bp_time_push
  * resets both, and the work counters of bp_push_work).  (The paper has no
  * counterpart; instrumentation.) */
@@ -384,7 +385,8 @@ int bp_push_work(bp_ctx *ctx, int64_t *full, int64_t *quiet);
 /* Work of the field updates since the last call: *active_tiles receives the
  * tiles the field kernels updated, summed over the steps (on grids of 1024
  * tiles or more they skip tiles whose neighbourhood has never held a field
- * and receives no current: their E, B and J stay exactly zero), *steps the
+ * and receives no current: their E, B and J stay exactly zero; in the tiles
+ * they update, J is formed where a deposit can reach), *steps the
  * steps counted; the count restarts at zero.  Smaller grids update every
  * tile and count nothing.  Synchronous.  (The paper has no counterpart;
  * instrumentation.) */

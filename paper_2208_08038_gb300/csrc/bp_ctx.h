@@ -114,9 +114,9 @@ struct bp_ctx {
   std::string err;
   float jscale = 0.0f, jinv = 0.0f;
   bp_adjoint adj;
-  cudaStream_t cap_stream = nullptr;  // captures the step graph
-  // the step clock (device; see kClockWords) and the graph of a step's
-  // launches, with the launch arguments it was captured
+  cudaStream_t cap_stream = nullptr;  // captures the step graphs
+  // the step clock (device; see kClockWords) and the graphs of the step's
+  // launches, with the launch arguments they were captured
   // with (rebuilt when any of them changes)
   long long *clk = nullptr;
   cudaGraphExec_t step_exec = nullptr;

@@ -3,18 +3,21 @@
 //
 // Each forward operator is replaced by its transpose or vector-Jacobian
 // product, applied in reverse order:
-//   E^{n+1} = E^n + dt (curl B^{n+1/2} - J) with Mur faces  ->  k_adj_mur (last
-//       pass first) + k_adj_e (gathers curl^T of the interior adjoint, J adjoint)
+//   E^{n+1} = E^n + dt (curl B^{n+1/2} - J) with Mur faces  ->  k_adj_ex
+//       (open faces on x alone or none: the faces themselves go with the next
+//       k_adj_b), else k_adj_mur (last pass first) + k_adj_e; both gather
+//       curl^T of the interior adjoint and form the J adjoint
 //   B^{n+1/2} = B^n - dt/2 curl E^n                          ->  k_adj_b
 //   per particle: Esirkepov deposit, drift, Boris, internal modified-Coulomb
-//       field (arXiv 2208.08038 Sec. 2), gather              ->  k_adj_work
-//       (the step's list of 256-ion chunks of the occupied tiles), k_adj_push
+//       field (arXiv 2208.08038 Sec. 2), gather              ->  a list
+//       of 256-ion chunks of the occupied tiles (made by k_adj_ex, or by
+//       k_adj_work beside k_adj_e), k_adj_push
 //       (recompute of the push; the deposit's transpose reads the current
 //       adjoint like a gather; Boris, force and drift transposes; the
 //       gather's position derivatives; stores each ion's gathered-field
 //       adjoints), k_adj_scatter (the gather's transpose: those adjoints
-//       scattered like a deposit into a 64-bit fixed-point box per chunk,
-//       added into a per-cell accumulator), k_adj_fxsum (the accumulator
+//       scattered like a deposit into a 64-bit fixed-point box per run of a
+//       tile's chunks, added into a per-cell accumulator), k_adj_fxsum (the accumulator
 //       converted once and added to the field adjoints, then cleared)
 //   B^n = B^{n-1/2} - dt/2 curl E^n                          ->  k_adj_b
 // The particle adjoints are indexed by load order, so re-sorting between

@@ -1,6 +1,7 @@
 // k_sort.cu -- integer work: the counting sort of particles by tile-major cell
-// (key = tile * cells_per_tile + cell within tile), run only when the device
-// status word says a particle left its tile's margin; the seeded device-side
+// (key = tile * cells_per_tile + cell within tile) as one cooperative kernel,
+// which does its work only when the device status word says a particle left
+// its tile's margin; the seeded device-side
 // medium generator; and the FP64 Gauss-law residual.
 #include <cstring>
 

@@ -201,8 +201,11 @@ int bp_step(bp_ctx *ctx, int64_t n_steps);
 
 /* Wait for the stream and return the device status word as a bp_status:
  * BP_ERR_DOMAIN, BP_ERR_NONFINITE or BP_ERR_TIMEOUT from the kernels,
- * BP_ERR_CUDA for a failed CUDA call.  (The paper has no counterpart:
- * completion and error reporting of this interface.) */
+ * BP_ERR_CUDA for a failed CUDA call.  After BP_ERR_TIMEOUT the particles may
+ * be half sorted (also those of a load just made): no later step sorts or
+ * pushes them, bp_load_particles and bp_set_lattice return the same error,
+ * and bp_reset makes the context usable again.  (The paper has no
+ * counterpart: completion and error reporting of this interface.) */
 int bp_sync(bp_ctx *ctx);
 
 /* Copy field component comp (nz*ny*nx floats, x fastest) to dst: a device
@@ -399,6 +402,13 @@ int bp_field_work(bp_ctx *ctx, int64_t *active_tiles, int64_t *steps);
  * it, sizes nothing.  BP_OK for n >= 0 on a context in the sorted mode, else
  * BP_ERR_ARG. */
 int bp_set_record_capacity(bp_ctx *ctx, int64_t n);
+
+/* How often a block of the particle sort polls its grid barrier before it
+ * gives up (BP_ERR_TIMEOUT): 0 gives up at once, a negative number restores
+ * the default (some ten seconds).  Takes effect at the next launch.  (The
+ * paper has no counterpart: a limit of this implementation, settable so that
+ * a program can provoke the error and test how it recovers.) */
+int bp_set_sort_wait(bp_ctx *ctx, int64_t polls);
 
 #ifdef __cplusplus
 }

@@ -93,6 +93,7 @@ _SIGS = {
     "bp_kernel_launches": (_i64, [_p]),
     "bp_time_push": (_i, [_p, _i]),
     "bp_set_record_capacity": (_i, [_p, C.c_int64]),
+    "bp_set_sort_wait": (_i, [_p, C.c_int64]),
     "bp_read_field_async": (_i, [_p, _i, _p]),
     "bp_push_time": (_i, [_p, C.POINTER(_d), C.POINTER(_i64)]),
     "bp_push_work": (_i, [_p, C.POINTER(_i64), C.POINTER(_i64)]),
@@ -369,6 +370,10 @@ class Context:
 
     def set_record_capacity(self, n: int):
         self._check(self._L.bp_set_record_capacity(self._h, int(n)), "bp_set_record_capacity")
+
+    def set_sort_wait(self, polls: int):
+        """Polls of the sort's grid barrier before it gives up (negative: the default)."""
+        self._check(self._L.bp_set_sort_wait(self._h, int(polls)), "bp_set_sort_wait")
 
     def time_push(self, enable: bool):
         self._check(self._L.bp_time_push(self._h, int(enable)), "bp_time_push")

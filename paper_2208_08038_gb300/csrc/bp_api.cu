@@ -204,6 +204,13 @@ int initial_sort(bp_ctx *c, Species &s, long long n) {
   return check_launch(c, "initial sort");
 }
 
+// the sort's barrier and histogram as they are between two sorts (a sort that
+// gave up leaves neither so)
+void clear_sort(bp_ctx *c) {
+  cudaMemsetAsync(c->sb.bar, 0, sizeof(unsigned) * 2, c->stream);
+  if (c->sb.hist) cudaMemsetAsync(c->sb.hist, 0, sizeof(int) * (c->g.ncell + 1), c->stream);
+}
+
 }  // namespace
 
 extern "C" {
@@ -348,6 +355,7 @@ int bp_create(const bp_grid_desc *gd, const bp_allocator *al, void *stream, bp_c
   cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
   if (c->sms < 1) c->sms = 1;
   c->sb.blocks = sort_blocks(c->sms);
+  c->sb.polls = kSortPolls;
   c->sb.bar = (unsigned *)dalloc(c, sizeof(unsigned) * 2);
   if (!c->sb.bar) {
     bp_destroy(c);
@@ -466,8 +474,10 @@ int finish_load(bp_ctx *c, Species &s, long long n, void *stage) {
   cudaError_t e = cudaStreamSynchronize(st);
   dfree(c, stage);
   if (e != cudaSuccess) return cuda_fail(c, e, "load");
-  int stw = 0;
-  cudaMemcpy(&stw, c->status, sizeof(int), cudaMemcpyDeviceToHost);
+  int sw[3] = {0, 0, 0};
+  cudaMemcpy(sw, c->status, sizeof sw, cudaMemcpyDeviceToHost);
+  const int stw = sw[0];
+  if (sw[2]) return fail(c, BP_ERR_TIMEOUT, "an earlier device wait timed out (bp_reset first)");
   if (stw & ST_NONFINITE) return fail(c, BP_ERR_NONFINITE, "non-finite position or momentum in the load");
   if (stw & ST_DOMAIN) return fail(c, BP_ERR_DOMAIN, "a particle lies outside the grid or has a bad param_idx");
   int rc = initial_sort(c, s, n);
@@ -989,9 +999,10 @@ int bp_sync(bp_ctx *c) {
     }
     c->ev_used = 0;
   }
-  int st = 0;
-  e = cudaMemcpy(&st, c->status, sizeof(int), cudaMemcpyDeviceToHost);
+  int sw[3] = {0, 0, 0};
+  e = cudaMemcpy(sw, c->status, sizeof sw, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(c, e, "status");
+  const int st = sw[0] | (sw[2] ? ST_TIMEOUT : 0);
   if (st & ST_NONFINITE) return fail(c, BP_ERR_NONFINITE, "non-finite momentum");
   if (st & ST_DOMAIN) return fail(c, BP_ERR_DOMAIN, "a two-body ion left the region its tile handles or the grid");
   if (st & ST_TIMEOUT) return fail(c, BP_ERR_TIMEOUT, "device wait timed out");
@@ -1411,6 +1422,7 @@ int bp_load(bp_ctx *c, const char *path) {
   bool ok = true;
   for (int k = 0; k < 6; ++k) ok = ok && rd_dev(f, c->F[k], sizeof(float) * g.ncell);
   cudaMemset(c->status, 0, sizeof(int) * 4);
+  clear_sort(c);
   ok = ok && rd_dev(f, c->status, sizeof(int));
   fclose(f);
   if (!ok) return fail(c, BP_ERR_IO, "bp_load: truncated fields (%s)", path);
@@ -1457,6 +1469,12 @@ int64_t bp_kernel_launches(const bp_ctx *c) {
 int bp_set_record_capacity(bp_ctx *c, int64_t n) {
   if (!c || n < 0 || !c->det) return BP_ERR_ARG;
   return BP_OK;  // no particle leaves a record any more: nothing to size
+}
+
+int bp_set_sort_wait(bp_ctx *c, int64_t polls) {
+  if (!c) return BP_ERR_ARG;
+  c->sb.polls = polls < 0 || polls > kSortPolls ? kSortPolls : (int)polls;
+  return BP_OK;
 }
 
 int bp_time_push(bp_ctx *c, int enable) {
@@ -1516,6 +1534,7 @@ int bp_reset(bp_ctx *c) {
   reset_active(c);
   if (c->jfx) cudaMemsetAsync(c->jfx, 0, sizeof(unsigned long long) * 3 * (size_t)c->g.ncell, st);
   cudaMemsetAsync(c->status, 0, sizeof(int) * 4, st);
+  clear_sort(c);
   c->step = 0;
   for (auto &p : c->pr) p.count = 0;
   for (auto &s : c->sp) s.loaded = false;
@@ -1741,7 +1760,7 @@ int bp_backward(bp_ctx *c, int probe_id, const float *dl_dprobe, int sid, double
     for (int f = 0; f < 6; ++f) cl_add(c, L, ad.ck_fields[seg] + (size_t)f * g.ncell, c->F[f], sizeof(float) * g.ncell);
     for (size_t q = 0; q < c->sp.size(); ++q)
       cl_parts(c, L, ad.ck_parts[seg][q].p, c->sp[q].p, g.D, c->sp[q].sp.kind == BP_TWO_BODY);
-    cl_add(c, L, ad.ck_status + 4 * seg, c->status, sizeof(int) * 4);
+    cl_add(c, L, ad.ck_status + 4 * seg, c->status, sizeof(int) * 2);
     cl_flush(c, L);
     refresh_marks(c);
     const long long base = (long long)seg * K;
@@ -1812,10 +1831,12 @@ int bp_backward(bp_ctx *c, int probe_id, const float *dl_dprobe, int sid, double
     }
     // the reductions below read the adjoint stream's results
     cudaStreamWaitEvent(st, ad.rev_done[0], 0);
-    int ast = 0;
+    int ast = 0, gave_up = 0;
     cudaError_t e = cudaMemcpyAsync(&ast, ad.status, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&gave_up, c->status + 2, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(c, e, "backward");
+    if (gave_up) return fail(c, BP_ERR_TIMEOUT, "bp_backward: device wait timed out");
     if (ast & ST_DOMAIN)
       return fail(c, BP_ERR_DOMAIN, "bp_backward: a bound electron a cell or more from its nucleus (not followed by the reverse pass)");
   }

@@ -12,7 +12,9 @@
 #define BP_MAX_PROBE 32
 
 // bits of the device status word (status[0]); status[1] holds a bit for each
-// loaded species that ST_NEED_SORT is about (none: all of them)
+// loaded species that ST_NEED_SORT is about (none: all of them); status[2] is
+// set with ST_TIMEOUT and stays when the other two are rewritten (a load, an
+// adjoint checkpoint): while it is set no sort and no push runs
 enum { ST_NEED_SORT = 1, ST_DOMAIN = 2, ST_NONFINITE = 4, ST_TIMEOUT = 8 };
 
 // Grid geometry as the kernels see it.  Axes >= D have n = 1, L = 1, box 1.
@@ -179,6 +181,13 @@ struct LaserP {
 
 // ---------------------------------------------------------------------------
 // small device helpers
+
+// a bounded wait gave up
+__device__ __forceinline__ void set_timeout(int *status) {
+  atomicOr(status + 2, 1);
+  atomicOr(status, ST_TIMEOUT);
+}
+__device__ __forceinline__ bool timed_out(const int *status) { return *(volatile const int *)(status + 2) != 0; }
 
 __host__ __device__ __forceinline__ int wrap_mod(int i, int n) {
   int m = i % n;
@@ -604,12 +613,15 @@ void launch_clock_set(long long *clk, const ClockState &v, cudaStream_t s);
 struct SortBufs {
   int *hist;       // [ncell + 1]
   int *bsum;       // [blocks] the sort blocks' totals
-  unsigned *bar;   // [2] their barrier
+  unsigned *bar;   // [2] their barrier: arrivals, barriers passed
+  int polls;       // how often a block polls a barrier before it gives up (ST_TIMEOUT)
   int blocks;      // blocks of the sort's cooperative launch resident at once
   int *tmp_cell;
   float *tmp_f;    // enough floats for the largest species' float payload
   int *tmp_i;      // pidx / id payload
 };
+// some ten seconds, longer than any kernel another stream may hold the GPU with
+constexpr int kSortPolls = 1 << 26;
 // the sort of every species, if the status word asks for it; blocks resident at once
 cudaError_t launch_sort(const GridP &g, int nsp, const SpecP *sp, const PartP *p, const SortBufs &b, int *status,
                         cudaStream_t s);

@@ -1366,6 +1366,7 @@ __global__ void __launch_bounds__(128, 8) k_push_quiet(const __grid_constant__ G
   if (tid == 0) nquiet = 0;
   bool marked = false, occupied = false;
   int ions = 0;
+  const bool stop = timed_out(A.status);
   if (warp < qt && t < g.ntiles) {
     marked = near_mark<D>(g, t, lane);
     // a tile without particles has nothing to push or deposit, whatever its
@@ -1375,6 +1376,9 @@ __global__ void __launch_bounds__(128, 8) k_push_quiet(const __grid_constant__ G
   marked = __any_sync(0xFFFFFFFFu, marked);
   ions = __reduce_add_sync(0xFFFFFFFFu, ions);
   occupied = ions > 0;
+  // a sort gave up: the tiles' particle ranges may not fit together, and the
+  // push's lists stay empty
+  if (stop) return;
   __syncthreads();  // nquiet cleared
   if (warp < qt && t < g.ntiles && lane == 0) {
     if (!occupied) {
@@ -1601,7 +1605,7 @@ __device__ __forceinline__ void stage_done(const GridP &g, const PushArgs &A, co
   const int T0[3] = {tc[0] * Geo<D>::L0, tc[1] * Geo<D>::L1, tc[2] * Geo<D>::L2};
   if (tma_tile<D>(g, T, T0)) {
     if (!mbar_wait(bar, phase)) {
-      if (threadIdx.x == 0) atomicOr(A.status, ST_TIMEOUT);
+      if (threadIdx.x == 0) set_timeout(A.status);
       failed = !mbar_wait(bar, phase);  // one more bounded wait for the loads in flight
     }
     phase ^= 1u;
@@ -1776,6 +1780,9 @@ __global__ void __launch_bounds__(push_threads(D), PB) k_push(GridP g, PushArgs 
   __shared__ int next;
   __shared__ __align__(8) unsigned long long bar;  // completion of the TMA staging
   __shared__ int give_up, marked;
+  // (no push after a sort that gave up, as in k_push_quiet; read here, beside
+  // the tile's marks)
+  const int stop = direct && threadIdx.x == 0 ? *(volatile const int *)(A.status + 2) : 0;
   if (threadIdx.x == 0) {
     mbar_init(&bar);
     give_up = 0;
@@ -1796,7 +1803,7 @@ __global__ void __launch_bounds__(push_threads(D), PB) k_push(GridP g, PushArgs 
       mark = __any_sync(0xFFFFFFFFu, near_mark<D>(g, (int)blockIdx.x, (int)threadIdx.x));
     if (threadIdx.x == 0) {
       if (direct) {
-        next = first ? (int)blockIdx.x : -1;
+        next = first && !stop ? (int)blockIdx.x : -1;
         marked = mark;
       } else {
         const int k = atomicAdd(A.tile_ctr, 1);

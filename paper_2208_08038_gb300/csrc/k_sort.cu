@@ -55,10 +55,12 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *sh, int &total) 
 }
 
 // A barrier over the blocks of a cooperative launch (all resident at once).
-// bar[0]: arrivals, bar[1]: barriers passed.  The wait is bounded (some ten
-// seconds of polls, longer than any kernel another stream may hold the GPU
-// with): false, with ST_TIMEOUT set, when it gives up.
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, int *status) {
+// The wait is bounded (SortBufs::polls): false, with ST_TIMEOUT set, when it
+// gives up.  The barrier, the histogram and the particle arrays are then
+// left as they are, so every later sort and push stays away (status[2]) until
+// the host has cleared the first two and the particles are loaded anew.
+__device__ __forceinline__ bool grid_barrier(const SortBufs &b, int *status) {
+  unsigned *const bar = b.bar;
   __shared__ int passed;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -71,15 +73,15 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, int *status) {
       __threadfence();
       atomicAdd(bar + 1, 1u);
     } else {
-      int it = 0;
-      while (*gen == g0 && it < (1 << 26)) {
+      passed = 0;
+      for (int it = 0; it < b.polls; ++it) {
+        if (*gen != g0) {
+          passed = 1;
+          break;
+        }
         __nanosleep(64);
-        ++it;
       }
-      if (*gen == g0) {
-        passed = 0;
-        atomicOr(status, ST_TIMEOUT);
-      }
+      if (!passed) set_timeout(status);
     }
     __threadfence();
   }
@@ -104,8 +106,9 @@ struct SortArgs {
 };
 __global__ void __launch_bounds__(SORT_BS, 3) k_sort(const __grid_constant__ GridP g, const __grid_constant__ SortArgs S) {
   // every block has read the flag when the last barrier lets one clear it
-  if (!(*(volatile const int *)S.status & ST_NEED_SORT)) return;
-  const int which = *(volatile const int *)(S.status + 1);  // bit s: species s; 0: all
+  const int4 st = __ldcv(reinterpret_cast<const int4 *>(S.status));
+  if (!(st.x & ST_NEED_SORT) || st.z) return;
+  const int which = st.y;  // bit s: species s; 0: all
   __shared__ int sh[32];
   const long long nh = g.ncell + 1;
   const long long tid = blockIdx.x * (long long)SORT_BS + threadIdx.x, nth = (long long)gridDim.x * SORT_BS;
@@ -122,12 +125,12 @@ __global__ void __launch_bounds__(SORT_BS, 3) k_sort(const __grid_constant__ Gri
       const int c = p.cell[q];
       if (c >= 0) atomicAdd(hist + sort_key(g, c), 1);
     }
-    if (!grid_barrier(S.b.bar, S.status)) return;
+    if (!grid_barrier(S.b, S.status)) return;
     int sum = 0, total;
     for (long long q = h0 + threadIdx.x; q < h1; q += SORT_BS) sum += hist[q];
     block_exclusive_scan(sum, sh, total);
     if (threadIdx.x == 0) bsum[blockIdx.x] = total;
-    if (!grid_barrier(S.b.bar, S.status)) return;
+    if (!grid_barrier(S.b, S.status)) return;
     int carry = 0;
     sum = 0;
     for (int q = threadIdx.x; q < (int)blockIdx.x; q += SORT_BS) sum += bsum[q];
@@ -143,11 +146,15 @@ __global__ void __launch_bounds__(SORT_BS, 3) k_sort(const __grid_constant__ Gri
       }
       carry += total;
     }
-    if (!grid_barrier(S.b.bar, S.status)) return;
+    if (!grid_barrier(S.b, S.status)) return;
     for (long long q = tid; q < n; q += nth) {
       const int c = p.cell[q];
       if (c < 0) continue;
       const int dst = atomicAdd(hist + sort_key(g, c), 1);
+      if (dst < 0 || dst >= cap) {  // only if the histogram was not clear
+        atomicOr(S.status, ST_DOMAIN);
+        continue;
+      }
       float *tf = S.b.tmp_f + dst;
       S.b.tmp_cell[dst] = c;
       for (int a = 0; a < g.D; ++a, tf += cap) *tf = p.off[a * cap + q];
@@ -159,7 +166,7 @@ __global__ void __launch_bounds__(SORT_BS, 3) k_sort(const __grid_constant__ Gri
       S.b.tmp_i[dst] = p.id[q];
       if (p.pidx) S.b.tmp_i[cap + dst] = p.pidx[q];
     }
-    if (!grid_barrier(S.b.bar, S.status)) return;
+    if (!grid_barrier(S.b, S.status)) return;
     const int m = p.tstart[g.ntiles];
     for (long long q = tid; q < nh; q += nth) hist[q] = 0;
     for (long long q = tid; q < m; q += nth) {
@@ -174,7 +181,7 @@ __global__ void __launch_bounds__(SORT_BS, 3) k_sort(const __grid_constant__ Gri
       p.id[q] = S.b.tmp_i[q];
       if (p.pidx) p.pidx[q] = S.b.tmp_i[cap + q];
     }
-    if (!grid_barrier(S.b.bar, S.status)) return;
+    if (!grid_barrier(S.b, S.status)) return;
   }
   if (tid == 0) {
     S.status[1] = 0;

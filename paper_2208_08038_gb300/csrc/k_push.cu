@@ -516,24 +516,6 @@ __device__ __noinline__ void deposit_general_pair(JT *__restrict__ J, const int 
   }
 }
 
-// 3D: one row of one body, (component c, nodes j and k along the other two
-// axes), the faces along c
-template <bool DET, typename JT>
-__device__ __forceinline__ void general_row3(JT *__restrict__ J, const int d[3], const PairAxis G[3], int c, int j, int k) {
-  const PairAxis &X = G[0], &Y = G[1], &Z = G[2];
-  // p < q: the other two axes
-  const float sp = c == 0 ? sel4(j, Y.S) : sel4(j, X.S), dp = c == 0 ? sel4(j, Y.DS) : sel4(j, X.DS);
-  const float sq = c == 2 ? sel4(k, Y.S) : sel4(k, Z.S), dq = c == 2 ? sel4(k, Y.DS) : sel4(k, Z.DS);
-  const float F = pair_factor(sp, dp, sq, dq);
-  const int sc = c == 0 ? 1 : (c == 1 ? Box<3>::J0 : Box<3>::JP);
-  JT *p = J + c * Box<3>::JCELLS +
-          Box<3>::ji(d[0] + Box<3>::OJ + X.base, d[1] + Box<3>::OJ + Y.base, d[2] + Box<3>::OJ + Z.base) +
-          j * (c == 0 ? Box<3>::J0 : 1) + k * (c == 2 ? Box<3>::J0 : Box<3>::JP);
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    jput<3, DET>(p + i * sc, (c == 0 ? X.P[i] : (c == 1 ? Y.P[i] : Z.P[i])) * F);
-}
-
 // one particle's deposit inputs, handed to its warp in shared memory (by value
 // they cost the push its registers: 3D, 32.5 M ions, 3.75 ms a step by value,
 // 3.60 this way)
@@ -544,42 +526,15 @@ struct PairJob {
   int two;
 };
 
-// 3D, in a warp that is not whole: its lanes (mask act) share out the rows of
-// the particle, every second lane those of the second body
-template <bool DET, typename JT>
-__device__ __forceinline__ void deposit_general3_lanes(JT *__restrict__ J, unsigned act, const PairJob &P) {
-  const int lane = threadIdx.x & 31, rank = __popc(act & ((1u << lane) - 1u)), n = __popc(act);
-  // one lane alone takes one body after the other
-  const int nb = P.two ? 2 : 1, split = n > 1 ? nb : 1;
-#pragma unroll 1
-  for (int b = rank % split; b < nb; b += split) {
-    PairAxis G[3];
-    int d[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      d[a] = P.d[b][a];
-      G[a] = pair_axis(P.f[b][a], P.e[b][a], P.q[b][a]);
-    }
-    const int of = split == 1 ? n : (n + 1 - b) >> 1;  // lanes of this body
-#pragma unroll 1
-    for (int it = rank / split; it < 48; it += of) general_row3<DET, JT>(J, d, G, it >> 4, it & 3, (it >> 2) & 3);
-  }
-}
-
-// 3D, the usual case of one such particle in a warp: the whole warp shares it
-// out, first a node of a body's axis per lane (24 of them), then the rows of
+// 3D: the whole warp shares out one such particle, first a node of a body's axis per lane (24 of them), then the rows of
 // both bodies, three a lane.  A thermal medium has one such particle in some 15
 // warps; alone, its lane's chain of some 3,000 dependent instructions held the
 // warp as long as several runs of particles, and the tile with it when it came
 // in one of the last runs.
 template <bool DET, typename JT>
-__device__ __noinline__ void deposit_general3_warp(JT *__restrict__ J, unsigned act, const PairJob *job) {
+__device__ __noinline__ void deposit_general3_warp(JT *__restrict__ J, const PairJob *job) {
   constexpr unsigned ALL = 0xFFFFFFFFu;
   const PairJob &P = *job;
-  if (act != ALL) {
-    deposit_general3_lanes<DET, JT>(J, act, P);
-    return;
-  }
   const int lane = threadIdx.x & 31;
   // lanes 12 b + 4 a + m: node m of axis a of body b (the last eight lanes repeat)
   const int nl = lane < 24 ? lane : lane - 24, nbody = nl / 12, naxis = (nl % 12) >> 2;
@@ -996,163 +951,173 @@ __device__ __forceinline__ bool push_far(const GridP &g, const SpecP &sp, const 
   return true;
 }
 
+// One particle's step.  In 3D every lane of the warp calls it, those without a
+// particle with have = false: the general-case deposits are the whole warp's.
 // JT fx64: fields and current are the global arrays (A.E, A.B at `at`; Jsm the
 // current at the box's origin, strides st)
 template <int D, bool DET, bool FREE, typename JT, typename ST = BoxStride<D>>
-__device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, long long i, const int T0[3],
+__device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, bool have, long long i, const int T0[3],
                               const float *Gsm, JT *Jsm, int *status, float scale, unsigned &blo, unsigned &bhi,
                               PairJob *jobs, bool nofield, int4 *far, int *far_n, int far_cap, int s, int t,
                               const PushArgs *A = nullptr, long long at = 0, const ST &st = ST()) {
   constexpr bool GLOBAL = std::is_same<JT, fx64>::value;
   const long long cap = P.cap;
   const bool two = sp.kind == BP_TWO_BODY;
-  int cell = P.cell[i];
-  if (cell < 0) return;
-  int c[3];
-  unpack_cell(g, cell, c);
+  int c[3], d[3] = {0, 0, 0}, d2[3] = {0, 0, 0}, nn[3] = {2, 2, 2};
   float f[3] = {0.0f, 0.0f, 0.0f}, r[3] = {0.0f, 0.0f, 0.0f}, u1[3], u2[3] = {0.0f, 0.0f, 0.0f};
+  float f2[3] = {0.0f, 0.0f, 0.0f}, v1[3], v2[3] = {0.0f, 0.0f, 0.0f};
+  float fn[3] = {0.0f, 0.0f, 0.0f}, de1[3] = {0.0f, 0.0f, 0.0f}, de2[3] = {0.0f, 0.0f, 0.0f}, rn[3];
+  float xi[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
+  float dxdt[3] = {g.dxdt[0], g.dxdt[1], g.dxdt[2]};  // (in 1D and 2D read further down: registers)
+  bool bad = false, fast = true, silent = true;
+  // kicks and moves; not live: no particle, or one that is left where it is
+  bool live = false;
+  do {
+    if (D == 3 && !have) break;
+    const int cell = P.cell[i];
+    if (cell < 0) break;
+    unpack_cell(g, cell, c);
 #pragma unroll
-  for (int a = 0; a < D; ++a) f[a] = P.off[a * cap + i];
+    for (int a = 0; a < D; ++a) f[a] = P.off[a * cap + i];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) u1[a] = P.u1[a * cap + i];
-  if (two) {
+    for (int a = 0; a < 3; ++a) u1[a] = P.u1[a * cap + i];
+    if (two) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      r[a] = P.r[a * cap + i];
-      u2[a] = P.u2[a * cap + i];
-    }
-  }
-  int d[3] = {0, 0, 0}, d2[3] = {0, 0, 0};
-  float f2[3] = {0.0f, 0.0f, 0.0f};
-  bool bad = false;
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    d[a] = rel_cell<D>(g, a, c[a], T0[a]);
-    bad |= outside_margin<D>(a, d[a]);
-    // body 2 sits at x1 - r
-    float rc = r[a] * g.idx[a];
-    bad |= !(fabsf(rc) < 1.0f);
-    float X = f[a] - rc;
-    float fl = floorf(X);
-    float fr = X - fl;
-    int di = (int)fl;
-    if (fr >= 1.0f) { fr = 0.0f; di += 1; }
-    d2[a] = d[a] + di;
-    f2[a] = fr;
-  }
-  if (bad) {
-    // sorted mode: perhaps a bound electron a cell or more from its nucleus,
-    // which k_push_far moves on the global grid after this kernel (it
-    // reports a domain error for anything else); atomic mode: a domain error
-    if (DET && two) {
-      const int k = atomicAdd(far_n, 1);
-      if (k < far_cap) {
-        far[k] = make_int4(s, (int)i, t, 0);
-        return;
+      for (int a = 0; a < 3; ++a) {
+        r[a] = P.r[a * cap + i];
+        u2[a] = P.u2[a * cap + i];
       }
     }
-    atomicOr(status, ST_DOMAIN);
-    return;
-  }
-  // A tile whose staged box holds no field (ahead of the field front) gathers
-  // exact zeros, so the gather is skipped.  A neutral ion there with r = 0 and
-  // u1 = u2 also keeps its momenta exactly (no internal force at r = 0, Boris
-  // rotation by zero fields), so its kicks are skipped too.
-  bool quiet = nofield && two && sp.qw1 == -sp.qw2;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) quiet &= (r[a] == 0.0f) && (u1[a] == u2[a]);
-  float E1[3], B1[3], E2[3], B2[3];
-  if (nofield) {
+    for (int a = 0; a < D; ++a) {
+      d[a] = rel_cell<D>(g, a, c[a], T0[a]);
+      bad |= outside_margin<D>(a, d[a]);
+      // body 2 sits at x1 - r
+      float rc = r[a] * g.idx[a];
+      bad |= !(fabsf(rc) < 1.0f);
+      float X = f[a] - rc;
+      float fl = floorf(X);
+      float fr = X - fl;
+      int di = (int)fl;
+      if (fr >= 1.0f) { fr = 0.0f; di += 1; }
+      d2[a] = d[a] + di;
+      f2[a] = fr;
+    }
+    if (bad) {
+      // sorted mode: perhaps a bound electron a cell or more from its nucleus,
+      // which k_push_far moves on the global grid after this kernel (it
+      // reports a domain error for anything else); atomic mode: a domain error
+      if (DET && two) {
+        const int k = atomicAdd(far_n, 1);
+        if (k < far_cap) {
+          far[k] = make_int4(s, (int)i, t, 0);
+          break;
+        }
+      }
+      atomicOr(status, ST_DOMAIN);
+      break;
+    }
+    // A tile whose staged box holds no field (ahead of the field front) gathers
+    // exact zeros, so the gather is skipped.  A neutral ion there with r = 0 and
+    // u1 = u2 also keeps its momenta exactly (no internal force at r = 0, Boris
+    // rotation by zero fields), so its kicks are skipped too.
+    bool quiet = nofield && two && sp.qw1 == -sp.qw2;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) E1[a] = B1[a] = E2[a] = B2[a] = 0.0f;
-  } else {
-    if constexpr (D == 3) {
-      Pos P1, P2;
-      make_pos<D>(d, f, P1);
-      make_pos<D>(two ? d2 : d, two ? f2 : f, P2);
-      gather_all_p3(Gsm, P1, P2, E1, B1, E2, B2);
+    for (int a = 0; a < 3; ++a) quiet &= (r[a] == 0.0f) && (u1[a] == u2[a]);
+    float E1[3], B1[3], E2[3], B2[3];
+    if (nofield) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) E1[a] = B1[a] = E2[a] = B2[a] = 0.0f;
     } else {
-      Loc L1, L2;
-      make_loc<D>(d, f, L1);
-      make_loc<D>(two ? d2 : d, two ? f2 : f, L2);
-      if constexpr (GLOBAL) gather_all_few(A->E, A->B, at, st.row, L1, L2, E1, B1, E2, B2);
-      else gather_all<D>(Gsm, L1, L2, E1, B1, E2, B2);
+      if constexpr (D == 3) {
+        Pos P1, P2;
+        make_pos<D>(d, f, P1);
+        make_pos<D>(two ? d2 : d, two ? f2 : f, P2);
+        gather_all_p3(Gsm, P1, P2, E1, B1, E2, B2);
+      } else {
+        Loc L1, L2;
+        make_loc<D>(d, f, L1);
+        make_loc<D>(two ? d2 : d, two ? f2 : f, L2);
+        if constexpr (GLOBAL) gather_all_few(A->E, A->B, at, st.row, L1, L2, E1, B1, E2, B2);
+        else gather_all<D>(Gsm, L1, L2, E1, B1, E2, B2);
+      }
     }
-  }
-  float v1[3], v2[3] = {0.0f, 0.0f, 0.0f};
-  if (two && !quiet) {
-    // modified Coulomb field (Sec. 2): on the nucleus q2 kappa r / (r^2 + ac^2)^{3/2},
-    // on the bound electron -q1 kappa r / (...), r = x1 - x2
-    const int pi = P.pidx ? P.pidx[i] : 0;
-    const float ac = sp.ac[pi];
-    float rr = r[0] * r[0] + r[1] * r[1] + r[2] * r[2] + ac * ac;
-    float rs = rsqrtf(rr);
-    float s = sp.kappa * rs * rs * rs;
+    if (two && !quiet) {
+      // modified Coulomb field (Sec. 2): on the nucleus q2 kappa r / (r^2 + ac^2)^{3/2},
+      // on the bound electron -q1 kappa r / (...), r = x1 - x2
+      const int pi = P.pidx ? P.pidx[i] : 0;
+      const float ac = sp.ac[pi];
+      float rr = r[0] * r[0] + r[1] * r[1] + r[2] * r[2] + ac * ac;
+      float rs = rsqrtf(rr);
+      float s = sp.kappa * rs * rs * rs;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      E1[a] = fmaf(sp.q2 * s, r[a], E1[a]);
-      E2[a] = fmaf(-sp.q1 * s, r[a], E2[a]);
+      for (int a = 0; a < 3; ++a) {
+        E1[a] = fmaf(sp.q2 * s, r[a], E1[a]);
+        E2[a] = fmaf(-sp.q1 * s, r[a], E2[a]);
+      }
+      boris(sp.h2, E2, B2, u2);
     }
-    boris(sp.h2, E2, B2, u2);
-  }
-  if (two) {
-    const float g2 = inv_gamma(u2);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) v2[a] = u2[a] * g2;
-  }
-  if (!quiet) boris(sp.h1, E1, B1, u1);
-  {
-    const float g1 = inv_gamma(u1);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) v1[a] = u1[a] * g1;
-  }
-  // drift: body 1 moves in cells by dt v / dx; the internal displacement by
-  // dt (v1 - v2) on all three axes; the deposited moves are the ones the
-  // stored FP32 state actually makes
-  float fn[3] = {0.0f, 0.0f, 0.0f}, de1[3] = {0.0f, 0.0f, 0.0f}, de2[3] = {0.0f, 0.0f, 0.0f}, rn[3];
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    fn[a] = drift_offset(g, a, f[a], v1[a]);
-    de1[a] = fn[a] - f[a];
-  }
-  if (two) {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      rn[a] = r[a] + g.dt * (v1[a] - v2[a]);
-      float dr = rn[a] - r[a];
-      if (a < D) de2[a] = de1[a] - dr * g.idx[a];
-    }
-  }
-  const float dxdt[3] = {g.dxdt[0], g.dxdt[1], g.dxdt[2]};
-  // fast path when every position keeps one nearest node per axis
-  bool fast = true;
-  float xi[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
-  int nn[3] = {2, 2, 2};
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    const float u1p = f[a] >= 0.5f ? 1.0f : 0.0f;
-    xi[0][a] = f[a] - u1p;
-    const float x1n = xi[0][a] + de1[a];
-    fast &= (x1n >= -0.5f) && (x1n < 0.5f);
-    nn[a] = d[a] + Box<D>::OJ + (int)u1p;
     if (two) {
-      const float u2p = f2[a] >= 0.5f ? 1.0f : 0.0f;
-      xi[1][a] = f2[a] - u2p;
-      const float x2n = xi[1][a] + de2[a];
-      fast &= (d2[a] == d[a]) && (u2p == u1p) && (x2n >= -0.5f) && (x2n < 0.5f);
-    }
-  }
-  // a neutral ion whose bodies coincide and move together carries no
-  // current (its two bodies' terms cancel exactly; Sec. 2 starts every ion
-  // so, and it stays so until a field acts on it): nothing to deposit
-  bool silent = two && sp.qw1 == -sp.qw2;
+      const float g2 = inv_gamma(u2);
 #pragma unroll
-  for (int a = 0; a < 3; ++a) silent &= (r[a] == 0.0f) && (v1[a] == v2[a]);
+      for (int a = 0; a < 3; ++a) v2[a] = u2[a] * g2;
+    }
+    if (!quiet) boris(sp.h1, E1, B1, u1);
+    {
+      const float g1 = inv_gamma(u1);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) v1[a] = u1[a] * g1;
+    }
+    // drift: body 1 moves in cells by dt v / dx; the internal displacement by
+    // dt (v1 - v2) on all three axes; the deposited moves are the ones the
+    // stored FP32 state actually makes
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      fn[a] = drift_offset(g, a, f[a], v1[a]);
+      de1[a] = fn[a] - f[a];
+    }
+    if (two) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        rn[a] = r[a] + g.dt * (v1[a] - v2[a]);
+        float dr = rn[a] - r[a];
+        if (a < D) de2[a] = de1[a] - dr * g.idx[a];
+      }
+    }
+    if constexpr (D < 3) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) dxdt[a] = g.dxdt[a];
+    }
+    // fast path when every position keeps one nearest node per axis
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      const float u1p = f[a] >= 0.5f ? 1.0f : 0.0f;
+      xi[0][a] = f[a] - u1p;
+      const float x1n = xi[0][a] + de1[a];
+      fast &= (x1n >= -0.5f) && (x1n < 0.5f);
+      nn[a] = d[a] + Box<D>::OJ + (int)u1p;
+      if (two) {
+        const float u2p = f2[a] >= 0.5f ? 1.0f : 0.0f;
+        xi[1][a] = f2[a] - u2p;
+        const float x2n = xi[1][a] + de2[a];
+        fast &= (d2[a] == d[a]) && (u2p == u1p) && (x2n >= -0.5f) && (x2n < 0.5f);
+      }
+    }
+    // a neutral ion whose bodies coincide and move together carries no
+    // current (its two bodies' terms cancel exactly; Sec. 2 starts every ion
+    // so, and it stays so until a field acts on it): nothing to deposit
+    silent = two && sp.qw1 == -sp.qw2;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) silent &= (r[a] == 0.0f) && (v1[a] == v2[a]);
+    live = true;
+  } while (false);
   if constexpr (D == 3) {
-    // the general case in 3D: rare in a thermal medium, so the warp's lanes
-    // share out one such particle after the other
-    const unsigned act = __activemask();
-    unsigned gen = __ballot_sync(act, !silent && !fast);
+    // the general case in 3D: rare in a thermal medium, so the whole warp
+    // shares out one such particle after the other.  Its lanes meet here
+    // whatever became of their own particles: the slot is the warp's, and two
+    // groups of it that arrived apart, each with its own active mask, would
+    // share it.  (32.5 M ions: 3.69 ms a step, 3.63 with such masks.)
+    unsigned gen = __ballot_sync(0xFFFFFFFFu, live && !silent && !fast);
     for (; gen; gen &= gen - 1) {
       PairJob &P = jobs[threadIdx.x >> 5];
       if ((int)(threadIdx.x & 31) == __ffs(gen) - 1) {
@@ -1170,11 +1135,12 @@ __device__ void push_particle(const GridP &g, const SpecP &sp, const PartP &P, l
         }
         P.two = two;
       }
-      __syncwarp(act);
-      deposit_general3_warp<DET, JT>(Jsm, act, &P);
-      __syncwarp(act);
+      __syncwarp();
+      deposit_general3_warp<DET, JT>(Jsm, &P);
+      __syncwarp();
     }
   }
+  if (!live) return;
   if (!silent) {
     if (fast) {
       float qw[2] = {sp.qw1, sp.qw2};
@@ -1685,10 +1651,19 @@ __device__ __forceinline__ void push_tile(const GridP &g, const PushArgs &A, con
       rn = __shfl_sync(0xFFFFFFFFu, rn, 0);
       const int k = at(r);
       const long long i = beg + k;
-      if (k < n && !(moved && quiet_done(A.p[s], i))) {
+      const bool have = k < n && !(moved && quiet_done(A.p[s], i));
+      if constexpr (D == 3) {
+        if (have) {
+          const int kn = at(rn);
+          if (kn < n) prefetch_particle<D>(A.p[s], beg + kn, two);
+          ++pushed;
+        }
+        push_particle<D, DET, FREE, JT>(g, A.sp[s], A.p[s], have, i, T0, Gsm, Jsm, A.status, A.jscale, blo, bhi, jobs,
+                                        nofield, A.far, A.far_n, A.far_cap, s, t);
+      } else if (have) {
         const int kn = at(rn);
         if (kn < n) prefetch_particle<D>(A.p[s], beg + kn, two);
-        push_particle<D, DET, FREE, JT>(g, A.sp[s], A.p[s], i, T0, Gsm, Jsm, A.status, A.jscale, blo, bhi, jobs,
+        push_particle<D, DET, FREE, JT>(g, A.sp[s], A.p[s], true, i, T0, Gsm, Jsm, A.status, A.jscale, blo, bhi, jobs,
                                         nofield, A.far, A.far_n, A.far_cap, s, t);
         ++pushed;
       }
@@ -1848,7 +1823,7 @@ __global__ void __launch_bounds__(128, 4) k_push_few(GridP g, PushArgs A) {
       const int end = A.p[s].tstart[t + 1];
       for (int i = A.p[s].tstart[t] + lane; i < end; i += 32) {
         unsigned blo = 0xFFFFFFFFu, bhi = 0u;
-        push_particle<2, true, false, fx64, GridStride>(g, A.sp[s], A.p[s], i, T0, nullptr, J, A.status, A.jscale, blo, bhi,
+        push_particle<2, true, false, fx64, GridStride>(g, A.sp[s], A.p[s], true, i, T0, nullptr, J, A.status, A.jscale, blo, bhi,
                                                         nullptr, false, A.far, A.far_n, A.far_cap, s, t, &A, at, st);
         ++pushed;
       }

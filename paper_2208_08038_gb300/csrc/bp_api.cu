@@ -80,11 +80,6 @@ int check_launch(bp_ctx *c, const char *what) {
   return BP_OK;
 }
 
-// fixed-point scale of the sorted deposit: a power of two such that one
-// particle's largest contribution (|q w| max(1, dx/dt)) maps to about 2^36.
-// A node of a tile box then holds the exact sum of up to 2^26 such maximal
-// contributions, and a quantum is about 1e-11 of the largest one (below the
-// FP32 rounding of the contributions themselves).
 // every tile updated, and its current cleared and formed, until the next push
 // recomputes the flags
 void reset_active(bp_ctx *c) {
@@ -101,6 +96,12 @@ void refresh_marks(bp_ctx *c) {
   reset_active(c);
 }
 
+// fixed-point scale of the sorted deposit: a power of two such that one
+// particle's largest contribution (|q w| max(1, dx/dt)) maps to about 2^36.
+// The global current then holds the exact sum of up to 2^26 such maximal
+// contributions per node (a tile's box, 2^11 of them, is emptied into it in
+// time: kLaneLoad, k_push.cu), and a quantum is about 1e-11 of the largest one
+// (below the FP32 rounding of the contributions themselves).
 void update_jscale(bp_ctx *c) {
   if (!c->det) {
     c->jscale = c->jinv = 0.0f;

@@ -356,7 +356,9 @@ __device__ __forceinline__ long long f2ll_rn(float x) {
 // |r| <= 2^15, both exact in FP32, so rne(v) = 2^16 h + rne(r); lo takes
 // rne(r), hi takes h (and is skipped when h = 0).  The node's value,
 // 2^16 sum(h) + sum(rne(r)), is the exact sum of rne(v) whatever the order,
-// while fewer than 2^16 adds reach one node.  Both roundings to an integer
+// while fewer than 2^16 adds reach one node and its |h| add up to less than
+// 2^31 (2^11 adds of 2^36); the callers flush the box before that (the push:
+// kLaneLoad, the adjoint's scatter: 64 chunks of adds below 2^31).  Both roundings to an integer
 // add 1.5 * 2^23 (whose ulp is 1) and read the integer off the bits, on the
 // FMA pipe; that needs |v| < 2^38 (callers scale contributions to <= 2^37).
 __device__ __forceinline__ void fx_add(unsigned int *lo, int hoff, float v) {

@@ -399,14 +399,18 @@ __device__ __forceinline__ float dqshape(float x) {
   return 0.0f;
 }
 
-// x / b for a normal b with its correctly rounded reciprocal r: a quotient
-// estimate and one correction by its exact remainder, correctly rounded
+// x / b for b >= 1 (or infinite) with its correctly rounded reciprocal r: a
+// quotient estimate and one correction by its exact remainder, correctly rounded
 // (Markstein, "Computation of elementary functions on the IBM RISC System/6000
-// processor", IBM J. Res. Dev. 34, 1990, theorem 8) while x r and the remainder
-// do not underflow
+// processor", IBM J. Res. Dev. 34, 1990, theorem 8) while the remainder does
+// not underflow (x = 0 or |x| >= 2^-100, b <= 2^60); below, and for larger b,
+// within one unit in the last place.  Where x or b is not finite the remainder
+// is NaN, and a finite one in its place leaves the estimate, the quotient, as
+// it is.
 __device__ __forceinline__ float quot(float x, float b, float r) {
   const float q = __fmul_rn(x, r);
-  return fmaf(fmaf(-b, q, x), r, q);
+  const float rem = fmaxf(fmaf(-b, q, x), -3.402823466e38f);  // (the finite one of the two)
+  return fmaf(rem, r, q);
 }
 
 // reverse of boris(): given the adjoint of the pushed momentum, the adjoints
@@ -418,7 +422,8 @@ __device__ __forceinline__ void boris_adj(float h, const float E[3], const float
   for (int a = 0; a < 3; ++a) um[a] = u0[a] + h * E[a];
   float gm = sqrtf(1.0f + um[0] * um[0] + um[1] * um[1] + um[2] * um[2]);
   // One division each for gamma, gamma^2 and 1 + t^2, the quotients from their
-  // reciprocals (quot: the same bits).  A zero field component sent each of the
+  // reciprocals (quot: the divisions' bits, but the last one where a dividend is
+  // below 2^-100).  A zero field component sent each of the
   // 16 divisions of a body down the division's out-of-line path: 35 of them were
   // a quarter of the reversed push's instructions (2D, 524 k ions: 107 us
   // before, 72 with this and one staging per tile).

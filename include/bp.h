@@ -196,7 +196,12 @@ int bp_add_probe(bp_ctx *ctx, int comp, const int64_t *nodes, int64_t npts, int6
  * and of one (captured on first use and again whenever a launch argument has
  * changed: particle arrays, lasers, probes, parameters); so do single steps
  * from the third such call in a row.  Other single steps and timed steps
- * launch the same kernels directly, with the same results bit for bit. */
+ * launch the same kernels directly, with the same results bit for bit.  (In
+ * the sorted mode a rerun of the same calls gives the same bits.  An ion whose
+ * bound electron is a cell or more away is gathered by a warp in a step with
+ * at most 2,432 such ions and by a thread in one with more: the two round the
+ * sum of its stencil differently, so there its last bits depend on the other
+ * ions of the run.) */
 int bp_step(bp_ctx *ctx, int64_t n_steps);
 
 /* Wait for the stream and return the device status word as a bp_status:

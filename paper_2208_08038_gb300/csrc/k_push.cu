@@ -1920,9 +1920,12 @@ __global__ void __launch_bounds__(128) k_push_far(GridP g, PushArgs A) {
       atomicOr(A.status, ST_DOMAIN);
   };
   // few ions (rare tears): a warp each, for the latency; many (a strong field
-  // over a whole crystal): a thread each
+  // over a whole crystal): a thread each.  A fixed number (a GB300's warps of
+  // this launch): the gather sums its nodes by lane, so the last bit of a far
+  // ion's fields depends on the form, and must not depend on the device.
+  constexpr int FEW_FAR = 2432;
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-  if (n <= nt / 32) {
+  if (n <= FEW_FAR) {
     for (int k = tid >> 5; k < n; k += nt / 32) move(k, std::integral_constant<int, D == 3 ? 32 : 16>{});
   } else {
     for (int k = tid; k < n; k += nt) move(k, std::integral_constant<int, 1>{});

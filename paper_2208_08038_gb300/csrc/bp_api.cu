@@ -520,9 +520,9 @@ int bp_set_lattice(bp_ctx *c, int sid, const double *sites, int64_t n_sites, int
   if (!stage) return fail(c, BP_ERR_OOM, "lattice staging");
   double *sx = (double *)stage;
   double *su = sx + (size_t)chunk * D;
-  int *sp_ = (int *)(su + (size_t)chunk * 3);
-  double *dsites = (double *)(stage + rows);
+  double *dsites = su + (size_t)chunk * 3;  // the doubles first: they stay aligned for an odd number of ions
   int *dparam = (int *)(dsites + (size_t)D * ns);
+  int *sp_ = dparam + ns;
   int zero = 0;
   cudaMemcpyAsync(c->status, &zero, sizeof(int), cudaMemcpyHostToDevice, st);
   if (n_sites > 0) cudaMemcpyAsync(dsites, sites, sizeof(double) * D * n_sites, cudaMemcpyHostToDevice, st);

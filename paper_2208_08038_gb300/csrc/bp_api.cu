@@ -478,6 +478,7 @@ int finish_load(bp_ctx *c, Species &s, long long n, void *stage) {
   int sw[3] = {0, 0, 0};
   cudaMemcpy(sw, c->status, sizeof sw, cudaMemcpyDeviceToHost);
   const int stw = sw[0];
+  if (sw[2] || (stw & (ST_NONFINITE | ST_DOMAIN))) launch_load_failed(c->status, st);
   if (sw[2]) return fail(c, BP_ERR_TIMEOUT, "an earlier device wait timed out (bp_reset first)");
   if (stw & ST_NONFINITE) return fail(c, BP_ERR_NONFINITE, "non-finite position or momentum in the load");
   if (stw & ST_DOMAIN) return fail(c, BP_ERR_DOMAIN, "a particle lies outside the grid or has a bad param_idx");
@@ -523,8 +524,8 @@ int bp_set_lattice(bp_ctx *c, int sid, const double *sites, int64_t n_sites, int
   double *dsites = su + (size_t)chunk * 3;  // the doubles first: they stay aligned for an odd number of ions
   int *dparam = (int *)(dsites + (size_t)D * ns);
   int *sp_ = dparam + ns;
-  int zero = 0;
-  cudaMemcpyAsync(c->status, &zero, sizeof(int), cudaMemcpyHostToDevice, st);
+  launch_load_begin(c->status, st);
+  c->launches++;
   if (n_sites > 0) cudaMemcpyAsync(dsites, sites, sizeof(double) * D * n_sites, cudaMemcpyHostToDevice, st);
   if (site_param && n_sites > 0) cudaMemcpyAsync(dparam, site_param, sizeof(int) * n_sites, cudaMemcpyHostToDevice, st);
   for (long long b = 0; b < n; b += chunk) {
@@ -555,14 +556,14 @@ int bp_load_particles(bp_ctx *c, int sid, const double *x, const double *u, cons
   else s.pidx_host.clear();  // all 0
   cudaStream_t st = c->stream;
   const long long chunk = std::min<long long>(std::max<long long>(n, 1), 1LL << 25);
-  int zero = 0;
   // Arrays in page-locked host memory that the device can address (pinned
   // or registered, e.g. torch's pin_memory()): the conversion kernel reads
   // them where they are, over the host link, with no staging copy.
   // Otherwise they are copied to a device staging buffer chunk by chunk.
   const void *dx = mapped_host(x), *du = u ? mapped_host(u) : nullptr, *dp = pidx ? mapped_host(pidx) : nullptr;
   if (dx && (!u || du) && (!pidx || dp)) {
-    cudaMemcpyAsync(c->status, &zero, sizeof(int), cudaMemcpyHostToDevice, st);
+    launch_load_begin(c->status, st);
+    c->launches++;
     for (long long b = 0; b < n; b += chunk) {
       const long long k = std::min(chunk, n - b);
       launch_load_convert(g, s.sp, s.p, static_cast<const double *>(dx) + b * D,
@@ -578,7 +579,8 @@ int bp_load_particles(bp_ctx *c, int sid, const double *x, const double *u, cons
   double *sx = (double *)stage;
   double *su = sx + (size_t)chunk * D;
   int *sp_ = (int *)(su + (size_t)chunk * 3);
-  cudaMemcpyAsync(c->status, &zero, sizeof(int), cudaMemcpyHostToDevice, st);
+  launch_load_begin(c->status, st);
+  c->launches++;
   for (long long b = 0; b < n; b += chunk) {
     long long k = std::min(chunk, n - b);
     cudaMemcpyAsync(sx, x + b * D, sizeof(double) * k * D, cudaMemcpyHostToDevice, st);

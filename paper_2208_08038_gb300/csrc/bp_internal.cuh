@@ -14,7 +14,8 @@
 // bits of the device status word (status[0]); status[1] holds a bit for each
 // loaded species that ST_NEED_SORT is about (none: all of them); status[2] is
 // set with ST_TIMEOUT and stays when the other two are rewritten (a load, an
-// adjoint checkpoint): while it is set no sort and no push runs
+// adjoint checkpoint): while it is set no sort and no push runs; status[3] is
+// set during a load when other species' particles wait for a sort
 enum { ST_NEED_SORT = 1, ST_DOMAIN = 2, ST_NONFINITE = 4, ST_TIMEOUT = 8 };
 
 // Grid geometry as the kernels see it.  Axes >= D have n = 1, L = 1, box 1.
@@ -634,6 +635,8 @@ void launch_gen_lattice(int D, const double *sites, int per_site, double jitter,
 void launch_pick(const PartP &p, int D, int two, long long count, const int *sid, const int *srow, int n,
                  int *cell_out, float *out, unsigned char *found, cudaStream_t s);
 void launch_set_sort_flag(int *status, cudaStream_t s);
+void launch_load_begin(int *status, cudaStream_t s);
+void launch_load_failed(int *status, cudaStream_t s);
 void launch_gen_medium(const GridP &g, const SpecP &sp, PartP &p, const int lo[3], const int hi[3], int ppc,
                        uint64_t seed, double sigma, long long first, long long count, cudaStream_t s);
 void launch_load_convert(const GridP &g, const SpecP &sp, PartP &p, const double *x, const double *u, const int *pidx,

@@ -185,14 +185,27 @@ __global__ void __launch_bounds__(SORT_BS, 3) k_sort(const __grid_constant__ Gri
   }
   if (tid == 0) {
     S.status[1] = 0;
-    atomicAnd(S.status, ~ST_NEED_SORT);
+    if (st.w) S.status[3] = 0;  // a load's sort: the species it did not see are still to be sorted
+    else atomicAnd(S.status, ~ST_NEED_SORT);
   }
 }
 
-// every species of the next launch_sort is to be sorted
+// every species of the next launch_sort, a load's, is to be sorted
 __global__ void k_set_flag(int *status) {
+  if (status[0] & ST_NEED_SORT) status[3] = 1;
   status[1] = 0;
-  atomicOr(status, ST_NEED_SORT);
+  status[0] |= ST_NEED_SORT;
+}
+
+// the status word cleared for a load, and what it held of other species' need
+// set again after a load that failed
+__global__ void k_load_begin(int *status) {
+  if (status[0] & ST_NEED_SORT) status[3] = 1;
+  status[0] = 0;
+}
+__global__ void k_load_failed(int *status) {
+  if (status[3]) status[0] |= ST_NEED_SORT;
+  status[1] = status[3] = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -435,6 +448,8 @@ cudaError_t launch_sort(const GridP &g, int nsp, const SpecP *sp, const PartP *p
 }
 
 void launch_set_sort_flag(int *status, cudaStream_t s) { k_set_flag<<<1, 1, 0, s>>>(status); }
+void launch_load_begin(int *status, cudaStream_t s) { k_load_begin<<<1, 1, 0, s>>>(status); }
+void launch_load_failed(int *status, cudaStream_t s) { k_load_failed<<<1, 1, 0, s>>>(status); }
 
 // particles whose load id is in the sorted list sid[0..n): copy the raw
 // state of particle slot i to row k of out (k = position of its id in the

@@ -100,8 +100,9 @@ void refresh_marks(bp_ctx *c) {
 // particle's largest contribution (|q w| max(1, dx/dt)) maps to about 2^36.
 // The global current then holds the exact sum of up to 2^26 such maximal
 // contributions per node (a tile's box, 2^11 of them, is emptied into it in
-// time: kLaneLoad, k_push.cu), and a quantum is about 1e-11 of the largest one
-// (below the FP32 rounding of the contributions themselves).
+// time: kLaneLoad, k_push.cu; the E update takes sums below 2^55, 2^19 of
+// them: fx_to_float), and a quantum is about 1e-11 of the largest one (below
+// the FP32 rounding of the contributions themselves).
 void update_jscale(bp_ctx *c) {
   if (!c->det) {
     c->jscale = c->jinv = 0.0f;

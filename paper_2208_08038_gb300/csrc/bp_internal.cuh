@@ -359,9 +359,9 @@ __device__ __forceinline__ long long f2ll_rn(float x) {
 // 2^16 sum(h) + sum(rne(r)), is the exact sum of rne(v) whatever the order,
 // while fewer than 2^16 adds reach one node and its |h| add up to less than
 // 2^31 (2^11 adds of 2^36); the callers flush the box before that (the push:
-// kLaneLoad, the adjoint's scatter: 64 chunks of adds below 2^31).  Both roundings to an integer
-// add 1.5 * 2^23 (whose ulp is 1) and read the integer off the bits, on the
-// FMA pipe; that needs |v| < 2^38 (callers scale contributions to <= 2^37).
+// kLaneLoad, the adjoint's scatter: 64 chunks of adds below 2^31).  Both
+// roundings to an integer add 1.5 * 2^23 (whose ulp is 1) and read the integer
+// off the bits, on the FMA pipe; that needs |v| < 2^38 (callers scale contributions to <= 2^37).
 __device__ __forceinline__ void fx_add(unsigned int *lo, int hoff, float v) {
   constexpr float M = 12582912.0f;
   const float hs = fmaf(v, 1.52587890625e-05f, M);  // M + rne(v / 2^16)

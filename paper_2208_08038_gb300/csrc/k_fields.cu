@@ -186,10 +186,10 @@ LaserSet make_laser_set(const LaserP *las, int nlas) {
   return ls;
 }
 
-// v * s for a 64-bit fixed-point value v and a power-of-two scale s, rounded
-// once: v = a 2^24 + b with 0 <= b < 2^24, both exact in FP32 while
-// |v| < 2^48, so the fma rounds the exact product (the 64-bit integer
-// conversion would run on the slow FP64 path)
+// v * s for a 64-bit fixed-point value v, |v| < 2^55, and a power-of-two scale
+// s: v = a 2^24 + b with 0 <= b < 2^24, both exact in FP32 while |v| < 2^48, so
+// the fma rounds the exact product once; above, a is rounded first (the 64-bit
+// integer conversion would run on the slow FP64 path)
 __device__ __forceinline__ float fx_to_float(long long v, float s) {
   const float a = (float)(int)(v >> 24);
   const float b = (float)(int)(v & 0xFFFFFFLL);

@@ -266,8 +266,8 @@ __device__ __forceinline__ float2 sel3(int k, const float2 *a) { return k == 0 ?
 // esirkepov3 for a two-body ion in 3D, sorted mode, on Blackwell's packed
 // FP32 pairs (FFMA2): the two bodies in the lanes of every setup term and of
 // each row's transverse factor F; a node's value is the bodies' two products
-// (one packed multiply) added, and a row's two nodes go through one packed
-// fixed-point split (fx_add2).  The outer loops stay rolled as in the scalar
+// (one packed multiply) added, and six nodes at a time go through the packed
+// fixed-point split (fx_add6).  The outer loops stay rolled as in the scalar
 // form (code size).
 __device__ __forceinline__ void esirkepov3_p3(unsigned int *__restrict__ J, const int n[3], const float (*xi)[3],
                                               const float (*de)[3], const float *qw, const float dxdt[3],
@@ -1610,6 +1610,7 @@ __device__ __forceinline__ void drain_box(const GridP &g, unsigned long long *jf
   using BX = Box<D>;
   const int T0[3] = {(t % g.nt[0]) * Geo<D>::L0, ((t / g.nt[0]) % g.nt[1]) * Geo<D>::L1,
                      (t / (g.nt[0] * g.nt[1])) * Geo<D>::L2};
+  __syncwarp();  // the other lanes' adds are in
 #pragma unroll 1
   for (int q = threadIdx.x & 31; q < 3 * BX::JCOMP; q += 32) {
     const int cc = q / BX::JCOMP, nd = q - cc * BX::JCOMP;

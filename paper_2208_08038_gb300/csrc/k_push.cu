@@ -20,7 +20,7 @@
 //                             associative: the same sums in any order),
 //          BP_DEPOSIT_ATOMIC: FP32 shared atomics,
 //     3. sorted mode: add every non-zero node of the box to the global 64-bit
-//        fixed-point current; atomic mode: write the box to the tile's slot
+//        fixed-point current (and before, when its words may fill); atomic mode: write the box to the tile's slot
 //        for the current-sum kernel,
 //   k_push_far    sorted mode: the ions k_push left on the far list (a bound
 //                 electron a cell or more from its nucleus), pushed with the
